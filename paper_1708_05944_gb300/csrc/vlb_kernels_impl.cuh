@@ -731,47 +731,133 @@ cudaError_t launch_shakhov(real* Fout, const real* Fprev, long long cells, int V
 
 // ---------------------------------------------------------------- caller layout <-> device layout
 // Caller rows hold f' then f'' (V values each); device rows hold the deviation
-// from R as interleaved (f', f'') pairs of Vp velocities.  One CTA per cell row
-// at a time; the row passes through shared memory, so src and dst may be the
-// same buffer when V == Vp.
+// from R as interleaved (f', f'') pairs of Vp velocities.  Bound by HBM (one read and one
+// write of the distribution): one warp per cell row, each lane holding NV neighbouring
+// velocities of every chunk of 32 NV, so that a chunk is two contiguous accesses of the
+// caller's row (f', f'') and one of the device row, and the rest state of the lane's
+// velocities stays in registers over all rows of the warp.  A row is read whole before any of
+// it is written, so src and dst may be the same buffer when V == Vp and the map is the identity.
+//
+// F -/+ R in single precision takes R as a float pair (hi, lo) and TwoSum: the sum is exact to
+// about 2^-48 before its one rounding, where the earlier sum in double cost three operations
+// of the 1/64-rate FP64 pipe per value.  2048 x 512 x 192 channel (1.6 GB), both directions
+// together: 5.5 ms before, 1.27 ms now (6.4 GB moved: 0.75 of the measured copy bandwidth).
 template <typename real>
-__global__ void deviation_kernel(const real* src, real* dst, long long cells, int Vp,
-                                 const __grid_constant__ ModelArgs m, int to_dev, CellMap map) {
-  __shared__ real buf[2 * MAXQ * MAXQ];
+struct RestValue {  // R of one velocity
+  real hi, lo;
+};
+template <typename real>
+__device__ __forceinline__ RestValue<real> rest_value(double R) {
+  RestValue<real> r;
+  r.hi = real(R);
+  r.lo = real(R - double(r.hi));
+  return r;
+}
+// x + sgn R, rounded once
+__device__ __forceinline__ float add_rest(float x, RestValue<float> r, float sgn) {
+  float s, e;
+  two_sum(x, sgn * r.hi, s, e);
+  const float t = __fadd_rn(s, __fadd_rn(e, sgn * r.lo));
+  return fabsf(s) <= 3.402823466e38f ? t : s;  // Inf and NaN stay what the plain sum gives
+}
+__device__ __forceinline__ double add_rest(double x, RestValue<double> r, double sgn) { return x + sgn * r.hi; }
+
+template <typename real, int NV, int CH>
+__global__ void __launch_bounds__(256) deviation_kernel(const real* src, real* dst, long long cells, int Vp,
+                                                        const __grid_constant__ ModelArgs m, int to_dev, CellMap map) {
+  using P = pair_t<real>;
+  const int lane = threadIdx.x & 31;
   const int V = m.nq0 * m.nq1;
-  for (long long c = blockIdx.x; c < cells; c += gridDim.x) {
+  RestValue<real> R[CH][NV];
+#pragma unroll
+  for (int k = 0; k < CH; ++k)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const int v = (32 * k + lane) * NV + q;
+      const int i = v < V ? v / m.nq1 : 0, j = v < V ? v - i * m.nq1 : 0;
+      R[k][q] = rest_value<real>(m.w0[i] * m.w1[j]);
+    }
+  const real sgn = to_dev ? real(-1) : real(1);
+  const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long c = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < cells; c += nw) {
     const long long cc = caller_cell(map, c);  // device cell c is the caller's cell cc
-    if (to_dev) {
-      for (int x = threadIdx.x; x < 2 * V; x += blockDim.x) buf[x] = src[cc * 2 * V + x];
-      __syncthreads();
-      for (int x = threadIdx.x; x < 2 * Vp; x += blockDim.x) {
-        const int v = x >> 1, d = x & 1;
-        real val = real(0);
-        if (v < V) {
-          const int i = v / m.nq1, j = v - i * m.nq1;
-          val = real(double(buf[d * V + v]) - m.w0[i] * m.w1[j]);
+    const real* a = src + (to_dev ? cc * 2 * V : c * 2 * Vp);
+    real* o = dst + (to_dev ? c * 2 * Vp : cc * 2 * V);
+    P x[CH][NV];
+#pragma unroll
+    for (int k = 0; k < CH; ++k) {
+      const int v = (32 * k + lane) * NV;
+#pragma unroll
+      for (int q = 0; q < NV; ++q) x[k][q] = p_set(real(0));
+      if (v < V) {
+        if (to_dev) {
+          if constexpr (NV == 2) {
+            const P f1 = p_load(a + v), f2 = p_load(a + V + v);
+            x[k][0] = p_make(f1.x, f2.x), x[k][1] = p_make(f1.y, f2.y);
+          } else {
+            x[k][0] = p_make(a[v], a[V + v]);
+          }
+        } else {
+          if constexpr (NV == 2) {
+            const float4 y = *reinterpret_cast<const float4*>(a + 2 * v);
+            x[k][0] = p_make(y.x, y.y), x[k][1] = p_make(y.z, y.w);
+          } else {
+            x[k][0] = p_load(a + 2 * v);
+          }
         }
-        dst[c * 2 * Vp + x] = val;
-      }
-    } else {
-      for (int x = threadIdx.x; x < 2 * Vp; x += blockDim.x) buf[x] = src[c * 2 * Vp + x];
-      __syncthreads();
-      for (int x = threadIdx.x; x < 2 * V; x += blockDim.x) {
-        const int d = x >= V, v = x - d * V;
-        const int i = v / m.nq1, j = v - i * m.nq1;
-        dst[cc * 2 * V + x] = real(double(buf[2 * v + d]) + m.w0[i] * m.w1[j]);
+#pragma unroll
+        for (int q = 0; q < NV; ++q)
+          x[k][q] = p_make(add_rest(x[k][q].x, R[k][q], sgn), add_rest(x[k][q].y, R[k][q], sgn));
       }
     }
-    __syncthreads();
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < CH; ++k) {
+      const int v = (32 * k + lane) * NV;
+      if (to_dev) {
+        if (v < Vp) {  // the padding velocities are zero
+          if constexpr (NV == 2)
+            *reinterpret_cast<float4*>(o + 2 * v) = make_float4(x[k][0].x, x[k][0].y, x[k][1].x, x[k][1].y);
+          else p_store(o + 2 * v, x[k][0]);
+        }
+      } else if (v < V) {
+        if constexpr (NV == 2) {
+          p_store(o + v, p_make(x[k][0].x, x[k][1].x));
+          p_store(o + V + v, p_make(x[k][0].y, x[k][1].y));
+        } else {
+          o[v] = x[k][0].x, o[V + v] = x[k][0].y;
+        }
+      }
+    }
+    __syncwarp();
   }
+}
+
+template <typename real, int NV>
+static cudaError_t go_deviation(const real* src, real* dst, long long cells, int Vp, const ModelArgs& m, int to_dev,
+                                cudaStream_t s, CellMap map) {
+  // eight warps a CTA, up to eight CTAs an SM, a row's loads in flight in each warp
+  long long blocks = (cells + 7) / 8;
+  if (blocks > 152 * 8) blocks = 152 * 8;
+  const int g = int(blocks > 0 ? blocks : 1), chunks = (Vp + 32 * NV - 1) / (32 * NV);
+  if (chunks <= 4) deviation_kernel<real, NV, 4><<<g, 256, 0, s>>>(src, dst, cells, Vp, m, to_dev, map);
+  else if (chunks <= 8) deviation_kernel<real, NV, 8><<<g, 256, 0, s>>>(src, dst, cells, Vp, m, to_dev, map);
+  else if (chunks <= 16) deviation_kernel<real, NV, 16><<<g, 256, 0, s>>>(src, dst, cells, Vp, m, to_dev, map);
+  else if constexpr (NV == 1) deviation_kernel<real, 1, 32><<<g, 256, 0, s>>>(src, dst, cells, Vp, m, to_dev, map);
+  else return cudaErrorInvalidValue;  // MAXQ^2 velocities are 16 chunks of 64
+  return cudaGetLastError();
 }
 
 template <typename real>
 cudaError_t launch_deviation(const real* src, real* dst, long long cells, int Vp, const ModelArgs& m,
                              int to_deviation, cudaStream_t s, CellMap map) {
-  const long long blocks = cells < 152 * 8 ? cells : 152 * 8;
-  deviation_kernel<real><<<int(blocks > 0 ? blocks : 1), 256, 0, s>>>(src, dst, cells, Vp, m, to_deviation, map);
-  return cudaGetLastError();
+  // two velocities a lane (8- and 16-byte accesses) where the caller's rows and buffer allow it
+  if constexpr (sizeof(real) == 4) {
+    const void* caller = to_deviation ? static_cast<const void*>(src) : static_cast<const void*>(dst);
+    if (m.nq0 * m.nq1 == Vp && reinterpret_cast<uintptr_t>(caller) % 8 == 0)
+      return go_deviation<real, 2>(src, dst, cells, Vp, m, to_deviation, s, map);
+  }
+  return go_deviation<real, 1>(src, dst, cells, Vp, m, to_deviation, s, map);
 }
 
 // ---------------------------------------------------------------- moments (FP64), one warp per cell

@@ -84,6 +84,10 @@ struct CellMap {
 };
 __host__ __device__ __forceinline__ long long caller_cell(const CellMap& m, long long q) {
   if (m.nx == 0) return q;
+  if (q < 0x7fffffffll) {  // a 32-bit division where it reaches
+    const unsigned s = unsigned(q) / unsigned(m.nx), p = unsigned(q) - s * unsigned(m.nx);
+    return (long long)p * m.nl + s;
+  }
   const long long s = q / m.nx, p = q - s * m.nx;
   return p * m.nl + s;
 }
@@ -102,7 +106,8 @@ cudaError_t launch_seed(real* F, long long cells, int Vp, const ModelArgs& m, co
 // Caller layout F (per cell: f' then f'', V values each) to and from the device
 // layout (per cell: Vp interleaved (f', f'') pairs of the deviation D = F - R;
 // padding zero).  to_deviation = 1: caller -> device, 0: device -> caller; each
-// element is summed in double.  src and dst may be the same buffer when V == Vp and
+// element is summed with R to twice its own precision and rounded once (single precision; in
+// double precision a plain sum).  src and dst may be the same buffer when V == Vp and
 // the cell map is the identity.
 template <typename real>
 cudaError_t launch_deviation(const real* src, real* dst, long long cells, int Vp, const ModelArgs& m,
