@@ -352,9 +352,9 @@ vlb_status setup_large(vlb_ctx* c) {
 
 // Rows per lambda segment and segments of a channel launch shape.  A fixed ts
 // is used as given (at least 3 rows per segment, the last one included); ts = 0
-// picks the segment count that minimises waves x (rows + 6) over the SMs of the
-// device, one resident CTA each: the 6 rows are the warm-up of a segment (window
-// rows below it and the equilibria of its first three rows).
+// picks the segment count that minimises waves x (rows + 6) over the resident
+// CTAs of the device: the 6 rows are the warm-up of a segment (its first four
+// rows' loads, the windows below it and the equilibria of its first three rows).
 void channel_segments(const vlb_ctx* c, const ChanVariant& v, int* seglen, int* nseg) {
   const int nl = c->cdesc.nl, nstrips = c->cdesc.nx / v.tp;
   auto count = [&](int L) {  // segments of L rows, 0 if the last would be shorter than 3
@@ -368,7 +368,7 @@ void channel_segments(const vlb_ctx* c, const ChanVariant& v, int* seglen, int* 
     *seglen = L, *nseg = n;
     return;
   }
-  const int sms = c->sms > 0 ? c->sms : 1;
+  const int sms = c->sms > 0 ? c->sms * c->chan_per_sm : 1;
   long long best = -1;
   *seglen = nl, *nseg = 1;
   for (int want = 1; want <= nl / 3; ++want) {
@@ -388,8 +388,8 @@ vlb_status do_chan_stage(vlb_ctx* c, int k, int prev, int out, bool clb = false)
   a.Fl = static_cast<const real*>(c->F[c->cur]);
   a.Fout = static_cast<real*>(c->F[out]);
   const double ca[3] = {0.0, 0.75, 1.0 / 3.0}, cc[3] = {1.0, 0.25, 2.0 / 3.0};
-  a.ca = real(ca[k - 1]);
-  a.ccdt = real(cc[k - 1] * c->inst[0].dt);
+  a.ca.x = a.ca.y = real(ca[k - 1]);
+  a.ccdt.x = a.ccdt.y = real(cc[k - 1] * c->inst[0].dt);
   a.tables = c->d_ctab;
   if constexpr (sizeof(real) == 8) a.geo = clb ? c->d_clbcgeo : c->d_cgeo;
   else a.geo = clb ? c->d_clbcgeof : c->d_cgeof;
@@ -407,7 +407,7 @@ vlb_status do_chan_stage(vlb_ctx* c, int k, int prev, int out, bool clb = false)
   const ChanVariant& v = c->cvariants[c->variant];
   channel_segments(c, v, &a.seglen, &a.nseg);
   const int grid = (a.nx / v.tp) * a.nseg;
-  cudaError_t e = launch_channel<real>(v, a, c->chan_kp.data(), c->nq0, c->nq1, grid, c->stream, clb);
+  cudaError_t e = launch_channel<real>(a, c->chan_kp.data(), c->nq0, c->nq1, c->margs.kind1, grid, c->stream, clb);
   if (e != cudaSuccess) return cuda_fail(c, e, "channel stage kernel launch");
   c->launches += 1;
   return VLB_OK;
@@ -417,8 +417,8 @@ vlb_status do_chan_stage(vlb_ctx* c, int k, int prev, int out, bool clb = false)
 // on the context stream.
 vlb_status upload_channel_tables(vlb_ctx* c) {
   std::vector<unsigned char> tb;
-  const bool ok = c->prec == VLB_FP64 ? channel_tables<double>(c->nq0, c->nq1, c->ax, c->margs, c->cdesc.T0, &tb)
-                                      : channel_tables<float>(c->nq0, c->nq1, c->ax, c->margs, c->cdesc.T0, &tb);
+  const bool ok = c->prec == VLB_FP64 ? channel_tables<double>(c->nq0, c->nq1, c->margs, c->cdesc.T0, &tb)
+                                      : channel_tables<float>(c->nq0, c->nq1, c->margs, c->cdesc.T0, &tb);
   if (!ok) return fail(c, VLB_ERR_UNSUPPORTED, "no channel kernel for this velocity set");
   if (!c->d_ctab) {
     VLB_CUDA(c, cudaMalloc(&c->d_ctab, tb.size()));
@@ -973,19 +973,15 @@ vlb_status vlb_create_channel(const vlb_model* model, vlb_precision prec, const 
   c->Vp = (c->V + 3) / 4 * 4;
   c->esize = prec == VLB_FP64 ? 8 : 4;
   {
-    // launch shapes: shared memory within an SM's, whole strips of columns; the
-    // single-precision CUDA-core force needs the split force block, the double-precision
-    // kernel contracts on its own (its shapes are the tc = 0 ones)
-    const bool kp_ok = channel_force_pairs(nq0, nq1, c->ax, &c->chan_kp);
-    if (!kp_ok) c->chan_kp.assign(16384, 0);
+    // launch shapes: shared memory within an SM's, whole strips of columns, the force block's structure
+    const bool kp_ok = prec == VLB_FP64 ? channel_force_pairs<double>(nq0, nq1, c->ax, &c->chan_kp)
+                                        : channel_force_pairs<float>(nq0, nq1, c->ax, &c->chan_kp);
     ChanVariant all[8];
-    const int n = channel_variants(nq0, nq1, all);
+    const int n = kp_ok ? channel_variants(nq0, nq1, all) : 0;
     for (int i = 0; i < n; ++i) {
-      const size_t sm = prec == VLB_FP64 ? channel_smem_bytes<double>(all[i], nq0, nq1)
-                                         : channel_smem_bytes<float>(all[i], nq0, nq1);
+      const size_t sm = prec == VLB_FP64 ? channel_smem_bytes<double>(all[i], nq0, nq1, &c->chan_per_sm)
+                                         : channel_smem_bytes<float>(all[i], nq0, nq1, &c->chan_per_sm);
       if (!(sm > 0 && sm <= 227 * 1024 && nx % all[i].tp == 0)) continue;
-      if (prec == VLB_FP64 && all[i].tc) continue;
-      if (prec == VLB_FP32_BULK && !all[i].tc && !kp_ok) continue;
       c->cvariants[c->n_cvariants++] = all[i];
     }
     // no vielbein kernel for this velocity set: the context can still run the Cartesian split
@@ -1031,21 +1027,22 @@ vlb_status vlb_create_channel(const vlb_model* model, vlb_precision prec, const 
     const double dchi = chi(xf[p + 1]) - chi(xf[p]);
     for (int s = 0; s < nl; ++s) {
       ChanCell<double> g{};
-      g.am = sqrt(1.0 + lf[s] * lf[s] * dp * dp) / (1.0 + ph);
-      g.ap = sqrt(1.0 + lf[s + 1] * lf[s + 1] * dp * dp) / (1.0 + ph);
+      const double am = sqrt(1.0 + lf[s] * lf[s] * dp * dp) / (1.0 + ph);
+      const double ap = sqrt(1.0 + lf[s + 1] * lf[s + 1] * dp * dp) / (1.0 + ph);
       const double rm = sqrt(1.0 + lc[s] * lc[s] * dpm * dpm), rp = sqrt(1.0 + lc[s] * lc[s] * dpp * dpp);
       g.bm = (1.0 + phm) / rm;
       g.bp = (1.0 + php) / rp;
       g.cm = lc[s] * dpm * (1.0 + phm) / rm;
       g.cp = lc[s] * dpp * (1.0 + php) / rp;
       const double dl = lf[s + 1] - lf[s];
-      g.idl = 1.0 / dl;
-      g.idx = 1.0 / dchi;
+      g.ap[0] = g.ap[1] = ap / dl;
+      g.nam[0] = g.nam[1] = -am / dl;
+      g.idx[0] = g.idx[1] = 1.0 / dchi;
       g.glxl = (g.bp - g.bm) / dchi;
-      g.glxx = -(g.ap - g.am) / dl + (g.cp - g.cm) / dchi;
+      g.glxx = -(ap - am) / dl + (g.cp - g.cm) / dchi;
       gd[size_t(s) * nx + p] = g;  // device cell order: s * n_xi + p
-      const double* src = &g.am;
-      float* dst = &gf[size_t(s) * nx + p].am;
+      const double* src = g.ap;
+      float* dst = gf[size_t(s) * nx + p].ap;
       for (int k = 0; k < 12; ++k) dst[k] = float(src[k]);
     }
   }
@@ -1258,17 +1255,18 @@ static vlb_status set_channel_formulation(vlb_ctx* c, int formulation) {
       const double a = 1.0 / (1.0 + cphi(xc)), dph = cdphi(xc);
       for (int s2 = 0; s2 < nl; ++s2) {
         ChanCell<double> g{};
-        g.am = g.ap = a;
-        g.glxl = a * lf[s2] * dph;
-        g.glxx = a * lf[s2 + 1] * dph;
+        const double idl = 1.0 / (lf[s2 + 1] - lf[s2]);  // V^lambda / d lambda at both faces
+        g.ap[0] = g.ap[1] = a * idl;
+        g.nam[0] = g.nam[1] = -a * idl;
+        g.glxl = a * lf[s2] * dph * idl;
+        g.glxx = a * lf[s2 + 1] * dph * idl;
         g.bm = 1.0 + cphi(xm);
         g.bp = 1.0 + cphi(xp);
         g.cm = g.cp = 0.0;
-        g.idl = 1.0 / (lf[s2 + 1] - lf[s2]);
-        g.idx = 1.0 / (cchi(xp) - cchi(xm));
+        g.idx[0] = g.idx[1] = 1.0 / (cchi(xp) - cchi(xm));
         gd[size_t(s2) * nx + p] = g;
-        const double* src = &g.am;
-        float* dst = &gf[size_t(s2) * nx + p].am;
+        const double* src = g.ap;
+        float* dst = gf[size_t(s2) * nx + p].ap;
         for (int q = 0; q < 12; ++q) dst[q] = float(src[q]);
       }
     }
@@ -1879,7 +1877,7 @@ int vlb_channel_variants(const vlb_ctx* c, int* ts, int* tp, int* nt, int max) {
 
 int vlb_channel_variant_tensor_cores(const vlb_ctx* c, int v) {
   if (!c || c->kind != 1 || v < 0 || v >= c->n_cvariants) return VLB_ERR_INVALID;
-  return c->cvariants[v].tc;
+  return 0;  // every launch shape contracts on the CUDA cores
 }
 
 int vlb_variants(const vlb_ctx* c, int* tc, int* nt, int* persistent, int max) {

@@ -1,36 +1,34 @@
 // One TVD-RK3 stage of the gradually expanding channel in the vielbein frame
 // (Sec. VII.A-C, Eq. canalie_boltz), as a marching kernel: each CTA owns a
-// strip of TP adjacent xi-columns and walks up a segment of lambda rows
-// (wall-normal, the contiguous direction of the cell index p * n_lambda + s).
-// For every row s it
+// strip of TP = 4 adjacent xi-columns and walks up a segment of lambda rows
+// (wall-normal).  A thread owns one velocity on all four columns.  Step s of the march
 //
-//   - pushes row s+3 into a per-thread six-row register window (f', f'') of
-//     its (column, velocity), so the lambda-WENO-5 interface value s+1/2
-//     comes from registers and every lambda interface is reconstructed once;
-//   - reduces the moments of row s+3; two dedicated equilibrium warps turn
-//     them into the row's truncated equilibrium (Sec. IV.D) asynchronously,
-//     handing rows over through mbarrier rings, two or three rows ahead of use;
-//   - reconstructs the xi interfaces of row s from a shared-memory ring that
-//     bulk copies (cp.async.bulk, mbarrier completion) fill PD rows ahead;
-//   - contracts the momentum-space force matrices of Eq. (canalie_boltz)
-//     over the row's cells: in single precision either on the CUDA cores
-//     (packed FP32x2 fmas on the reflection-split matrices, run by two extra
-//     warps) or on the tensor cores (mma.sync m16n8k8 TF32 with a hi/lo split
-//     of both operands, three products per tile), one template instance each,
-//     chosen per context by timing; in double precision on the CUDA cores;
-//   - combines advection, force, BGK relaxation and the RK3 weights and
-//     stores the cell's updated populations straight to global memory.
+//   - reconstructs the five xi interfaces of row s in one walk along the strip (the row and its
+//     halo come from a shared-memory ring that bulk copies fill) and the lambda interface of
+//     every column from the column's window of differences, kept in registers, so that each
+//     lambda interface is reconstructed once and each xi interface once per strip;
+//   - combines advection, force, BGK relaxation and the RK3 weights of row s and stores it
+//     straight to global memory;
+//   - prepares the rows ahead, by warp role: the momentum-space force of row s + 1, the moments
+//     and truncated equilibria of row s + 3, the inflow factors of row s + 2 and the reservoir
+//     ghost cells of row s + 1.
 //
-// The march is software-pipelined: step s combines row s-1 while it builds row
-// s's interface values and force (double-buffered by row parity), so all warp
-// roles work between the one barrier a step takes, and each column warp waits
-// for its own bulk copies.
+// One CTA barrier a step; two CTAs a SM overlap each other's barriers and serial parts (single
+// precision).  What bounds it: latency, with 12 warps a SM at 168 registers each; then the FP32
+// pipe (half busy: about 290 of its cycles per warp and cell-velocity row, of which the ten
+// reconstructions of a row's four columns take 160).  Why four columns a thread: the strip's xi
+// walk and the windows cost 33 packed operations an interface where five cells loaded afresh cost
+// 44 (windows of two columns or of raw rows in shared memory, twice the warps or half the
+// registers, measured 13.0 - 14.1 ms a step against 9.85); why unrolled: the same loop rolled
+// halves the reconstructions in flight (14.5).  A barrier at the step's end keeps the warps on
+// the same instructions; waiting later, at the next combine, lost more to instruction fetches
+// (12.5).  2048 x 512 x 192, single precision, a step of three stages: 20.3 ms for one thread per
+// (column, velocity) with 1024 threads of 64 registers, 9.85 ms now, 4.4 GB of 0.65 TB/s a
+// stage; double precision, 256 x 64: 10.9 and 7.35 ms; Cartesian split, 512 x 256: 2.39 and 1.17.
 //
-// Boundaries: the centreline mirror (Sec. VII.C.3) fills the window at the
-// bottom of the march, the diffuse wall (Sec. VII.C.4) at its top with n_w per
-// column from the zero-mass-flux balance, and the inlet/outlet reservoirs give
-// the xi-halo values past the first and last strip, evaluated by each thread
-// whose stencil reaches them.
+// Boundaries: the centreline mirror (Sec. VII.C.3) at the bottom of the march, the diffuse wall
+// (Sec. VII.C.4) at its top with n_w per column from the zero-mass-flux balance, and the
+// inlet/outlet reservoirs as halo cells of the first and last strip.
 //
 // Distribution buffers hold the deviation D = F - R from the rest state
 // (ModelArgs), with (f', f'') interleaved per velocity: a cell row is
@@ -40,57 +38,45 @@
 
 namespace vlb {
 
-// Per-cell geometry of the channel (Sec. VII.A): interface factors of
-// V^lambda = a p^lambda and V^xi = b p^xi - c p^lambda, 1/d lambda_s,
-// 1/d chi^xi_p and the discrete connection coefficients.
+// Per-cell geometry of the channel (Sec. VII.A): V^lambda = a p^lambda and V^xi = b p^xi - c p^lambda
+// at the interfaces, 1/d chi^xi_p and the discrete connection coefficients.  The interface factors
+// of lambda carry 1/d lambda_s, and what multiplies a pair is stored twice (the operand of a
+// packed operation).
 template <typename T>
 struct ChanCell {
-  T am, ap;          // a at s-1/2, s+1/2
-  T bm, bp, cm, cp;  // b, c at p-1/2, p+1/2
-  T idl, idx;        // 1 / d lambda_s, 1 / d chi_p
-  T glxl, glxx;      // Gamma_{l x l}, Gamma_{l x x}
-  T pad0, pad1;
+  T ap[2], nam[2], idx[2];  // a / d lambda at s+1/2, -a / d lambda at s-1/2, 1 / d chi_p
+  T bm, cm, bp, cp;         // b, c at p-1/2, p+1/2
+  T glxl, glxx;             // Gamma_{l x l}, Gamma_{l x x}
 };
 static_assert(sizeof(ChanCell<float>) == 48 && sizeof(ChanCell<double>) == 96, "bulk-copied geometry rows");
 
-// Tile counts of the force contractions of one cell on m16n8k8 tensor-core tiles.
-// lambda: D = [K0; Kt0] F, rows of the A operand interleaved per m-tile t as
-//   (K0 rows 8t..8t+7, Kt0 rows 8t..8t+7), F as the B operand [i'][2 j + d];
-// xi: D = F [K1^T | Kt1^T], F as the A operand with rows (i, d) of m-tile t =
-//   (8t + r/2, r & 1), the B operand [j'][2 j + e] (e = 0: K1, e = 1: Kt1), j' >= Q1 zero.
 template <int Q0, int Q1>
 struct ChanShape {
   static constexpr int V = Q0 * Q1;
-  static constexpr int ROW = 2 * V;         // reals per cell row
-  static constexpr int NWC = V / 32;        // warps per column (one velocity per thread)
-  static constexpr int MT = Q0 / 8;         // m-tiles (both contractions)
-  static constexpr int KKL = Q0 / 8;        // k-steps of the lambda contraction
-  static constexpr int NN = Q1 / 4;         // n-tiles (both contractions)
-  static constexpr int KKX = (Q1 + 7) / 8;  // k-steps of the xi contraction
-  static constexpr int S = 2 * NN;          // force subtasks per cell (one n-tile each)
-  static constexpr int EQW = Q0 + Q1 + 4;   // per-cell equilibrium record: n g0, g1, T, 1/tau, u^xi, pad
-  static_assert(V % 32 == 0 && Q0 % 8 == 0 && Q1 % 4 == 0, "velocity set shape of the channel kernel");
-  static_assert(Q0 + Q1 <= 32, "one lane per equilibrium factor");
+  static constexpr int ROW = 2 * V;        // reals per cell row
+  static constexpr int NW = V / 32;        // warps: one thread per velocity
+  static constexpr int TP = 4;             // columns per strip
+  // per-cell equilibrium record, in pairs: n g0_i twice, g1_j twice, (1, T), -1/tau twice, (u^xi, 0)
+  static constexpr int EQW = 2 * (Q0 + Q1 + 3);
+  static_assert(V % 32 == 0 && Q0 % 2 == 0 && Q1 % 2 == 0, "velocity set shape of the channel kernel");
+  static_assert(Q0 % 8 == 0 && Q0 + Q1 <= 32, "eight lanes per cell, four equilibrium factors each");
 };
 
-// Model tables of a channel context, in device memory, bulk-copied into each
-// CTA's shared memory.  gw0/gw1 are the factors of f_eq(1, 0, T0), the wall and
-// reservoir equilibrium at rest (they change with T0).
+// Model tables of a channel context, in device memory, copied into each CTA's shared memory.
+// gw0/gw1 are the factors of f_eq(1, 0, T0), the wall and reservoir equilibrium at rest (they
+// change with T0); sc0 sc1 is the power-of-two scale of the WENO walk (WenoWin) per velocity.
 template <typename real, int Q0, int Q1>
 struct alignas(16) ChanTables {
-  using S = ChanShape<Q0, Q1>;
-  uint32_t fl[S::MT][S::KKL][2][32][4];  // lambda A fragments, [hi|lo] TF32 bit patterns
-  uint32_t fx[S::KKX][S::NN][2][32][2];  // xi B fragments, [hi|lo]
-  real K0[Q0 * Q0], Kt0[Q0 * Q0];        // d/dp^lambda, d/dp^lambda (p^lambda .)
-  real K1[Q1 * Q1], Kt1[Q1 * Q1];        // d/dp^xi, d/dp^xi (p^xi .)
-  real p0[Q0], p1[Q1], iw0[Q0], iw1[Q1], w0[Q0], w1[Q1];
-  real tab0[Q0 * MAXN], tab1[Q1 * MAXN];  // equilibrium tables [k][s]
+  real p0[Q0], p1[Q1], w0[Q0], w1[Q1], sc0[Q0], sc1[Q1], isc0[Q0], isc1[Q1];
+  real tab[MAXN * (Q0 + Q1)];  // equilibrium tables of both axes, [s][k] (zero beyond an axis' order)
   real gw0[Q0], gw1[Q1];
   double wall_den;  // sum over p^lambda < 0 of gw0 p^lambda times sum of gw1: incoming flux of f_eq(1, 0, T0)
   double ref_flux_pos;  // sum over p^lambda > 0 of p^lambda R (ModelArgs)
-  // sums of R (ModelArgs: n, rho u0, rho u1, energy) as (hi, lo) in the bulk type (lo = 0 in double)
-  real ref_hi[4], ref_lo[4];
-  int N0, N1, kind0, kind1;
+  // sums of R (ModelArgs: n, rho u0, rho u1, energy) as (hi, lo) in the bulk type (lo = 0 in
+  // double), and the sum of the products w0_i w1_j of the bulk-type weights, the part of the mass
+  // that the stage's f_eq - R subtracts
+  real ref_hi[4], ref_lo[4], ref_sum[2];
+  int nmax, kind1, pad[2];  // the larger expansion order; axis 1 half range
 };
 
 // Host-side description of a channel context: grid size, Kn, time step, reservoirs,
@@ -115,8 +101,8 @@ struct ChanArgs {
   int nl, nx;
   int seglen;  // rows per lambda segment (the last one may be shorter, >= 3 rows)
   int nseg;
-  // Fout = F_prev + ca (F_l - F_prev) + ccdt L[F_prev] (see StageArgs)
-  real ca, ccdt;
+  // Fout = F_prev + ca (F_l - F_prev) + ccdt L[F_prev] (see StageArgs), each twice; ca = 0: no F_l
+  pair_t<real> ca, ccdt;
   real ikn, n_in, n_out, T0;  // 1/Kn, reservoir densities, wall and reservoir temperature
   unsigned long long max_polls;
   // flow-rate ends (Sec. VII.C.1-2), when flow != 0: per end e and row s,
@@ -127,327 +113,279 @@ struct ChanArgs {
 };
 
 // Shared-memory carve-up of a CTA, identical on host and device.  The ring holds
-// rows s-1 .. s+3+PD of the strip, each with its xi-halo (TP + 6 cells): row s-1
-// for the geometry of the combine, row s for the xi reconstruction and the force,
-// s+3 for the window, and PD rows in flight (bulk copies issued PD steps ahead).
-// The xi interface values and the force results are double-buffered by row parity:
-// step s writes row s's while it combines row s-1 from the other half.
-template <typename real, int Q0, int Q1, int TP>
+// rows s .. s+4 of the strip, each with its xi-halo (TP + 6 cells): row s for the xi
+// reconstruction and the combine, s+1 for the force, s+2 and s+3 for the lambda windows and the
+// moments, s+4 in flight (issued when step s begins, after the barrier that ends the use of row s-1).  Cells are padded so that the force tasks of neighbouring cells fall on consecutive
+// banks: cell stride = Q1 pairs modulo 128 bytes.
+template <typename real, int Q0, int Q1>
 struct ChanSmem {
   using S = ChanShape<Q0, Q1>;
   using Tab = ChanTables<real, Q0, Q1>;
   static constexpr bool F32 = sizeof(real) == 4;
-  static constexpr int NSYNC = (TP + 1) * S::V;  // TP column groups and one extra group, in step
-  static constexpr int NT = NSYNC + 64;          // and two equilibrium warps running ahead of them
-  static constexpr int NPR = 4;                  // moment-partial ring (rows r .. r+3)
-  // prefetch distance in rows: double precision copies each row in the step that needs it,
-  // which keeps its larger ring within an SM's shared memory
-  static constexpr int PD = F32 ? 2 : 0;
-  static constexpr int NRING = 5 + PD;        // ring rows
-  static constexpr int NB = PD + 1;           // mbarriers of the step groups (one more for the prologue)
-  static constexpr int NEQ = 8;               // equilibrium records (rows s-1 .. s+3 in use), a power of 2
-  static constexpr int RC = TP + 6;           // cells of a ring row
+  static constexpr int TP = S::TP;
+  static constexpr int NT = S::V;
+  static constexpr int NRING = 5;
+  static constexpr int RC = TP + 6;  // cells of a ring row
+  static constexpr int NEQ = 4;      // equilibrium records (rows s .. s+3)
+  static constexpr int NRES = 2;     // inflow factors (rows s+1, s+2)
   static constexpr size_t al(size_t x) { return (x + 15) & ~size_t(15); }
   static constexpr size_t rowb = size_t(S::ROW) * sizeof(real);
-  // mbarriers: NB step groups, the prologue, NPR partials-ready, NEQ equilibrium-ready
-  static constexpr size_t bar_off = 0;
-  static constexpr int NBAR = NB + 1 + NPR + NEQ;
-  static constexpr size_t tab_off = 128;
+  static constexpr size_t pad = (size_t(Q1) * 2 * sizeof(real)) % 128;
+  static constexpr int CS = int((rowb + pad) / sizeof(real));  // reals from cell to cell, in the ring and in lbl
+  static constexpr int XS = 2 * Q1 + 2;                        // reals from row i to row i+1 of a cell in lbx
+  static constexpr size_t bar_off = 0;  // one mbarrier per ring slot
+  static constexpr size_t tab_off = 64;
   static constexpr size_t ring_off = al(tab_off + sizeof(Tab));
-  static constexpr size_t geo_off = ring_off + size_t(NRING) * RC * rowb;
-  static constexpr size_t xif_off = al(geo_off + size_t(NRING) * TP * sizeof(ChanCell<real>));
-  static constexpr size_t lbl_off = xif_off + size_t(2) * (TP + 1) * S::V * 2 * sizeof(real);
-  static constexpr size_t lbuf_rows = F32 ? 2 * TP : 0;  // force results of two rows (single precision only)
-  static constexpr size_t lbx_off = lbl_off + lbuf_rows * rowb;
-  static constexpr size_t eq_off = lbx_off + lbuf_rows * rowb;
+  static constexpr size_t geo_off = ring_off + size_t(NRING) * RC * CS * sizeof(real);
+  static constexpr size_t lbl_off = geo_off + size_t(NRING) * TP * sizeof(ChanCell<real>);
+  static constexpr size_t lbx_off = lbl_off + size_t(2) * TP * CS * sizeof(real);
+  static constexpr size_t eq_off = al(lbx_off + size_t(2) * TP * Q0 * XS * sizeof(real));
   static constexpr size_t res_off = al(eq_off + size_t(NEQ) * TP * S::EQW * sizeof(real));
-  static constexpr size_t resn_off = al(res_off + size_t(NEQ) * 2 * Q1 * sizeof(real));
-  static constexpr size_t mvs_off = al(resn_off + size_t(NEQ) * 2 * sizeof(real));
-  static constexpr size_t red_off = al(mvs_off + size_t(TP + 2) * 4 * MAXN * sizeof(real));
-  static constexpr size_t wred_off = al(red_off + size_t(NPR) * TP * S::NWC * 4 * sizeof(real));
-  static constexpr size_t nwv_off = al(wred_off + size_t(2) * TP * S::NWC * sizeof(real));  // two wall sums
+  static constexpr size_t resn_off = al(res_off + size_t(NRES) * 2 * Q1 * sizeof(real));
+  static constexpr size_t mvs_off = al(resn_off + size_t(NRES) * 2 * sizeof(real));
+  static constexpr size_t wred_off = al(mvs_off + size_t(TP + 2) * 4 * MAXN * sizeof(real));
+  static constexpr size_t nwv_off = al(wred_off + size_t(2) * TP * S::NW * sizeof(real));  // two wall sums
   static constexpr size_t bytes = al(nwv_off + size_t(TP) * sizeof(double));
-  static_assert(sizeof(Tab) % 16 == 0, "tables are one bulk copy");
-  static_assert(rowb % 16 == 0 && (TP * sizeof(ChanCell<real>)) % 16 == 0, "rows are bulk copies");
-  static_assert(ring_off % 16 == 0 && geo_off % 16 == 0, "bulk destinations are 16-byte aligned");
-  static_assert(xif_off % 16 == 0 && lbl_off % 16 == 0 && lbx_off % 16 == 0, "pair arrays are aligned");
-  static_assert(bar_off + NBAR * sizeof(uint64_t) <= tab_off, "mbarriers fit before the tables");
-  static_assert((NEQ & (NEQ - 1)) == 0, "record slots by mask");
-  static_assert(TP >= 3, "only the end strips' stencils reach past the inlet / outlet");
-  static_assert(NT <= 1024, "one thread per (column, velocity) and an extra group");
+  static_assert(rowb % 128 == 0 && pad % 16 == 0, "cells are bulk copies");
+  static_assert((TP * sizeof(ChanCell<real>)) % 16 == 0, "geometry rows are bulk copies");
+  static_assert(ring_off % 16 == 0 && geo_off % 16 == 0 && lbl_off % 16 == 0 && lbx_off % 16 == 0, "alignment");
+  static_assert(NRING * sizeof(uint64_t) <= tab_off, "mbarriers fit before the tables");
+  static_assert((NEQ & (NEQ - 1)) == 0 && (NRES & (NRES - 1)) == 0, "record slots by mask");
+  // resident CTAs a SM the registers are sized for (228 KB of shared memory, 1 KB of it per CTA)
+  static constexpr int fit = int((228 * 1024) / (bytes + 1024));
+  static constexpr int min_ctas = sizeof(real) == 8 ? 1 : (fit * NT * 168 <= 65536 ? fit : 65536 / (NT * 168));
 };
 
-// Moment vector of the truncated equilibrium on one axis (the recurrences of
-// eq_moment_vector) with the loop unrolled to MAXN terms, the 1/l factors as
-// constants and one reciprocal of T: no division on the per-cell path.
+// Moment vector of the truncated equilibrium on one axis (the recurrences of eq_moment_vector),
+// every entry up to order nmax, with the 1/l factors as constants and one reciprocal of T.
 template <typename R>
-__device__ __forceinline__ void eq_moments_fast(int kind, int N, R u, R T, R* m) {
+__device__ __forceinline__ void eq_moments_fast(int kind, int nmax, R u, R T, R* m) {
+  R a, b, c;  // m_l = (u m_{l-1} + h c m_{l-2}) f: h = 1, f = 1 / l (full range) or h = l - 1, f = 1
   if (kind == 0) {
-    R a = R(1), b = u;
-    m[0] = a;
-    m[1] = b;
-#pragma unroll
-    for (int l = 2; l < MAXN; ++l) {
-      const R x = (u * b + (T - R(1)) * a) * R(1.0 / l);
-      if (l <= N) m[l] = x;
-      a = b;
-      b = x;
-    }
+    a = R(1), b = u, c = T - R(1);
   } else {
-    const R iT = rcp_rn(T);
     const R is2T = rsqrt_t(R(2) * T);
-    const R g0 = exp_t(-R(0.5) * u * u * iT) * is2T * R(0.56418958354775628695);  // N(0; u, T) = e^.. / sqrt(2 pi T)
-    R a = R(0.5) * (R(1) + erf_t<R>(u * is2T));
-    R b = u * a + T * g0;
-    m[0] = a;
-    m[1] = b;
+    const R x = u * is2T;
+    const R g0 = exp_t(-x * x) * is2T * R(0.56418958354775628695);  // N(0; u, T) = e^.. / sqrt(2 pi T)
+    a = R(0.5) * (R(1) + erf_t<R>(x));
+    b = u * a + T * g0, c = T;
+  }
+  m[0] = a;
+  m[1] = b;
 #pragma unroll
-    for (int l = 2; l < MAXN; ++l) {
-      const R x = u * b + R(l - 1) * T * a;
-      if (l <= N) m[l] = x;
-      a = b;
-      b = x;
-    }
+  for (int l = 2; l < MAXN; ++l) {
+    if (l > nmax) break;
+    const R x = (u * b + (kind == 0 ? R(1) : R(l - 1)) * c * a) * (kind == 0 ? R(1.0 / l) : R(1));
+    m[l] = x;
+    a = b;
+    b = x;
   }
 }
 
-// Force matrices of the channel split by the reflection of each axis (see
-// KArgs): with J the node permutation p -> -p, K0 J = -J K0 and K1 J = -J K1
-// (derivatives), Kt0 J = J Kt0 and Kt1 J = J Kt1 (derivatives of p f).  On the
-// even and odd parts e_k = f_k + f_Jk, o_k = f_k - f_Jk (k over the first half):
+// Coefficients of a packed contraction: single precision holds each duplicated into a pair, the
+// operand of a packed fma over (f', f''); double precision holds them once.
+template <typename real>
+struct CoefOf {
+  using type = float2;
+};
+template <>
+struct CoefOf<double> {
+  using type = double;
+};
+__device__ __forceinline__ float2 k_mul(float2 k, float2 x) { return p_mul(k, x); }
+__device__ __forceinline__ float2 k_fma(float2 k, float2 x, float2 a) { return p_fma(k, x, a); }
+__device__ __forceinline__ double2 k_mul(double k, double2 x) { return p_mul(p_set(k), x); }
+__device__ __forceinline__ double2 k_fma(double k, double2 x, double2 a) { return p_fma(p_set(k), x, a); }
+__device__ __forceinline__ float2 k_pair(float2 k) { return k; }
+__device__ __forceinline__ double2 k_pair(double k) { return p_set(k); }
+
+// Force matrices of the channel.  On each axis K = d/dp and Kt = d/dp (p .) of the projected
+// expansions satisfy
+//   Kt = K diag(p) + z v^T:
+// multiplying the expansion by p raises its degree by one, and its top term is a multiple of the
+// polynomial that vanishes on the nodes; on the full range its derivative is projected out
+// (z = 0), on the half range the projection of the jump at p = 0 leaves a rank-1 term.  So
+//   wa K f + wb Kt f = K ((wa + wb p) f) + wb (v . f) z,
+// one contraction in place of two.  K is split by the reflection of its axis (see KArgs): with J
+// the permutation p -> -p, K J = -J K, and with e = f + J f, o = f - J f (k over half the nodes)
 //   P[i][k] = (K[i][k] + K[i][Jk]) / 2,  M[i][k] = (K[i][k] - K[i][Jk]) / 2,
-//   odd K:  (K f)_i = P e + M o,  (K f)_Ji = M o - P e;
-//   even K: (K f)_i = P e + M o,  (K f)_Ji = P e - M o.
-// Every coefficient is duplicated into a pair, the operand of a packed fma over
-// (f', f''); the block travels as a kernel parameter, so the coefficients are
-// uniform constant-bank operands.
-template <int Q0, int Q1>
+//   (K f)_i = P e + M o,  (K f)_Ji = M o - P e;  z and v are odd (v_Jk = -v_k).
+// The block travels as a kernel parameter: the coefficients are uniform constant-bank operands.
+template <typename real, int Q0, int Q1>
 struct ChanKP {
+  using C = typename CoefOf<real>::type;
   static constexpr int H0 = Q0 / 2, H1 = Q1 / 2;
-  float2 P0[H0 * H0], M0[H0 * H0], Pt0[H0 * H0], Mt0[H0 * H0];  // K0, Kt0: [i][k]
-  float2 P1[H1 * H1], M1[H1 * H1], Pt1[H1 * H1], Mt1[H1 * H1];  // K1, Kt1: [j][k]
+  C P0[H0 * H0], M0[H0 * H0], p0[H0], v0[H0], z0[H0];
+  C P1[H1 * H1], M1[H1 * H1], p1[H1], v1[H1], z1[H1];
 };
 
-// lambda force task of column j of one cell on the CUDA cores: out[(i, j)] =
-// G_lxx (p^xi_j)^2 (K0 f)_i + G_lxl p^xi_j (Kt0 f)_i for both fields.
-template <int Q0, int Q1>
-__device__ __forceinline__ void force_lambda_cc(const ChanKP<Q0, Q1>& kp, const float* F, int j, float wa, float wb,
-                                                float* out) {
-  constexpr int H = Q0 / 2;
-  float2 e[H], o[H];
+// wa K f + wb Kt f of one line of 2 H nodes: node k of the first half at F + k sF, its mirror at
+// Fm + k sM; results likewise to O, Om.  Everything is in pairs (f', f'').
+template <typename real, int H, bool RANK1, typename C>
+__device__ __forceinline__ void force_line(const C* __restrict__ Pm, const C* __restrict__ Mm, const C* __restrict__ pk,
+                                           const C* __restrict__ vk, const C* __restrict__ zk, const real* F,
+                                           const real* Fm, int sF, int sM, real wa, real wb, real* O, real* Om, int sO,
+                                           int sOm) {
+  using P = pair_t<real>;
+  const P WA = p_set(wa), WB = p_set(wb), NWB = p_set(-wb);
+  P e[H], o[H], t = p_set(real(0));
 #pragma unroll
   for (int k = 0; k < H; ++k) {
-    const float2 f = p_load(F + 2 * (k * Q1 + j)), g = p_load(F + 2 * ((k + H) * Q1 + j));
-    e[k] = p_add(f, g);
-    o[k] = p_sub(f, g);
+    const P f = p_load(F + k * sF), g = p_load(Fm + k * sM);
+    // (wa + wb p) f at the node, (wa - wb p) g at its mirror
+    const P a = p_mul(k_fma(pk[k], WB, WA), f), b = k_fma(pk[k], NWB, WA);
+    e[k] = p_fma(b, g, a);
+    o[k] = p_sub(a, p_mul(b, g));
+    if constexpr (RANK1) t = k_fma(vk[k], p_sub(f, g), t);
   }
-  const float2 WA = p_set(wa), WB = p_set(wb);
+  if constexpr (RANK1) t = p_mul(t, WB);
 #pragma unroll
   for (int i = 0; i < H; ++i) {
-    float2 A = p_mul(kp.P0[i * H], e[0]), B = p_mul(kp.M0[i * H], o[0]);
-    float2 C = p_mul(kp.Pt0[i * H], e[0]), D = p_mul(kp.Mt0[i * H], o[0]);
+    P A, B = k_mul(Mm[i * H], o[0]);
+    if constexpr (RANK1) A = k_fma(Pm[i * H], e[0], k_mul(zk[i], t));
+    else A = k_mul(Pm[i * H], e[0]);
 #pragma unroll
     for (int k = 1; k < H; ++k) {
-      A = p_fma(kp.P0[i * H + k], e[k], A);
-      B = p_fma(kp.M0[i * H + k], o[k], B);
-      C = p_fma(kp.Pt0[i * H + k], e[k], C);
-      D = p_fma(kp.Mt0[i * H + k], o[k], D);
+      A = k_fma(Pm[i * H + k], e[k], A);
+      B = k_fma(Mm[i * H + k], o[k], B);
     }
-    // row i: wa (A + B) + wb (C + D); row Ji: wa (B - A) + wb (C - D)
-    p_store(out + 2 * (i * Q1 + j), p_fma(WA, p_add(A, B), p_mul(WB, p_add(C, D))));
-    p_store(out + 2 * ((i + H) * Q1 + j), p_fma(WA, p_sub(B, A), p_mul(WB, p_sub(C, D))));
+    p_store(O + i * sO, p_add(B, A));
+    p_store(Om + i * sOm, p_sub(B, A));
   }
 }
 
-// xi force task of row i of one cell on the CUDA cores: out[(i, j)] =
-// -G_lxx p^lambda_i (Kt1 f)_j - G_lxl (p^lambda_i)^2 (K1 f)_j for both fields
-// (wa = -G_lxx p^lambda_i, wb = -G_lxl (p^lambda_i)^2).
-template <int Q0, int Q1>
-__device__ __forceinline__ void force_xi_cc(const ChanKP<Q0, Q1>& kp, const float* F, int i, float wa, float wb,
-                                            float* out) {
-  constexpr int H = Q1 / 2;
-  float2 e[H], o[H];
+// Moments (Eq. macro_red), tau = Kn / (n T) (Eq. canalie_tau) and the normalised truncated
+// equilibrium (Sec. IV.D, reading 18) of four cells by one warp, eight lanes each: row holds the
+// lane's cell's V pairs, mv is 4 MAXN reals of scratch, rec its record.  The mass sum is
+// compensated in single precision.  Serial per cell, so it takes the whole warp's latency: four
+// cells at once cost what one does.
+template <typename real, int Q0, int Q1>
+__device__ __forceinline__ void channel_equilibrium(const ChanTables<real, Q0, Q1>& tb, const real* row, real* mv,
+                                                    real* rec, real ikn) {
+  constexpr bool F32 = sizeof(real) == 4;
+  constexpr int RP = Q0 / 8, FP = (Q0 + Q1 + 7) / 8;  // rows i and factors per lane
+  const int h = threadIdx.x & 7;
+  // sum over the lane's rows i = h + 8 r: the p^xi weights are uniform, p^lambda enters per row
+  real sn = 0, sr = 0, sp = 0, se = 0;
 #pragma unroll
-  for (int k = 0; k < H; ++k) {
-    const float2 f = p_load(F + 2 * (i * Q1 + k)), g = p_load(F + 2 * (i * Q1 + Q1 - 1 - k));
-    e[k] = p_add(f, g);
-    o[k] = p_sub(f, g);
+  for (int r = 0; r < RP; ++r) {
+    const real* f = row + 2 * (h + 8 * r) * Q1;
+    const real pr = tb.p0[h + 8 * r];
+    real n = 0;
+#pragma unroll
+    for (int j = 0; j < Q1; ++j) {
+      const pair_t<real> x = p_load(f + 2 * j);
+      const real pj = tb.p1[j], t = pj * x.x;
+      n += x.x;
+      sp += t;
+      se += pj * t + x.y;
+    }
+    sn += n;
+    sr += pr * n;
+    se += pr * pr * n;
   }
-  const float2 WA = p_set(wa), WB = p_set(wb);
+  auto sum8 = [](real x) -> real {
 #pragma unroll
-  for (int j = 0; j < H; ++j) {
-    float2 A = p_mul(kp.P1[j * H], e[0]), B = p_mul(kp.M1[j * H], o[0]);
-    float2 C = p_mul(kp.Pt1[j * H], e[0]), D = p_mul(kp.Mt1[j * H], o[0]);
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+  };
+  sr = sum8(sr), sp = sum8(sp), se = sum8(se);
+  real nn, th, tl;  // th + tl: the cell's mass that f_eq - R has to carry
+  if constexpr (F32) {
+    float e = 0.f, nh, nlo;
 #pragma unroll
-    for (int k = 1; k < H; ++k) {
-      A = p_fma(kp.P1[j * H + k], e[k], A);
-      B = p_fma(kp.M1[j * H + k], o[k], B);
-      C = p_fma(kp.Pt1[j * H + k], e[k], C);
-      D = p_fma(kp.Mt1[j * H + k], o[k], D);
+    for (int o = 4; o > 0; o >>= 1) {  // as half_sum_comp
+      const float s2 = __shfl_xor_sync(0xffffffffu, sn, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
+      float t, er;
+      two_sum(sn, s2, t, er);
+      sn = t;
+      e = __fadd_rn(__fadd_rn(e, e2), er);
     }
-    // K1 odd: (K1 f)_j = A + B, (K1 f)_Jj = B - A; Kt1 even: (Kt1 f)_j = C + D, (Kt1 f)_Jj = C - D
-    p_store(out + 2 * (i * Q1 + j), p_fma(WA, p_add(C, D), p_mul(WB, p_add(A, B))));
-    p_store(out + 2 * (i * Q1 + Q1 - 1 - j), p_fma(WA, p_sub(C, D), p_mul(WB, p_sub(B, A))));
-  }
-}
-
-// ------------------------------------------------------------------ tensor-core helpers
-__device__ __forceinline__ uint32_t tf32_rna(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
-// x = hi + lo with hi, lo TF32 (hi carries the top 11 significand bits, lo the next 11)
-__device__ __forceinline__ void tf32_split(float x, uint32_t& hi, uint32_t& lo) {
-  hi = tf32_rna(x);
-  lo = tf32_rna(__fsub_rn(x, __uint_as_float(hi)));
-}
-__device__ __forceinline__ void mma_tf32(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// Force subtask of one cell on the tensor cores (single precision): n-tile nn of
-// the lambda contraction (k < NN) or of the xi contraction (k >= NN), written to
-// fl_out (lambda part, pairs) or fx_out (xi part, scalars):
-//   lambda: G_lxx (p^xi)^2 K0 f + G_lxl p^xi Kt0 f,
-//   xi:    -G_lxx p^lambda Kt1 f - G_lxl (p^lambda)^2 K1 f    (Eq. canalie_boltz).
-template <int Q0, int Q1>
-__device__ __forceinline__ void force_subtask_tc(const ChanTables<float, Q0, Q1>& tb, const float* F, float glxx,
-                                                 float glxl, int k, int lane, float* fl_out, float* fx_out) {
-  using S = ChanShape<Q0, Q1>;
-  const int g = lane >> 2, tq = lane & 3;
-  float acc[S::MT][4];
-#pragma unroll
-  for (int t = 0; t < S::MT; ++t) acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.0f;
-  if (k < S::NN) {
-    const int nn = k;
-#pragma unroll
-    for (int kk = 0; kk < S::KKL; ++kk) {
-      uint32_t bh0, bl0, bh1, bl1;
-      tf32_split(F[(8 * kk + tq) * (2 * Q1) + 8 * nn + g], bh0, bl0);
-      tf32_split(F[(8 * kk + tq + 4) * (2 * Q1) + 8 * nn + g], bh1, bl1);
-#pragma unroll
-      for (int t = 0; t < S::MT; ++t) {
-        const uint4 h4 = *reinterpret_cast<const uint4*>(tb.fl[t][kk][0][lane]);
-        const uint4 l4 = *reinterpret_cast<const uint4*>(tb.fl[t][kk][1][lane]);
-        const uint32_t ah[4] = {h4.x, h4.y, h4.z, h4.w}, alo[4] = {l4.x, l4.y, l4.z, l4.w};
-        mma_tf32(acc[t], alo, bh0, bh1);
-        mma_tf32(acc[t], ah, bl0, bl1);
-        mma_tf32(acc[t], ah, bh0, bh1);
-      }
-    }
-    const int j = 4 * nn + tq;
-    const float px = tb.p1[j];
-    const float wa = glxx * px * px, wb = glxl * px;
-#pragma unroll
-    for (int t = 0; t < S::MT; ++t) {
-      const int i = 8 * t + g;
-      float2 o;
-      o.x = fmaf(wa, acc[t][0], wb * acc[t][2]);
-      o.y = fmaf(wa, acc[t][1], wb * acc[t][3]);
-      *reinterpret_cast<float2*>(fl_out + 2 * (i * Q1 + j)) = o;
-    }
+    two_sum(sn, tb.ref_hi[0], nh, nlo);
+    nn = nh + (nlo + (e + tb.ref_lo[0]));
+    two_sum(sn, tb.ref_sum[0], th, tl);
+    tl = tl + (e + tb.ref_sum[1]);
   } else {
-    const int nn = k - S::NN;
-    const int d = g & 1;
-#pragma unroll
-    for (int kk = 0; kk < S::KKX; ++kk) {
-      const uint2 bh = *reinterpret_cast<const uint2*>(tb.fx[kk][nn][0][lane]);
-      const uint2 bl = *reinterpret_cast<const uint2*>(tb.fx[kk][nn][1][lane]);
-      const int ja = 8 * kk + tq, jb = ja + 4;
-#pragma unroll
-      for (int t = 0; t < S::MT; ++t) {
-        const int ia = 8 * t + (g >> 1), ib = ia + 4;
-        const float x0 = ja < Q1 ? F[ia * (2 * Q1) + 2 * ja + d] : 0.0f;
-        const float x1 = ja < Q1 ? F[ib * (2 * Q1) + 2 * ja + d] : 0.0f;
-        const float x2 = jb < Q1 ? F[ia * (2 * Q1) + 2 * jb + d] : 0.0f;
-        const float x3 = jb < Q1 ? F[ib * (2 * Q1) + 2 * jb + d] : 0.0f;
-        uint32_t ah[4], alo[4];
-        tf32_split(x0, ah[0], alo[0]);
-        tf32_split(x1, ah[1], alo[1]);
-        tf32_split(x2, ah[2], alo[2]);
-        tf32_split(x3, ah[3], alo[3]);
-        mma_tf32(acc[t], alo, bh.x, bh.y);
-        mma_tf32(acc[t], ah, bl.x, bl.y);
-        mma_tf32(acc[t], ah, bh.x, bh.y);
-      }
-    }
-    const int j = 4 * nn + tq;
-#pragma unroll
-    for (int t = 0; t < S::MT; ++t) {
-      const int ia = 8 * t + (g >> 1), ib = ia + 4;
-      const float pa = tb.p0[ia], pb = tb.p0[ib];
-      fx_out[2 * (ia * Q1 + j) + d] = -fmaf(glxx * pa, acc[t][1], glxl * pa * pa * acc[t][0]);
-      fx_out[2 * (ib * Q1 + j) + d] = -fmaf(glxx * pb, acc[t][3], glxl * pb * pb * acc[t][2]);
-    }
+    nn = sum8(sn) + tb.ref_hi[0];
+    th = nn, tl = 0.0;
   }
-}
-
-// Geometry of one cell into registers with vector loads (12 reals).
-template <typename real>
-__device__ __forceinline__ void load_geo(const ChanCell<real>* g, real* o) {
-  if constexpr (sizeof(real) == 4) {
-    const float4* q = reinterpret_cast<const float4*>(g);
+  const real inv = rcp_rn(nn);
+  const real u0 = (sr + (tb.ref_hi[1] + tb.ref_lo[1])) * inv, u1 = (sp + (tb.ref_hi[2] + tb.ref_lo[2])) * inv;
+  const real T = ((se + (tb.ref_hi[3] + tb.ref_lo[3])) * inv - (u0 * u0 + u1 * u1)) * (real(1) / real(3));
+  if (h < 4) {  // moment vectors [axis][side]; axis 0 is half range
+    const real u = (h & 2 ? u1 : u0) * (h & 1 ? real(-1) : real(1));
+    eq_moments_fast<real>(h & 2 ? tb.kind1 : 1, tb.nmax, u, T, mv + h * MAXN);
+  }
+  __syncwarp();
+  real g[FP], a0 = real(0), a1 = real(0);
+  const real* m[FP];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float4 x = q[k];
-      o[4 * k] = x.x, o[4 * k + 1] = x.y, o[4 * k + 2] = x.z, o[4 * k + 3] = x.w;
-    }
+  for (int q = 0; q < FP; ++q) {
+    const int k = h + 8 * q;  // axis 0 for q < RP
+    g[q] = real(0);
+    m[q] = mv + (q < RP ? (k >= Q0 / 2 ? 1 : 0) : 2 + (tb.kind1 == 1 && k - Q0 >= Q1 / 2 ? 1 : 0)) * MAXN;
+  }
+#pragma unroll 1
+  for (int s = 0; s <= tb.nmax; ++s)
+#pragma unroll
+    for (int q = 0; q < FP; ++q)
+      if (h + 8 * q < Q0 + Q1) g[q] += tb.tab[s * (Q0 + Q1) + h + 8 * q] * m[q][s];
+#pragma unroll
+  for (int q = 0; q < FP; ++q) {
+    if (q < RP) g[q] *= nn, a0 += g[q];
+    else a1 += g[q];
+  }
+  a0 = sum8(a0), a1 = sum8(a1);
+  // g0 <- g0 target / (sum g0 sum g1); single precision: g0 (1 - delta), the target in float-float
+  real scale;
+  if constexpr (F32) {
+    const float Ah = a0 * a1, Al = fmaf(a0, a1, -Ah);
+    scale = (__fsub_rn(Ah, th) + (Al - tl)) * rcp_rn(Ah);
   } else {
-    const double2* q = reinterpret_cast<const double2*>(g);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const double2 x = q[k];
-      o[2 * k] = x.x, o[2 * k + 1] = x.y;
-    }
+    scale = th / (a0 * a1);
   }
+#pragma unroll
+  for (int q = 0; q < FP; ++q) {
+    real val = g[q];
+    if (q < RP) {
+      if constexpr (F32) val = fmaf(-val, scale, val);
+      else val *= scale;
+    }
+    if (h + 8 * q < Q0 + Q1) p_store(rec + 2 * (h + 8 * q), p_make(val, val));
+  }
+  if (h == 0) {
+    const real nit = -(nn * T * ikn);
+    p_store(rec + 2 * (Q0 + Q1), p_make(real(1), T));
+    p_store(rec + 2 * (Q0 + Q1) + 2, p_make(nit, nit));
+    p_store(rec + 2 * (Q0 + Q1) + 4, p_make(u1, real(0)));
+  }
+  __syncwarp();
 }
-enum { G_AM = 0, G_AP, G_BM, G_BP, G_CM, G_CP, G_IDL, G_IDX, G_GLXL, G_GLXX };
 
 // ------------------------------------------------------------------ the stage kernel
-// Device cell (s, p) of the channel is s * n_xi + p (xi fastest), so the cells of a
-// strip's row and its xi-halo are one contiguous bulk copy.
+// Device cell (s, p) of the channel is s * n_xi + p (xi fastest).
 //
-// TC selects the single-precision force contraction: true, the tensor cores
-// (mma.sync TF32, three products per tile) on the column-group warps; false,
-// packed FP32x2 fmas with the split matrices of kp on the extra warps.  The
-// double-precision kernel contracts in FP64 on the column-group threads.
+// HX: axis 1 is half range (its mirror node is k + Q1/2 and its Kt has the rank-1 term).
 //
 // CLB runs the Cartesian-split formulation (Sec. VII.G, Eq. canalie_coord_beq_cons) on the
 // same march: momenta (p^x, p^y) on the model's axes, no force term, fluxes of F = D + R, and
 // the geometry record read as V^lambda = am p^x - glxl p^y at s - 1/2 and ap p^x - glxx p^y at
 // s + 1/2 (a = 1 / (1 + phi), glxl / glxx = a lambda phi' at the interfaces), V^xi = b p^y
 // (c = 0).  The lambda upwind side and the wall's incoming half-plane (Eq. canalie_coord_nw)
-// then depend on the column and the interface.
-template <typename real, int Q0, int Q1, int TP, bool TC, bool CLB = false>
-__global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, TP>::NT, 1)
-    channel_stage_kernel(const __grid_constant__ ChanArgs<real> a, const __grid_constant__ ChanKP<Q0, Q1> kp) {
+// then depend on the column and the interface: the lambda window holds the six cells around an
+// interface and the walk's terms are formed per interface from the five of the upwind side.
+template <typename real, int Q0, int Q1, bool CLB, bool HX>
+__global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0, Q1>::min_ctas)
+    channel_stage_kernel(const __grid_constant__ ChanArgs<real> a, const __grid_constant__ ChanKP<real, Q0, Q1> kp) {
   using S = ChanShape<Q0, Q1>;
-  using L = ChanSmem<real, Q0, Q1, TP>;
+  using L = ChanSmem<real, Q0, Q1>;
   using Tab = ChanTables<real, Q0, Q1>;
   using P = pair_t<real>;
-  constexpr int V = S::V, ROW = S::ROW, NWC = S::NWC, EQW = S::EQW;
-  constexpr int NMAIN = TP * V;    // threads of the column groups
-  constexpr int NMW = NMAIN / 32;  // their warps
-  constexpr int PD = L::PD, NRING = L::NRING, NB = L::NB, RC = L::RC;
-  constexpr bool F32 = L::F32;
+  constexpr int V = S::V, ROW = S::ROW, EQW = S::EQW, TP = S::TP, NW = S::NW;
+  constexpr int NRING = L::NRING, RC = L::RC, CS = L::CS, XS = L::XS;
   extern __shared__ __align__(128) unsigned char smem[];
-
-  constexpr int NSYNC = L::NSYNC;  // threads of the named barrier the step phases use
-  const int tid = threadIdx.x, lane = tid & 31;
-  const bool is_main = tid < NMAIN;
-  const bool is_eqw = tid >= NSYNC;       // the two equilibrium warps
-  const int qw = is_eqw ? (tid - NSYNC) >> 5 : -1;
-  const int c = is_main ? tid / V : TP;  // column of a main thread; TP marks the extra group
-  const int v = is_main ? tid - c * V : (is_eqw ? lane : tid - NMAIN);
+  const int v = threadIdx.x, lane = v & 31, warp = v >> 5;
   const int i = v / Q1, j = v - i * Q1;
-  const int wc = v >> 5;                             // warp within the group
-  const int mw = is_main ? tid >> 5 : -1;            // main warp index
-  const int ew = is_main ? -1 : (tid - NMAIN) >> 5;  // extra warp index
 
   const int nl = a.nl, nx = a.nx;
   const int nstrips = nx / TP;
@@ -455,211 +393,145 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, TP>::NT, 1)
   const int p0 = strip * TP;
   const int sA = seg * a.seglen, sB = min(sA + a.seglen, nl);
   const bool inlet = p0 == 0, outlet = p0 + TP == nx;
-  const bool top = sB == nl;
-  const bool need_fl = a.ca != real(0);
+  const bool need_fl = a.ca.x != real(0);
   const int rlast = min(sB + 2, nl - 1);  // last row a segment reads
   const int pa = max(p0 - 3, 0), pb = min(p0 + TP + 3, nx);  // xi cells of a ring row in memory
 
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::bar_off);  // NB step groups, then the prologue
-  uint64_t* pready = bar + NB + 1;     // [NPR] moment partials of row r in slot r % NPR written
-  uint64_t* eready = pready + L::NPR;  // [NEQ] equilibrium record of row r in slot r % NEQ written
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::bar_off);  // [NRING]: the row of the slot has landed
   const Tab& tb = *reinterpret_cast<const Tab*>(smem + L::tab_off);
-  real* ring = reinterpret_cast<real*>(smem + L::ring_off);                      // [NRING][RC][ROW]
+  real* ring = reinterpret_cast<real*>(smem + L::ring_off);                      // [NRING][RC][CS]
   ChanCell<real>* gring = reinterpret_cast<ChanCell<real>*>(smem + L::geo_off);  // [NRING][TP]
-  P* xif = reinterpret_cast<P*>(smem + L::xif_off);                              // [TP+1][V]
-  real* lbl = reinterpret_cast<real*>(smem + L::lbl_off);                        // [TP][ROW] (single precision)
-  real* lbx = reinterpret_cast<real*>(smem + L::lbx_off);                        // [TP][ROW]
-  real* eqr = reinterpret_cast<real*>(smem + L::eq_off);                         // [4][TP][EQW]
-  real* resr = reinterpret_cast<real*>(smem + L::res_off);                       // [4][2][Q1]
-  real* resn = reinterpret_cast<real*>(smem + L::resn_off);                      // [4][2] inflow densities
+  real* lbl = reinterpret_cast<real*>(smem + L::lbl_off);                        // [2][TP][CS]: lambda force
+  real* lbx = reinterpret_cast<real*>(smem + L::lbx_off);                        // [2][TP][Q0][XS]: xi force
+  real* eqr = reinterpret_cast<real*>(smem + L::eq_off);                         // [NEQ][TP][EQW]
+  real* resr = reinterpret_cast<real*>(smem + L::res_off);                       // [NRES][2][Q1]
+  real* resn = reinterpret_cast<real*>(smem + L::resn_off);                      // [NRES][2] inflow densities
   real* mvs = reinterpret_cast<real*>(smem + L::mvs_off);                        // [TP+2][4][MAXN]
-  real* red = reinterpret_cast<real*>(smem + L::red_off);                        // [NPR][TP][NWC][4]
-  real* wred = reinterpret_cast<real*>(smem + L::wred_off);                      // [TP][NWC]
+  real* wred = reinterpret_cast<real*>(smem + L::wred_off);                      // [2][TP][NW]
   double* nwv = reinterpret_cast<double*>(smem + L::nwv_off);                    // [TP]
 
   auto dcell = [&](int s, int p) -> size_t { return size_t(s) * nx + p; };
-  // cell cc in [-3, TP + 3) of the ring row in slot k
-  auto krow = [&](int k, int cc) -> real* { return ring + size_t(k * RC + cc + 3) * ROW; };
-  auto row_bytes = [&]() -> unsigned { return unsigned((pb - pa) * L::rowb + TP * sizeof(ChanCell<real>)); };
-  auto row_issue = [&](int r, uint64_t* b) {  // row r with its halo, and its geometry
-    const int k = r % NRING;
-    bulk_g2s(krow(k, pa - p0), a.Fprev + dcell(r, pa) * ROW, unsigned((pb - pa) * L::rowb), b);
-    bulk_g2s(gring + k * TP, a.geo + dcell(r, p0), unsigned(TP * sizeof(ChanCell<real>)), b);
+  auto slot = [&](int r) -> int { return (r - sA) % NRING; };
+  // cell cc in [-3, TP + 3) of ring slot k
+  auto cell = [&](int k, int cc) -> real* { return ring + (k * RC + cc + 3) * CS; };
+  int issued = -1;  // warp 0: the last row whose copies it has started
+  // row r with its halo (one bulk copy per cell: cells are padded) and its geometry, by warp 0
+  auto row_issue = [&](int r) {
+    const int k = slot(r), n = pb - pa;
+    issued = r;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (lane == 0) mbar_expect_tx(bar + k, unsigned(n * L::rowb + TP * sizeof(ChanCell<real>)));
+    __syncwarp();
+    if (lane < n) bulk_g2s(cell(k, pa - p0 + lane), a.Fprev + dcell(r, pa + lane) * ROW, unsigned(L::rowb), bar + k);
+    if (lane == n) bulk_g2s(gring + k * TP, a.geo + dcell(r, p0), unsigned(TP * sizeof(ChanCell<real>)), bar + k);
   };
+  auto row_wait = [&](int r) -> bool { return mbar_wait(bar + slot(r), unsigned((r - sA) / NRING) & 1u, a.max_polls); };
 
-  // ---- prologue: tables and rows sA .. sA+2+PD
-  if (tid == 0) {
-    for (int b = 0; b <= NB; ++b) mbar_init(bar + b, 1);
-    for (int k = 0; k < L::NPR; ++k) mbar_init(pready + k, NMW);
-    for (int k = 0; k < L::NEQ; ++k) mbar_init(eready + k, 2);
+  // ---- prologue: tables and rows sA .. sA+3
+  if (v == 0) {
+    for (int k = 0; k < NRING; ++k) mbar_init(bar + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
-  const int rtop = min(sA + 2 + PD, rlast);
-  if (tid == NMAIN) {  // one arrival with every byte of the prologue, then the copies
-    const unsigned total = unsigned(sizeof(Tab)) + unsigned(rtop - sA + 1) * row_bytes();
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(bar + NB, total);
-    bulk_g2s(smem + L::tab_off, a.tables, unsigned(sizeof(Tab)), bar + NB);
-    for (int r = sA; r <= rtop; ++r) row_issue(r, bar + NB);
-  }
-  P W0, W1, W2, W3, W4, W5;  // F(s-3 .. s+2) before the push of step s
-  W0 = W1 = W2 = p_set(real(0));
-  if (is_main && sA > 0) {  // window rows below the segment (each thread its own populations)
-    const real* base = a.Fprev + 2 * v;
-    W0 = p_load(base + dcell(sA - 3, p0 + c) * ROW);
-    W1 = p_load(base + dcell(sA - 2, p0 + c) * ROW);
-    W2 = p_load(base + dcell(sA - 1, p0 + c) * ROW);
-  }
   {
-    bool ok = true;
-    if (tid == 0) ok = mbar_wait(bar + NB, 0, a.max_polls);
-    ok = __syncthreads_and(ok);
-    if (!ok) {
-      if (tid == 0) {
-        atomicOr(a.err, ERR_TIMEOUT);
-        mbar_wait(bar + NB, 0, a.max_polls);
-      }
-      __syncthreads();
-      return;
-    }
+    const uint4* src = reinterpret_cast<const uint4*>(a.tables);
+    uint4* dst = reinterpret_cast<uint4*>(smem + L::tab_off);
+    for (int x = v; x < int(sizeof(Tab) / 16); x += V) dst[x] = src[x];
   }
-  // per-thread constants
+  __syncthreads();
+  if (warp == 0)
+    for (int r = sA; r <= min(sA + 3, rlast); ++r) row_issue(r);
+
+  // per-thread constants; the walks' values are scaled by sc, their results by isc
+  const real isc = tb.isc0[i] * tb.isc1[j];
+  const P SC = p_set(tb.sc0[i] * tb.sc1[j]);
   const real pl = tb.p0[i], px = tb.p1[j];
-  const real sc = tb.iw0[i] * tb.iw1[j];
+  const real plI = pl * isc, pxI = px * isc;
+  const P PLI = p_set(plI);
   const real Rij = tb.w0[i] * tb.w1[j];
+  const P NR = p_set(-Rij);
   const bool lpos = pl >= real(0);
+  const int off = lpos ? 0 : 1;  // the lambda window of step s is centred on row s + off
   const real T0 = a.T0;
+  WenoSide<real> wl;
+  wl.set(CLB || lpos);  // (the Cartesian split's windows are in upwind order)
 
-  // moments of row r (main threads): per-warp partial sums of the deviation
-  auto moment_partials = [&](P f, int r) {
-    const real f1 = f.x, f2 = f.y;
-    const real sn = f1, srr = pl * f1, spp = px * f1, se = (pl * pl + px * px) * f1 + f2;
-    const bool h16 = lane & 16, h8 = lane & 8;
-    real k0 = h16 ? spp : sn, k1 = h16 ? se : srr;
-    const real t0 = h16 ? sn : spp, t1 = h16 ? srr : se;
-    k0 += __shfl_xor_sync(0xffffffffu, t0, 16);
-    k1 += __shfl_xor_sync(0xffffffffu, t1, 16);
-    real kq = h8 ? k1 : k0;
-    kq += __shfl_xor_sync(0xffffffffu, h8 ? k0 : k1, 8);
-    kq += __shfl_xor_sync(0xffffffffu, kq, 4);
-    kq += __shfl_xor_sync(0xffffffffu, kq, 2);
-    kq += __shfl_xor_sync(0xffffffffu, kq, 1);
-    // lanes 0, 8, 16, 24: n, rho u0, rho u1, energy
-    if ((lane & 7) == 0) red[(((r % L::NPR) * TP + c) * NWC + wc) * 4 + (lane >> 3)] = kq;
+  bool good = true;  // every wait of this thread so far ended in time
+  // a wait ran out: let the copies in flight land (bounded), then leave together
+  auto give_up = [&]() {
+    if (v == 0) {
+      atomicOr(a.err, ERR_TIMEOUT);
+      for (int r = max(sA, issued - NRING + 1); r <= issued; ++r) row_wait(r);
+    }
+    __syncthreads();
   };
+  for (int r = sA; r <= min(sA + 3, rlast); ++r) good = row_wait(r) && good;
+  if (!__syncthreads_and(good)) {
+    give_up();
+    return;
+  }
 
-  // equilibrium record of cell cc of row r (one extra warp): n, u, T, tau and the
-  // factors n g0_i, g1_j normalised so that sum_ij n g0_i g1_j = n (reading 18)
-  auto eq_job = [&](int r, int cc) {
-    real* mv = mvs + cc * 4 * MAXN;
-    const real* rp = red + ((r % L::NPR) * TP + cc) * NWC * 4;
-    // cross-warp sums of the partials plus the sums of R; n compensated (float-float)
-    // on the single-precision path
-    real q[4], nlo = real(0);
-    {
-      real sn = real(0), e = real(0);
-#pragma unroll
-      for (int w = 0; w < NWC; ++w) {
-        const real x = rp[w * 4];
-        if constexpr (F32) {
-          float t, er;
-          two_sum(sn, x, t, er);
-          sn = t;
-          e += er;
-        } else {
-          sn += x;
+  // ---- the roles of the rows ahead.  With at least six warps: warps 0 and 1 contract along
+  // lambda, 2 and 3 along xi, 4 takes the equilibria, 5 the inflow factors; fewer take all in turn.
+  constexpr bool SPLIT = NW >= 6;
+  auto force_row = [&](int r) {
+    if constexpr (!CLB) {
+      const int k = slot(r);
+      real* ol = lbl + (r & 1) * TP * CS;
+      real* ox = lbx + (r & 1) * TP * Q0 * XS;
+      // Eq. (canalie_boltz): G_lxx (p^xi)^2 K0 f + G_lxl p^xi Kt0 f along lambda,
+      // -G_lxl (p^lambda)^2 K1 f - G_lxx p^lambda Kt1 f along xi
+      if (!SPLIT || warp < 2)
+        for (int t = v; t < TP * Q1; t += SPLIT ? 64 : V) {
+          const int cc = t / Q1, jj = t - cc * Q1;
+          const ChanCell<real>& g = gring[k * TP + cc];
+          const real pj = tb.p1[jj];
+          const real* F = cell(k, cc) + 2 * jj;
+          real* O = ol + cc * CS + 2 * jj;
+          force_line<real, Q0 / 2, true>(kp.P0, kp.M0, kp.p0, kp.v0, kp.z0, F, F + Q0 * Q1, 2 * Q1, 2 * Q1,
+                                         g.glxx * pj * pj, g.glxl * pj, O, O + Q0 * Q1, 2 * Q1, 2 * Q1);
         }
-      }
-      if constexpr (F32) {
-        float t, er;
-        two_sum(sn, tb.ref_hi[0], t, er);
-        q[0] = t;
-        nlo = er + e + tb.ref_lo[0];
-      } else {
-        q[0] = sn + tb.ref_hi[0];
-      }
+      if (!SPLIT || (warp & ~1) == 2)
+        for (int t = SPLIT ? v - 64 : v; t < TP * Q0; t += SPLIT ? 64 : V) {
+          const int cc = t / Q0, ii = t - cc * Q0;
+          const ChanCell<real>& g = gring[k * TP + cc];
+          const real pi = tb.p0[ii];
+          const real* F = cell(k, cc) + 2 * ii * Q1;
+          real* O = ox + (cc * Q0 + ii) * XS;
+          constexpr int M = HX ? Q1 : 2 * (Q1 - 1), sM = HX ? 2 : -2;  // mirror of node 0, step
+          force_line<real, Q1 / 2, HX>(kp.P1, kp.M1, kp.p1, kp.v1, kp.z1, F, F + M, 2, sM, -g.glxl * pi * pi,
+                                       -g.glxx * pi, O, O + M, 2, sM);
+        }
     }
-#pragma unroll
-    for (int k = 1; k < 4; ++k) {
-      real sk = real(0);
-#pragma unroll
-      for (int w = 0; w < NWC; ++w) sk += rp[w * 4 + k];
-      q[k] = sk + (tb.ref_hi[k] + tb.ref_lo[k]);
-    }
-    const real nn = q[0] + nlo;
-    const real inn = rcp_rn(nn);
-    const real u0 = q[1] * inn, u1 = q[2] * inn;
-    const real T = (q[3] * inn - (u0 * u0 + u1 * u1)) * (real(1) / real(3));
-    if (lane < 4) {
-      const int ax = lane >> 1, side = lane & 1;
-      const real u = (ax ? u1 : u0) * (side ? real(-1) : real(1));
-      eq_moments_fast<real>(ax ? tb.kind1 : tb.kind0, ax ? tb.N1 : tb.N0, u, T, mv + lane * MAXN);
-    }
-    __syncwarp();
-    real g = real(0);
-    if (lane < Q0) {
-      const real* m = mv + ((tb.kind0 == 1 && tb.p0[lane] < real(0)) ? 1 : 0) * MAXN;
-      for (int s = 0; s <= tb.N0; ++s) g += tb.tab0[lane * MAXN + s] * m[s];
-      g *= nn;
-    } else if (lane < Q0 + Q1) {
-      const int jj = lane - Q0;
-      const real* m = mv + (2 + ((tb.kind1 == 1 && tb.p1[jj] < real(0)) ? 1 : 0)) * MAXN;
-      for (int s = 0; s <= tb.N1; ++s) g += tb.tab1[jj * MAXN + s] * m[s];
-    }
-    real s0 = lane < Q0 ? g : real(0), s1 = (lane >= Q0 && lane < Q0 + Q1) ? g : real(0);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-    }
-    // scale = n / (s0 s1), n in float-float on the single-precision path
-    const real iden = rcp_rn(s0 * s1);
-    const real scl = q[0] * iden + nlo * iden;
-    real val = g;
-    if (lane < Q0) val = g * scl;
-    else if (lane == Q0 + Q1) val = T;
-    else if (lane == Q0 + Q1 + 1) val = nn * T * a.ikn;  // 1/tau, tau = Kn / (n T) (Eq. canalie_tau)
-    else if (lane == Q0 + Q1 + 2) val = u1;
-    if (lane < EQW) eqr[((r & (L::NEQ - 1)) * TP + cc) * EQW + lane] = val;
-    __syncwarp();
   };
-
+  auto eq_row = [&](int r) {
+    if (warp != (SPLIT ? 4 : 0)) return;
+    const int cc = lane >> 3;
+    channel_equilibrium<real, Q0, Q1>(tb, cell(slot(r), cc), mvs + cc * 4 * MAXN,
+                                      eqr + ((r & (L::NEQ - 1)) * TP + cc) * EQW, a.ikn);
+  };
   // inflow factors g_xi(u^xi, T0) of row r at one end: reservoirs, u^xi of the adjacent
-  // cell from its moment partials; flow-rate ends, u^xi = Q_s and the density n_s of
-  // Eq. (canalie_inlet_s)
+  // cell; flow-rate ends, u^xi = Q_s and the density n_s of Eq. (canalie_inlet_s)
   auto res_job = [&](int r, int end) {
-    const int cc = end == 0 ? 0 : TP - 1;
-    real ures;
-    if (a.flow) {
-      ures = a.qflow[(2 * end) * nl + r];
-    } else {
-      const real* rp = red + ((r % L::NPR) * TP + cc) * NWC * 4;
-      real sn = real(0), sp = real(0);
-#pragma unroll
-      for (int w = 0; w < NWC; ++w) sn += rp[w * 4], sp += rp[w * 4 + 2];
-      ures = (sp + (tb.ref_hi[2] + tb.ref_lo[2])) * rcp_rn(sn + (tb.ref_hi[0] + tb.ref_lo[0]));
-    }
+    const int cc = end == 0 ? 0 : TP - 1, rs = r & (L::NRES - 1);
+    const real ures = a.flow ? a.qflow[(2 * end) * nl + r] : eqr[((r & (L::NEQ - 1)) * TP + cc) * EQW + 2 * (Q0 + Q1) + 4];
     real* mv = mvs + (TP + end) * 4 * MAXN;
-    if (lane < 2) eq_moments_fast<real>(tb.kind1, tb.N1, lane ? -ures : ures, T0, mv + lane * MAXN);
+    if (lane < 2) eq_moments_fast<real>(tb.kind1, tb.nmax, lane ? -ures : ures, T0, mv + lane * MAXN);
     __syncwarp();
     if (lane < Q1) {
-      const real* m = mv + ((tb.kind1 == 1 && tb.p1[lane] < real(0)) ? 1 : 0) * MAXN;
+      const real* m = mv + ((tb.kind1 == 1 && lane >= Q1 / 2) ? 1 : 0) * MAXN;
       real g = real(0);
-      for (int s = 0; s <= tb.N1; ++s) g += tb.tab1[lane * MAXN + s] * m[s];
-      resr[((r & (L::NEQ - 1)) * 2 + end) * Q1 + lane] = g;
+      for (int s = 0; s <= tb.nmax; ++s) g += tb.tab[s * (Q0 + Q1) + Q0 + lane] * m[s];
+      resr[(rs * 2 + end) * Q1 + lane] = g;
     }
     __syncwarp();
     if (a.flow) {
       // n_s sum_{entering} V f'_eq(1, (0, Q_s), T0) + sum_{leaving} V f'_adjacent = (1 + phi) Q_s,
-      // V = b p^xi - c p^lambda of the end interface (the decision of end_ghost);
-      // the adjacent cell is row r of the ring (its slot is refilled only after this row's
-      // record is waited for), FP64 sums as for n_w
-      const int k = r % NRING;
+      // V = b p^xi - c p^lambda of the end interface (the decision of fill_ghosts); FP64 sums as for n_w
+      const int k = slot(r);
       const ChanCell<real>& gk = gring[k * TP + cc];
       const real bb = end == 0 ? gk.bm : gk.bp, cq = end == 0 ? gk.cm : gk.cp;
-      const real* Fa = krow(k, cc);
-      const real* gr = resr + ((r & (L::NEQ - 1)) * 2 + end) * Q1;
+      const real* Fa = cell(k, cc);
+      const real* gr = resr + (rs * 2 + end) * Q1;
       double lv = 0.0, en = 0.0;
       for (int vv = lane; vv < V; vv += 32) {
         const int ii = vv / Q1, jj = vv - ii * Q1;
@@ -673,365 +545,315 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, TP>::NT, 1)
         lv += __shfl_xor_sync(0xffffffffu, lv, o);
         en += __shfl_xor_sync(0xffffffffu, en, o);
       }
-      if (lane == 0) resn[(r & (L::NEQ - 1)) * 2 + end] = real((double(a.qflow[(2 * end + 1) * nl + r]) - lv) / en);
+      if (lane == 0) resn[rs * 2 + end] = real((double(a.qflow[(2 * end + 1) * nl + r]) - lv) / en);
       __syncwarp();
     }
   };
-  auto res_jobs = [&](int r) {  // equilibrium warps: both ends where the strip has one
+  auto res_row = [&](int r) {
+    if (!(inlet || outlet) || warp != (SPLIT ? 5 : 0)) return;
+#pragma unroll 1
     for (int end = 0; end < 2; ++end)
-      if ((end == 0 ? inlet : outlet) && qw == end) res_job(r, end);
+      if (end == 0 ? inlet : outlet) res_job(r, end);
   };
-
-  // xi-halo value of velocity (ii, jj) of row r beyond strip end `end` (the inlet / outlet
-  // reservoirs): populations entering the domain see f_eq(n_res, (0, u^xi), T0) - R, the
-  // others the adjacent cell (zeroth order).  Every thread whose stencil reaches past an
-  // end evaluates it itself; the bulk copy leaves those cells out.
-  auto end_ghost = [&](int r, int end, int ii, int jj) -> P {
-    const int k = r % NRING, ce = end == 0 ? 0 : TP - 1;
-    real gm[12];
-    load_geo(gring + k * TP + ce, gm);
-    const real pli = tb.p0[ii], pxj = tb.p1[jj];
-    const real Vx = end == 0 ? gm[G_BM] * pxj - gm[G_CM] * pli : gm[G_BP] * pxj - gm[G_CP] * pli;
-    const bool inflow = end == 0 ? (Vx > real(0)) : (Vx < real(0));
-    if (inflow) {
-      const int e8 = (r & (L::NEQ - 1)) * 2 + end;
-      const real nres = a.flow ? resn[e8] : (end == 0 ? a.n_in : a.n_out);
-      const real e = nres * tb.gw0[ii] * resr[e8 * Q1 + jj];
-      const real R = tb.w0[ii] * tb.w1[jj];
-      return p_make(e - R, e * T0 - R);
-    }
-    return p_load(krow(k, ce) + 2 * (ii * Q1 + jj));
-  };
-  // the upwind-ordered five-cell stencil of xi interface cl - 1/2 of ring slot k (cells
-  // cl-3 .. cl+1 when up, cl+2 .. cl-2 otherwise), with the reservoir ghosts at the ends
-  auto xi_stencil = [&](int r, int k, int cl, bool up, int vv, P* h) {
-    const int ii = vv / Q1, jj = vv - ii * Q1;
-    const int c0 = up ? cl - 3 : cl + 2, sd = up ? 1 : -1;
-    if (!((inlet && cl < 3) || (outlet && cl > TP - 3))) {  // no end within reach (warp-uniform)
+  // reservoir halo cells of row r past an end strip (the bulk copy leaves them out): populations
+  // entering the domain see f_eq(n_res, (0, u^xi), T0) - R, the others the adjacent cell (zeroth order)
+  auto fill_ghosts = [&](int r) {
+    const int k = slot(r), rs = r & (L::NRES - 1);
 #pragma unroll
-      for (int q = 0; q < 5; ++q) h[q] = p_load(krow(k, c0 + q * sd) + 2 * vv);
-      return;
+    for (int end = 0; end < 2; ++end) {
+      if (!(end == 0 ? inlet : outlet)) continue;
+      const int ce = end == 0 ? 0 : TP - 1;
+      const ChanCell<real>& g = gring[k * TP + ce];
+      const real Vx = end == 0 ? g.bm * px - g.cm * pl : g.bp * px - g.cp * pl;
+      P q;
+      if (end == 0 ? (Vx > real(0)) : (Vx < real(0))) {
+        const real nres = a.flow ? resn[rs * 2 + end] : (end == 0 ? a.n_in : a.n_out);
+        const real e = nres * tb.gw0[i] * resr[(rs * 2 + end) * Q1 + j];
+        q = p_make(e - Rij, e * T0 - Rij);
+      } else {
+        q = p_load(cell(k, ce) + 2 * v);
+      }
+      for (int d = 1; d <= 3; ++d) p_store(cell(k, end == 0 ? -d : TP - 1 + d) + 2 * v, q);
     }
-    const P gin = inlet ? end_ghost(r, 0, ii, jj) : p_set(real(0));
-    const P gout = outlet ? end_ghost(r, 1, ii, jj) : p_set(real(0));
+  };
+
+  // ---- lambda windows.  Value of row r of column c at or below row sA + 2: the ring, global
+  // memory below the segment, the centreline mirror below row 0 (ghost 1-k of cell k,
+  // p^lambda -> -p^lambda, Sec. VII.C.3)
+  auto low_row = [&](int r, int c) -> P {
+    if (r >= sA) return p_load(cell(slot(r), c) + 2 * v);
+    if (r >= 0) return p_load(a.Fprev + dcell(r, p0 + c) * ROW + 2 * v);
+    return p_load(cell(slot(-1 - r), c) + 2 * (refl(1, Q0, i) * Q1 + j));
+  };
+  // vielbein: the window centred on row s + off; Cartesian split: F(s-2 .. s+3) of step s (scaled).
+  // Before the march's pass sA - 1, which brings in one row more and reconstructs interface sA - 1/2.
+  WenoWin<real, !L::F32> win[CLB ? 1 : TP];
+  P raw[CLB ? TP : 1][6];
+  P flo[TP];  // lambda interface s - 1/2 (scaled)
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const int cc = c0 + q * sd;
-      h[q] = (inlet && cc < 0) ? gin : (outlet && cc >= TP) ? gout : p_load(krow(k, cc) + 2 * vv);
-    }
-  };
-
-  // xi interface TP - 1/2 of row s (the right edge of the strip) for the 32 velocities of chunk ch
-  auto edge_weno = [&](int r, int k, int ch, P* xo) {
-    const int vv = 32 * ch + lane, ii = vv / Q1, jj = vv - ii * Q1;
-    const real pli = tb.p0[ii], pxj = tb.p1[jj];
-    real gm[12];
-    load_geo(gring + k * TP + TP - 1, gm);
-    const bool up = gm[G_BP] * pxj - gm[G_CP] * pli >= real(0);
-    P h[5];
-    xi_stencil(r, k, TP, up, vv, h);
-    xo[TP * V + vv] = weno5p<real>(h[0], h[1], h[2], h[3], h[4], tb.iw0[ii] * tb.iw1[jj]);
-  };
-
-  // window rows from the ring (the centreline mirror below row 0: ghost 1-k of
-  // cell k, p^lambda -> -p^lambda, Sec. VII.C.3)
-  if (is_main) {
-    if (sA == 0) {
-      const int ib = refl(1, Q0, i);
-      W0 = p_load(krow(2 % NRING, c) + 2 * (ib * Q1 + j));
-      W1 = p_load(krow(1 % NRING, c) + 2 * (ib * Q1 + j));
-      W2 = p_load(krow(0, c) + 2 * (ib * Q1 + j));
-    }
-    W3 = p_load(krow(sA % NRING, c) + 2 * v);
-    W4 = p_load(krow((sA + 1) % NRING, c) + 2 * v);
-    W5 = p_load(krow((sA + 2) % NRING, c) + 2 * v);
-  }
-  // moments of rows sA .. sA+2, equilibria and reservoir factors of rows sA, sA+1
-  // (row sA+2's come in the first step)
-  for (int r = sA; r < min(sA + 3, sB); ++r) {
-    if (is_main) moment_partials(p_load(krow(r % NRING, c) + 2 * v), r);
-    __syncthreads();
-    if (is_eqw && r < sA + 2) {
-      for (int job = qw; job < TP; job += 2) eq_job(r, job);
-      res_jobs(r);
-    }
-    __syncthreads();
-  }
-  // row sA+2's partials are the first the equilibrium warps take from the ring
-  if (is_main && sA + 2 < min(nl, sB) && lane == 0) mbar_arrive(pready + (sA + 2) % L::NPR);
-  // lambda interface r - 1/2 from the window W0 .. W5 = F(r-3 .. r+2), upwind by V^lambda: the sign
-  // of p^lambda (vielbein), or of V^lambda = am p^x - glxl p^y of row r's record (Cartesian split)
-  auto lam_face = [&](const ChanCell<real>& g, bool lower) -> P {
+  for (int c = 0; c < TP; ++c) {
     if constexpr (CLB) {
-      const bool up = (lower ? g.am * pl - g.glxl * px : g.ap * pl - g.glxx * px) >= real(0);
-      return weno5p<real>(up ? W0 : W5, up ? W1 : W4, up ? W2 : W3, up ? W3 : W2, up ? W4 : W1, sc);
+#pragma unroll
+      for (int q = 1; q < 6; ++q) raw[c][q] = p_mul(low_row(sA - 4 + q, c), SC);
     } else {
-      (void)g, (void)lower;
-      return lpos ? weno5p<real>(W0, W1, W2, W3, W4, sc) : weno5p<real>(W5, W4, W3, W2, W1, sc);
+      const int b = sA - 3 + off;
+      const P x = p_mul(low_row(b, c), SC);  // (its lower neighbour's terms leave the window at once)
+      win[c].start(x, x, p_mul(low_row(b + 1, c), SC), p_mul(low_row(b + 2, c), SC), p_mul(low_row(b + 3, c), SC));
+    }
+    flo[c] = p_set(real(0));
+  }
+  // Cartesian split: the window of the interface between w[2] and w[3] in upwind order
+  auto clb_win = [](const P* w, bool up) -> WenoWin<real, false> {
+    WenoWin<real, false> t;
+    t.start(p_sel(up, w[0], w[5]), p_sel(up, w[1], w[4]), p_sel(up, w[2], w[3]), p_sel(up, w[3], w[2]),
+            p_sel(up, w[4], w[1]));
+    return t;
+  };
+  // ---- the wall (Sec. VII.C.4), when the march first needs row nl: n_w per column from the
+  // zero-mass-flux balance; rows nl-3 .. nl-1 stay in the ring from there on
+  auto wall_out = [&](int c) -> bool {  // this velocity leaves through the wall
+    if constexpr (CLB) {
+      const ChanCell<real>& gw = gring[slot(nl - 1) * TP + c];
+      return gw.ap[0] * pl - gw.glxx * px > real(0);
+    } else {
+      return pl > real(0);
     }
   };
-  P fm = p_set(real(0));
-  if (is_main) fm = lam_face(gring[(sA % NRING) * TP + c], true);
-  P gh0 = p_set(real(0)), gh1 = p_set(real(0));  // wall ghosts of rows nl, nl+1 (and nl+2)
-  bool wout = false;                              // this velocity leaves through the wall
+  // any row of the lambda stencils, once wall_density has run where it lies beyond the wall
+  auto any_row = [&](int r, int c) -> P {
+    if (r >= nl) return p_load(cell(slot(min(r, nl + 1)), c) + 2 * v);
+    const int vv = r < 0 ? refl(1, Q0, i) * Q1 + j : v;
+    return p_load(a.Fprev + dcell(r < 0 ? -1 - r : r, p0 + c) * ROW + 2 * vv);
+  };
+  // ghosts of rows nl (G1) and nl+1, nl+2 (G2) of the populations leaving column c: quadratic
+  // extrapolation (Eq. extrapol)
+  auto extrapolate = [&](int c, P& G1, P& G2) {
+    const P F3 = p_load(cell(slot(nl - 3), c) + 2 * v), F2 = p_load(cell(slot(nl - 2), c) + 2 * v),
+            F1 = p_load(cell(slot(nl - 1), c) + 2 * v);
+    G1 = p_add(p_sub(p_mul(p_set(real(3)), F1), p_mul(p_set(real(3)), F2)), F3);
+    G2 = p_add(p_sub(p_mul(p_set(real(6)), F1), p_mul(p_set(real(8)), F2)), p_mul(p_set(real(3)), F3));
+  };
+  // The wall's n_w, and its ghost rows into the ring slots of rows nl and nl + 1 (rows nl-5 and
+  // nl-4 have left them; row nl + 2 reads as nl + 1): each thread its own velocity
+  auto wall_density = [&]() {
+#pragma unroll 1
+    for (int c = 0; c < TP; ++c) {
+      real fl = real(0), fd = real(0);
+      const bool out = wall_out(c);
+      real Vw = pl;
+      if constexpr (CLB) {
+        // V^lambda at the wall interface (row nl-1's upper face); the outgoing flux is of F = D + R,
+        // the incoming one of f_eq(1, 0, T0), both over this column's half-planes (Eq. canalie_coord_nw)
+        const ChanCell<real>& gw = gring[slot(nl - 1) * TP + c];
+        Vw = gw.ap[0] * pl - gw.glxx * px;
+        if (!out) fd = tb.gw0[i] * tb.gw1[j] * Vw;
+      }
+      if (out) {
+        WenoWin<real, false> t;
+        P G1, G2;
+        extrapolate(c, G1, G2);
+        t.start(p_mul(p_load(cell(slot(nl - 3), c) + 2 * v), SC), p_mul(p_load(cell(slot(nl - 2), c) + 2 * v), SC),
+                p_mul(p_load(cell(slot(nl - 1), c) + 2 * v), SC), p_mul(G1, SC), p_mul(G2, SC));
+        fl = (t.face_any(true).x * isc + (CLB ? Rij : real(0))) * Vw;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        fl += __shfl_xor_sync(0xffffffffu, fl, o);
+        if constexpr (CLB) fd += __shfl_xor_sync(0xffffffffu, fd, o);
+      }
+      if (lane == 0) wred[c * NW + warp] = fl, wred[(TP + c) * NW + warp] = fd;
+    }
+    __syncthreads();
+    if (v < TP) {
+      double num = CLB ? 0.0 : tb.ref_flux_pos;  // vielbein: the outgoing flux of R, then of D
+      double den = CLB ? 0.0 : tb.wall_den;
+      for (int w = 0; w < NW; ++w) {
+        num += double(wred[v * NW + w]);
+        if (CLB) den += double(wred[(TP + v) * NW + w]);
+      }
+      const double nwc = -num / den;  // Eq. (nw) / (canalie_coord_nw)
+      nwv[v] = nwc;
+      a.nw[p0 + v] = nwc;
+      if (!isfinite(nwc)) atomicOr(a.err, ERR_NONFINITE);
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int c = 0; c < TP; ++c) {
+      P G1, G2;
+      if (wall_out(c)) {
+        extrapolate(c, G1, G2);
+      } else {  // f_eq(n_w, 0, T0) - R (Eq. weno_populate)
+        const real e = real(nwv[c]) * tb.gw0[i] * tb.gw1[j];
+        G1 = G2 = p_make(e - Rij, e * T0 - Rij);
+      }
+      p_store(cell(slot(nl), c) + 2 * v, G1);
+      p_store(cell(slot(nl + 1), c) + 2 * v, G2);
+    }
+  };
+
+  // this thread's F_l and F_out of the strip's first cell in row s; F_l is loaded one step ahead
+  const real* Fl = a.Fl + dcell(sA, p0) * ROW + 2 * v;
+  real* Fo = a.Fout + dcell(sA, p0) * ROW + 2 * v;
+  const size_t rstep = size_t(nx) * ROW;
+  P flr[TP];
+#pragma unroll
+  for (int c = 0; c < TP; ++c) {
+    flr[c] = p_set(real(0));
+    if (need_fl) flr[c] = p_load(Fl + c * ROW);
+  }
   __syncthreads();
 
-  // ---- the equilibrium warps: rows sA+2 .. in order, each as soon as the column warps have
-  // reduced its moments, two or three rows ahead of the step that uses it; they take part in
-  // no step barrier (the step phases synchronise on named barrier 1 of the other NSYNC threads)
-  const int rend = min(nl, sB);
-  if (is_eqw) {
-    unsigned pph = 0;
-    for (int r = sA + 2; r < rend; ++r) {
-      const int k = r % L::NPR;
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(pready + k, (pph >> k) & 1u, a.max_polls);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      pph ^= 1u << k;
-      if (!ok) {  // the column warps stopped (their own wait ran out): leave
-        if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
-        return;
-      }
-      __syncwarp();
-      for (int job = qw; job < TP; job += 2) eq_job(r, job);
-      res_jobs(r);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(eready + (r & (L::NEQ - 1)));
-    }
-    return;
-  }
-  unsigned eph = 0;          // thread 0: parity of the next wait, per equilibrium-ready slot
-  int eq_waited = sA + 1;    // rows up to this one have their records (the prologue made sA, sA+1)
-  unsigned phase_bits = 0;   // main threads: parity of the next wait, per step mbarrier
-  bool good = true;          // every wait of this thread so far ended in time
-  P flr = p_set(real(0));    // F_l of the row being finished, prefetched one step ahead
-  if (is_main && need_fl) flr = p_load(a.Fl + dcell(sA, p0 + c) * ROW + 2 * v);
-  P fp = p_set(real(0));     // lambda interface s + 1/2 of the row whose interfaces were built last
-  P frc = p_set(real(0));    // force of that row (double-precision path)
-  auto sync_all = [&]() { named_bar(1, NSYNC); };
-  auto sync_and = [&](bool v) { return named_bar_and(1, NSYNC, v); };
+  // ---- the march.  Its first three passes only run the roles of the first rows; the third also
+  // reconstructs the lambda interfaces sA - 1/2.
+#pragma unroll 1
+  for (int s = sA - 3; s < sB; ++s) {
+    if (s >= sA - 1) {
+    const bool full = s >= sA;
+    if (full && warp == 0 && s + 4 <= rlast) row_issue(s + 4);
+    if (s > sA && s + 3 <= rlast) good = row_wait(s + 3) && good;
+    if (s == nl - 3) wall_density();
+    const int k0 = full ? slot(s) : 0;
+    const int k3 = slot(min(s + 2 + (CLB ? 1 : off), nl + 1));  // the row that joins the lambda windows
+    const ChanCell<real>* geo = gring + k0 * TP;
+    const P R2 = p_set(CLB ? Rij * SC.x : real(0));
 
-  // combine of cell (r, c) (main threads), once row r's interface values and force are
-  // written (the step barrier after row r's step): F(r) = W2, lambda interfaces r -/+ 1/2 in
-  // fm / fp, xi interfaces and force from the row-parity half of the buffers
-  auto combine = [&](int r) {
-    real gm[12];
-    load_geo(gring + (r % NRING) * TP + c, gm);
-    const P* xb = xif + (r & 1) * (TP + 1) * V;
-    const P FL = xb[c * V + v], FR = xb[(c + 1) * V + v];
-    const real Vm = gm[G_BM] * px - gm[G_CM] * pl, Vp = gm[G_BP] * px - gm[G_CP] * pl;
-    P adv;
-    if constexpr (CLB) {
-      // Eq. (canalie_coord_beq_cons): fluxes of F = D + R, V^lambda per interface (no force term
-      // balances the rest state's advection here)
-      const P R2 = p_set(Rij);
-      const real Vlm = gm[G_AM] * pl - gm[G_GLXL] * px, Vlp = gm[G_AP] * pl - gm[G_GLXX] * px;
-      adv = p_mul(p_set(gm[G_IDL]), p_sub(p_mul(p_set(Vlp), p_add(fp, R2)), p_mul(p_set(Vlm), p_add(fm, R2))));
-      adv = p_fma(p_set(gm[G_IDX]), p_sub(p_mul(p_set(Vp), p_add(FR, R2)), p_mul(p_set(Vm), p_add(FL, R2))), adv);
-    } else {
-      // chi flux differences (Sec. VII.B)
-      adv = p_mul(p_set(pl * gm[G_IDL]), p_sub(p_mul(p_set(gm[G_AP]), fp), p_mul(p_set(gm[G_AM]), fm)));
-      adv = p_fma(p_set(gm[G_IDX]), p_sub(p_mul(p_set(Vp), FR), p_mul(p_set(Vm), FL)), adv);
-    }
-    if constexpr (F32 && !CLB) {
-      const real* lb = lbl + (r & 1) * TP * ROW;
-      const real* lx = lbx + (r & 1) * TP * ROW;
-      frc = p_add(p_load(lb + c * ROW + 2 * v), p_load(lx + c * ROW + 2 * v));
-    }
-    const real* rec = eqr + ((r & (L::NEQ - 1)) * TP + c) * EQW;
-    const real geq = rec[i] * rec[Q0 + j];
-    const P deq = p_make(geq - Rij, geq * rec[Q0 + Q1] - Rij);
-    const real itau = rec[Q0 + Q1 + 1];
-    const P F = W2;  // F(r)
-    // L = -advection + force - (F - f_eq) / tau
-    const P Lv = p_sub(p_sub(frc, adv), p_mul(p_set(itau), p_sub(F, deq)));
-    P o = p_fma(p_set(a.ccdt), Lv, F);
-    if (need_fl) o = p_fma(p_set(a.ca), p_sub(flr, F), o);
-    p_store(a.Fout + dcell(r, p0 + c) * ROW + 2 * v, o);
-    if (need_fl && r + 1 < sB) flr = p_load(a.Fl + dcell(r + 1, p0 + c) * ROW + 2 * v);
-  };
-
-  // ---- the march: step s finishes row s-1 (the combine) while it builds row s's interface
-  // values and force; one barrier per step, after which row s's outputs are complete.  The
-  // last pass (s = sB) only finishes row sB-1.
-  for (int s = sA; s <= sB; ++s) {
-    const bool build = s < sB;
-    const int k0 = s % NRING, k3 = (s + 3) % NRING;
-    if (build && is_main && s - PD >= sA && s + 3 <= rlast) {  // the group issued PD steps ago brought row s+3
-      const int b = (s - PD) % NB;
-      good = mbar_wait(bar + b, (phase_bits >> b) & 1u, a.max_polls) && good;
-      phase_bits ^= 1u << b;
-    }
-    if (build && tid == NMAIN && s + 3 + PD <= rlast) {  // row s+3+PD into the slot row s-2 left
-      uint64_t* b = bar + s % NB;
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_expect_tx(b, row_bytes());
-      row_issue(s + 3 + PD, b);
-    }
-    // the wall (Sec. VII.C.4): at the first row whose window reaches it, n_w per
-    // column from the zero-mass-flux balance and the ghosts of rows nl .. nl+2
-    if (build && top && s == nl - 3) {
-      if (is_main) {
-        // W3 .. W5 = F(nl-3 .. nl-1); outgoing populations: quadratic extrapolation (Eq. extrapol)
-        const P G0 = p_add(p_sub(p_mul(p_set(real(3)), W5), p_mul(p_set(real(3)), W4)), W3);
-        const P G1 = p_add(p_sub(p_mul(p_set(real(6)), W5), p_mul(p_set(real(8)), W4)), p_mul(p_set(real(3)), W3));
-        real fl = real(0), fd = real(0);
-        if constexpr (CLB) {
-          // V^lambda at the wall interface (row nl-1's upper face); the outgoing flux is of F = D + R,
-          // the incoming one of f_eq(1, 0, T0), both over this column's half-planes (Eq. canalie_coord_nw)
-          const ChanCell<real>& gw = gring[((nl - 1) % NRING) * TP + c];
-          const real Vw = gw.ap * pl - gw.glxx * px;
-          if (Vw > real(0)) fl = (weno5p<real>(W3, W4, W5, G0, G1, sc).x + Rij) * Vw;
-          else fd = tb.gw0[i] * tb.gw1[j] * Vw;
-          wout = Vw > real(0);
-        } else {
-          if (pl > real(0)) fl = weno5p<real>(W3, W4, W5, G0, G1, sc).x * pl;
-          wout = pl > real(0);
-        }
+    // ---- xi: V F (CLB: of F = D + R) at the five interfaces of the strip in one walk.  V^xi = b p^xi
+    // - c p^lambda (Eq. canalie_V), times isc; an interface's upwind cell follows the last one's,
+    // unless V^xi changes its sign between the two.
+    P dphi[TP];
+    if (full) {
+      auto xi_load = [&](int cc) -> P { return p_mul(p_load(cell(k0, cc) + 2 * v), SC); };
+      auto xi_vel = [&](int c) -> real {
+        const P bc = p_load(c < TP ? &geo[c].bm : &geo[TP - 1].bp);
+        return bc.x * pxI - bc.y * plI;
+      };
+      auto flux = [&](real V, P f) -> P { return p_mul(p_set(V), CLB ? p_add(f, R2) : f); };
+      WenoWin<real, true> wx;
+      WenoSide<real> sx;
+      WenoRange<real> range;
+      real V = xi_vel(0);
+      bool up = V >= real(0);
+      sx.set(up);
+      const real* q = cell(k0, up ? -3 : -2) + 2 * v;
+      wx.start(p_mul(p_load(q), SC), p_mul(p_load(q + CS), SC), p_mul(p_load(q + 2 * CS), SC),
+               p_mul(p_load(q + 3 * CS), SC), p_mul(p_load(q + 4 * CS), SC));
+      P phi[TP + 1];
+      phi[0] = flux(V, wx.face(sx, range));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          fl += __shfl_xor_sync(0xffffffffu, fl, o);
-          if constexpr (CLB) fd += __shfl_xor_sync(0xffffffffu, fd, o);
-        }
-        if (lane == 0) wred[c * NWC + wc] = fl, wred[(TP + c) * NWC + wc] = fd;
-        gh0 = G0;
-        gh1 = G1;
-      }
-      sync_all();
-      if (!is_main && lane == 0)
-        for (int cc = ew; cc < TP; cc += NWC) {
-          double num = CLB ? 0.0 : tb.ref_flux_pos;  // vielbein: the outgoing flux of R, then of D
-          double den = CLB ? 0.0 : tb.wall_den;
-          for (int w = 0; w < NWC; ++w) {
-            num += double(wred[cc * NWC + w]);
-            if (CLB) den += double(wred[(TP + cc) * NWC + w]);
-          }
-          const double nwc = -num / den;  // Eq. (nw) / (canalie_coord_nw)
-          nwv[cc] = nwc;
-          a.nw[p0 + cc] = nwc;
-          if (!isfinite(nwc)) atomicOr(a.err, ERR_NONFINITE);
-        }
-      sync_all();
-      if (is_main && !wout) {  // incoming: f_eq(n_w, 0, T0) - R (Eq. weno_populate)
-        const real e = real(nwv[c]) * tb.gw0[i] * tb.gw1[j];
-        gh0 = gh1 = p_make(e - Rij, e * T0 - Rij);
-      }
-    }
-    if (is_main && s > sA) {
-      combine(s - 1);
-      fm = fp;
-    }
-    if (!build) break;
-
-    // ==== row s: interface values and force, into the row-parity half of the buffers
-    P* xo = xif + (s & 1) * (TP + 1) * V;
-    real* lo = lbl + (s & 1) * TP * ROW;
-    real* xo2 = lbx + (s & 1) * TP * ROW;
-    if (is_main) {
-      const int rn = s + 3;
-      const P fnew = rn < nl ? p_load(krow(k3, c) + 2 * v) : (rn == nl ? gh0 : gh1);
-      if (rn < rend) {
-        moment_partials(fnew, rn);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(pready + rn % L::NPR);  // the equilibrium warps take row rn from here
-      }
-      W0 = W1, W1 = W2, W2 = W3, W3 = W4, W4 = W5, W5 = fnew;  // W = F(s-2 .. s+3)
-      real gm[12];
-      load_geo(gring + k0 * TP + c, gm);
-      // xi interface c - 1/2: upwind by V^xi = b p^xi - c p^lambda (Eq. canalie_V)
-      const bool up = gm[G_BM] * px - gm[G_CM] * pl >= real(0);
-      P h[5];
-      xi_stencil(s, k0, c, up, v, h);
-      const P FL = weno5p<real>(h[0], h[1], h[2], h[3], h[4], sc);
-      // lambda interface s + 1/2 from the window, upwind by p^lambda (a > 0): independent of
-      // the xi one, so the two interleave
-      fp = lam_face(gring[k0 * TP + c], false);
-      xo[c * V + v] = FL;
-      if constexpr (CLB) {
-        // no force term
-      } else if constexpr (F32 && TC) {
-        // force subtasks of the row's cells on the tensor cores (mma.sync needs the
-        // warp converged after the data-dependent WENO branches)
-        __syncwarp();
-        for (int t = mw; t < TP * S::S; t += NMW) {
-          const int cc = t / S::S, kt = t - cc * S::S;
-          const ChanCell<real>& gk = gring[k0 * TP + cc];
-          force_subtask_tc<Q0, Q1>(tb, krow(k0, cc), gk.glxx, gk.glxl, kt, lane, lo + cc * ROW, xo2 + cc * ROW);
-        }
-      } else if constexpr (!F32) {
-        const real* F = krow(k0, c);
-        P s0 = p_set(real(0)), s1 = p_set(real(0)), s2 = p_set(real(0)), s3 = p_set(real(0));
-        for (int ip = 0; ip < Q0; ++ip) {
-          const P f = p_load(F + 2 * (ip * Q1 + j));
-          s0 = p_fma(p_set(tb.K0[i * Q0 + ip]), f, s0);
-          s1 = p_fma(p_set(tb.Kt0[i * Q0 + ip]), f, s1);
-        }
-        for (int jp = 0; jp < Q1; ++jp) {
-          const P f = p_load(F + 2 * (i * Q1 + jp));
-          s2 = p_fma(p_set(tb.K1[j * Q1 + jp]), f, s2);
-          s3 = p_fma(p_set(tb.Kt1[j * Q1 + jp]), f, s3);
-        }
-        // G_lxx [(p^xi)^2 K0 f - p^lambda Kt1 f] - G_lxl [(p^lambda)^2 K1 f - p^xi Kt0 f]
-        const P A = p_fma(p_set(px * px), s0, p_mul(p_set(-pl), s3));
-        const P B = p_fma(p_set(pl * pl), s2, p_mul(p_set(-px), s1));
-        frc = p_fma(p_set(gm[G_GLXX]), A, p_mul(p_set(-gm[G_GLXL]), B));
-      }
-    } else if constexpr (F32 && !TC && !CLB) {
-      // force tasks of the row's cells on the CUDA cores (lambda: one per (cell, column
-      // j); xi: one per (cell, row i)) in units of 32 (one warp), then the strip's
-      // right-edge xi interface, over the extra warps
-      constexpr int NTL = TP * Q1, NTX = TP * Q0;
-      constexpr int NWL = (NTL + 31) / 32, NWX = (NTX + 31) / 32;
-      for (int u = ew; u < NWL + NWX + NWC; u += NWC) {
-        if (u < NWL) {
-          const int t = 32 * u + lane;
-          if (t < NTL) {
-            const int cc = t / Q1, jj = t - cc * Q1;
-            const ChanCell<real>& gk = gring[k0 * TP + cc];
-            const float pxj = tb.p1[jj];
-            force_lambda_cc<Q0, Q1>(kp, krow(k0, cc), jj, gk.glxx * pxj * pxj, gk.glxl * pxj, lo + cc * ROW);
-          }
-        } else if (u < NWL + NWX) {
-          const int t = 32 * (u - NWL) + lane;
-          if (t < NTX) {
-            const int cc = t / Q0, ii = t - cc * Q0;
-            const ChanCell<real>& gk = gring[k0 * TP + cc];
-            const float pli = tb.p0[ii];
-            force_xi_cc<Q0, Q1>(kp, krow(k0, cc), ii, -gk.glxx * pli, -gk.glxl * pli * pli, xo2 + cc * ROW);
-          }
+      for (int c = 1; c <= TP; ++c) {
+        V = xi_vel(c);
+        if ((V >= real(0)) == up) {
+          wx.push(p_mul(p_load(q + (4 + c) * CS), SC));
         } else {
-          edge_weno(s, k0, u - NWL - NWX, xo);
+          up = !up;
+          sx.set(up);
+          q += up ? -CS : CS;
+          wx.start(p_mul(p_load(q + c * CS), SC), p_mul(p_load(q + (1 + c) * CS), SC), p_mul(p_load(q + (2 + c) * CS), SC),
+                   p_mul(p_load(q + (3 + c) * CS), SC), p_mul(p_load(q + (4 + c) * CS), SC));
+        }
+        phi[c] = flux(V, wx.face(sx, range));
+      }
+      if (__any_sync(0xffffffffu, !range.ok())) {  // some weights left their range
+#pragma unroll 1
+        for (int c = 0; c <= TP; ++c) {
+          V = xi_vel(c);
+          up = V >= real(0);
+          const int n = up ? c - 1 : c;
+          wx.start(xi_load(n - 2), xi_load(n - 1), xi_load(n), xi_load(n + 1), xi_load(n + 2));
+          const P x = flux(V, wx.face_any(up));
+          const int to = wx.in_range(up) ? -1 : c;
+#pragma unroll
+          for (int k = 0; k <= TP; ++k) phi[k] = p_sel(k == to, x, phi[k]);
         }
       }
-    } else {
-      // the strip's right-edge xi interface of row s, 32 velocities per extra warp
-      for (int ch = ew; ch < NWC; ch += NWC) edge_weno(s, k0, ch, xo);
+#pragma unroll
+      for (int c = 0; c < TP; ++c) dphi[c] = p_mul(p_load(geo[c].idx), p_sub(phi[c + 1], phi[c]));
     }
-    // the step barrier; before it, the records of rows s (the next combine) and s+1 (the
-    // reservoir ghosts of the next step) must be written
-    {
-      const int want = min(s + 1, rend - 1);
-      if (tid == 0)
-        while (eq_waited < want) {
-          const int r = ++eq_waited, k = r & (L::NEQ - 1);
-          good = mbar_wait(eready + k, (eph >> k) & 1u, a.max_polls) && good;
-          eph ^= 1u << k;
-        }
-      if (!sync_and(good)) {
-        // a wait ran out: wait (bounded) for the bulk copies still in flight -- the groups
-        // issued at steps s-PD .. s (the one waited for this step may be the late one) --
-        // then leave together
-        if (tid == 0) {
-          atomicOr(a.err, ERR_TIMEOUT);
-          for (int g = s - PD; g <= s; ++g)
-            if (g >= sA && g + 3 + PD <= rlast) {
-              const int b = g % NB;
-              mbar_wait(bar + b, g == s - PD ? ((phase_bits >> b) & 1u) ^ 1u : (phase_bits >> b) & 1u, a.max_polls);
-            }
-        }
-        sync_all();
-        return;
+
+    // ---- lambda interface s + 1/2 of every column
+    P fhi[TP];
+    WenoRange<real> range;
+    auto lam_up = [&](int c) -> bool {  // upwind side of interface s + 1/2, Cartesian split
+      const ChanCell<real>& g = geo[c];
+      return (full ? g.ap[0] * pl - g.glxx * px : -(g.nam[0] * pl + g.glxl * px)) >= real(0);
+    };
+#pragma unroll
+    for (int c = 0; c < TP; ++c) {
+      const P fnew = p_mul(p_load(cell(k3, c) + 2 * v), SC);
+      if constexpr (CLB) {
+#pragma unroll
+        for (int q = 0; q < 5; ++q) raw[c][q] = raw[c][q + 1];
+        raw[c][5] = fnew;
+        fhi[c] = clb_win(raw[c], lam_up(c)).face(wl, range);
+      } else {
+        win[c].push(fnew);
+        fhi[c] = win[c].face(wl, range);
       }
+    }
+    if (__any_sync(0xffffffffu, !range.ok())) {
+#pragma unroll 1
+      for (int c = 0; c < TP; ++c) {
+        // from memory: the windows' older terms are not kept
+        const bool up = CLB ? lam_up(c) : lpos;
+        const int b = s + (up ? 0 : 1) - 2;
+        WenoWin<real, false> w;
+        w.start(p_mul(any_row(b, c), SC), p_mul(any_row(b + 1, c), SC), p_mul(any_row(b + 2, c), SC),
+                p_mul(any_row(b + 3, c), SC), p_mul(any_row(b + 4, c), SC));
+        const P x = w.face_any(up);
+        const int to = w.in_range(up) ? -1 : c;
+#pragma unroll
+        for (int k = 0; k < TP; ++k) fhi[k] = p_sel(k == to, x, fhi[k]);
+      }
+    }
+
+    // ---- the combine of row s
+    if (full) {
+      const real* rec = eqr + (s & (L::NEQ - 1)) * TP * EQW;
+      const real* fb = lbl + (s & 1) * TP * CS + 2 * v;
+      const real* xb = lbx + ((s & 1) * TP * Q0 + i) * XS + 2 * j;
+#pragma unroll
+      for (int c = 0; c < TP; ++c) {
+        const ChanCell<real>& g = geo[c];
+        P adv;
+        if constexpr (CLB) {
+          // Eq. (canalie_coord_beq_cons): fluxes of F = D + R, V^lambda per interface (no force term
+          // balances the rest state's advection here)
+          const real Vlm = g.nam[0] * plI + g.glxl * pxI, Vlp = g.ap[0] * plI - g.glxx * pxI;
+          adv = p_add(p_fma(p_set(Vlp), p_add(fhi[c], R2), p_mul(p_set(Vlm), p_add(flo[c], R2))), dphi[c]);
+        } else {
+          // chi flux differences (Sec. VII.B)
+          adv = p_fma(PLI, p_fma(p_load(g.ap), fhi[c], p_mul(p_load(g.nam), flo[c])), dphi[c]);
+        }
+        // L = -advection + force - (F - f_eq) / tau
+        const real* rc = rec + c * EQW;
+        const P deq = p_fma(p_mul(p_load(rc + 2 * i), p_load(rc + 2 * (Q0 + j))), p_load(rc + 2 * (Q0 + Q1)), NR);
+        const P F = p_load(cell(k0, c) + 2 * v);
+        P Lv = p_sub(p_mul(p_sub(F, deq), p_load(rc + 2 * (Q0 + Q1) + 2)), adv);
+        if constexpr (!CLB) Lv = p_add(Lv, p_add(p_load(fb + c * CS), p_load(xb + c * Q0 * XS)));
+        P o = p_fma(a.ccdt, Lv, F);
+        if (need_fl) o = p_fma(a.ca, p_sub(flr[c], F), o);
+        p_store(Fo + c * ROW, o);
+      }
+      Fl += rstep;
+      Fo += rstep;
+      if (need_fl && s + 1 < sB)
+#pragma unroll
+        for (int c = 0; c < TP; ++c) flr[c] = p_load(Fl + c * ROW);
+    }
+#pragma unroll
+    for (int c = 0; c < TP; ++c) flo[c] = fhi[c];
+    }
+    // ---- the rows ahead
+    if (s + 3 < sB) eq_row(s + 3);
+    if (s + 2 >= sA && s + 2 < sB) res_row(s + 2);
+    if (s + 1 >= sA && s + 1 < sB) {
+      force_row(s + 1);
+      if (inlet || outlet) fill_ghosts(s + 1);
+    }
+    if (!__syncthreads_and(good)) {
+      give_up();
+      return;
     }
   }
 }

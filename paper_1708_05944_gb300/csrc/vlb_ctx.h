@@ -87,10 +87,11 @@ struct vlb_ctx {
   ChanDesc cdesc{};
   ChanVariant cvariants[8];
   int n_cvariants = 0;
+  int chan_per_sm = 1;  // resident CTAs of the channel stage kernel per SM
   ChanCell<double>* d_cgeo = nullptr;
   ChanCell<float>* d_cgeof = nullptr;
   CellMap cmap;  // device cell order against the caller's (identity for Couette)
-  std::vector<unsigned char> chan_kp;  // ChanKP block (split force matrices), a kernel parameter
+  std::vector<unsigned char> chan_kp;  // ChanKP block (force matrices), a kernel parameter
   void* d_ctab = nullptr;  // ChanTables of the model shape in the context's real type
   size_t ctab_bytes = 0;
   std::vector<double> chan_lc;    // lambda of the row centres

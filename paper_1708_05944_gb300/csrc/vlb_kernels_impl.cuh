@@ -205,22 +205,22 @@ cudaError_t stage_config(StageVariant v, const ModelArgs& m, int Vp, int* nbuf, 
 }
 
 // ---------------------------------------------------------------- channel dispatch
-template <typename real, int Q0, int Q1, int TP, bool TC, bool CLB = false>
+template <typename real, int Q0, int Q1, bool CLB, bool HX>
 static cudaError_t go_channel(const ChanArgs<real>& a, const void* kpb, int grid, cudaStream_t s) {
-  using L = ChanSmem<real, Q0, Q1, TP>;
-  auto kern = channel_stage_kernel<real, Q0, Q1, TP, TC, CLB>;
+  using L = ChanSmem<real, Q0, Q1>;
+  auto kern = channel_stage_kernel<real, Q0, Q1, CLB, HX>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(L::bytes));
   if (e != cudaSuccess) return e;
-  ChanKP<Q0, Q1> kp;
+  ChanKP<real, Q0, Q1> kp;
   memcpy(&kp, kpb, sizeof(kp));
   kern<<<grid, L::NT, L::bytes, s>>>(a, kp);
   return cudaGetLastError();
 }
 
 #ifdef VLB_DEFINE_SHARED
-// {rows per segment (0: host's choice, 1 << 20: one segment), columns per strip, threads, tensor-core force}
-static const ChanVariant kChan16x12[] = {{0, 4, 1024, 0}, {0, 4, 1024, 1}, {1 << 20, 4, 1024, 0}, {64, 4, 1024, 0}};
-static const ChanVariant kChan8x4[] = {{0, 4, 224, 0}, {0, 8, 352, 0}, {0, 4, 224, 1}, {1 << 20, 4, 224, 0}};
+// {rows per segment (0: host's choice, 1 << 20: one segment), columns per strip, threads}
+static const ChanVariant kChan16x12[] = {{0, 4, 192}, {128, 4, 192}, {1 << 20, 4, 192}, {64, 4, 192}};
+static const ChanVariant kChan8x4[] = {{0, 4, 32}, {64, 4, 32}, {16, 4, 32}, {1 << 20, 4, 32}};
 
 int channel_variants(int nq0, int nq1, ChanVariant* out) {
   const ChanVariant* v = nullptr;
@@ -230,77 +230,83 @@ int channel_variants(int nq0, int nq1, ChanVariant* out) {
   for (int i = 0; i < n; ++i) out[i] = v[i];
   return n;
 }
-
-template <int Q0, int Q1>
-static bool fill_force_pairs(const AxisTables* ax, std::vector<unsigned char>* out) {
-  using KP = ChanKP<Q0, Q1>;
-  out->assign(sizeof(KP), 0);
-  KP& kp = *reinterpret_cast<KP*>(out->data());
-  // each axis: nodes mirror each other under J, K J = -J K and Kt J = J Kt, to rounding
-  for (int a = 0; a < 2; ++a) {
-    const AxisTables& t = ax[a];
-    const int nq = t.nq;
-    double kmax = 0.0, tmax = 0.0, pmax = 0.0;
-    for (int k = 0; k < nq * nq; ++k) kmax = std::max(kmax, std::fabs(t.K[k])), tmax = std::max(tmax, std::fabs(t.Kt[k]));
-    for (int k = 0; k < nq; ++k) pmax = std::max(pmax, std::fabs(t.p[k]));
-    for (int r = 0; r < nq; ++r) {
-      if (std::fabs(t.p[refl(t.kind, nq, r)] + t.p[r]) > 1e-13 * pmax) return false;
-      for (int q = 0; q < nq; ++q) {
-        const int rr = refl(t.kind, nq, r), qq = refl(t.kind, nq, q);
-        if (std::fabs(t.K[rr * nq + qq] + t.K[r * nq + q]) > 1e-12 * kmax) return false;
-        if (std::fabs(t.Kt[rr * nq + qq] - t.Kt[r * nq + q]) > 1e-12 * tmax) return false;
-      }
-    }
-  }
-  // the kernels take the mirror of k as k + H on the half-range lambda axis and Q1 - 1 - k
-  // on the full-range xi axis
-  if (ax[0].kind != 1 || ax[1].kind != 0) return false;
-  auto put = [](float2* P, float2* M, const std::vector<double>& K, int nq, int kind) {
-    const int H = nq / 2;
-    for (int r = 0; r < H; ++r)
-      for (int q = 0; q < H; ++q) {
-        const double x = K[r * nq + q], y = K[r * nq + refl(kind, nq, q)];
-        const float pv = float(0.5 * (x + y)), mv = float(0.5 * (x - y));
-        P[r * H + q] = make_float2(pv, pv);
-        M[r * H + q] = make_float2(mv, mv);
-      }
-  };
-  put(kp.P0, kp.M0, ax[0].K, Q0, 1);
-  put(kp.Pt0, kp.Mt0, ax[0].Kt, Q0, 1);
-  put(kp.P1, kp.M1, ax[1].K, Q1, 0);
-  put(kp.Pt1, kp.Mt1, ax[1].Kt, Q1, 0);
-  return true;
-}
-
-bool channel_force_pairs(int nq0, int nq1, const AxisTables* ax, std::vector<unsigned char>* out) {
-  if (nq0 == 16 && nq1 == 12) return fill_force_pairs<16, 12>(ax, out);
-  if (nq0 == 8 && nq1 == 4) return fill_force_pairs<8, 4>(ax, out);
-  return false;
-}
 #endif
 
-template <typename real>
-size_t channel_smem_bytes(ChanVariant v, int nq0, int nq1) {
-  if (nq0 == 16 && nq1 == 12 && v.tp == 4) return ChanSmem<real, 16, 12, 4>::bytes;
-  if (nq0 == 8 && nq1 == 4 && v.tp == 4) return ChanSmem<real, 8, 4, 4>::bytes;
-  if (nq0 == 8 && nq1 == 4 && v.tp == 8) return ChanSmem<real, 8, 4, 8>::bytes;
-  return 0;
+static inline void put_coef(float2& c, double x) { c.x = c.y = float(x); }
+static inline void put_coef(double& c, double x) { c = x; }
+
+// One axis of the ChanKP block: the split of K and Kt = K diag(p) + z v^T.  False if a matrix
+// lacks the reflection symmetry or the rank-1 form the kernel relies on.
+template <typename C>
+static bool fill_force_axis(const AxisTables& t, C* P, C* M, C* p, C* v, C* z) {
+  const int nq = t.nq, H = nq / 2;
+  double kmax = 0.0, tmax = 0.0, pmax = 0.0;
+  for (int k = 0; k < nq * nq; ++k) kmax = std::max(kmax, std::fabs(t.K[k])), tmax = std::max(tmax, std::fabs(t.Kt[k]));
+  for (int k = 0; k < nq; ++k) pmax = std::max(pmax, std::fabs(t.p[k]));
+  for (int r = 0; r < nq; ++r) {
+    const int rr = refl(t.kind, nq, r);
+    if (std::fabs(t.p[rr] + t.p[r]) > 1e-13 * pmax) return false;
+    for (int q = 0; q < nq; ++q) {
+      const int qq = refl(t.kind, nq, q);
+      if (std::fabs(t.K[rr * nq + qq] + t.K[r * nq + q]) > 1e-12 * kmax) return false;
+      if (std::fabs(t.Kt[rr * nq + qq] - t.Kt[r * nq + q]) > 1e-12 * tmax) return false;
+    }
+  }
+  // E = Kt - K diag(p) = z v^T from its largest entry, in the symmetric scaling sqrt(w_q / w_r) E
+  // whose entries are of one size; the residual has to vanish to rounding
+  std::vector<double> E(nq * nq);
+  double emax = 0.0, scale = 0.0;
+  int rm = 0, qm = 0;
+  for (int r = 0; r < nq; ++r)
+    for (int q = 0; q < nq; ++q) {
+      const double s = std::sqrt(t.w[q] / t.w[r]);
+      E[r * nq + q] = s * (t.Kt[r * nq + q] - t.K[r * nq + q] * t.p[q]);
+      scale = std::max(scale, s * std::fabs(t.Kt[r * nq + q]));
+      if (std::fabs(E[r * nq + q]) > emax) emax = std::fabs(E[r * nq + q]), rm = r, qm = q;
+    }
+  std::vector<double> zz(nq, 0.0), vv(nq, 0.0);
+  if (emax > 1e-11 * scale)
+    for (int k = 0; k < nq; ++k) zz[k] = E[k * nq + qm] / E[rm * nq + qm], vv[k] = E[rm * nq + k];
+  else if (t.kind == 1) return false;
+  for (int r = 0; r < nq; ++r) {
+    const int rr = refl(t.kind, nq, r);
+    if (std::fabs(zz[rr] + zz[r]) > 1e-11 || std::fabs(vv[rr] + vv[r]) > 1e-11 * scale) return false;
+    for (int q = 0; q < nq; ++q)
+      if (std::fabs(E[r * nq + q] - zz[r] * vv[q]) > 1e-11 * scale) return false;
+  }
+  for (int r = 0; r < H; ++r) {
+    put_coef(p[r], t.p[r]);
+    put_coef(z[r], zz[r] * std::sqrt(t.w[r]));
+    put_coef(v[r], vv[r] / std::sqrt(t.w[r]));
+    for (int q = 0; q < H; ++q) {
+      const double x = t.K[r * nq + q], y = t.K[r * nq + refl(t.kind, nq, q)];
+      put_coef(P[r * H + q], 0.5 * (x + y));
+      put_coef(M[r * H + q], 0.5 * (x - y));
+    }
+  }
+  return true;
+}
+template <typename real, int Q0, int Q1>
+static bool fill_force_block(const AxisTables* ax, std::vector<unsigned char>* out) {
+  using KP = ChanKP<real, Q0, Q1>;
+  out->assign(sizeof(KP), 0);
+  KP& kp = *reinterpret_cast<KP*>(out->data());
+  return ax[0].kind == 1 && fill_force_axis(ax[0], kp.P0, kp.M0, kp.p0, kp.v0, kp.z0) &&
+         fill_force_axis(ax[1], kp.P1, kp.M1, kp.p1, kp.v1, kp.z1);
 }
 
-// TF32 part of x rounded to nearest, ties away from zero (the rounding of
-// cvt.rna.tf32.f32): the low 13 significand bits cleared.
-static inline uint32_t host_tf32(float x) {
-  uint32_t u;
-  memcpy(&u, &x, 4);
-  if ((u & 0x7f800000u) == 0x7f800000u) return u;
-  return (u + 0x1000u) & 0xffffe000u;
+template <typename real>
+bool channel_force_pairs(int nq0, int nq1, const AxisTables* ax, std::vector<unsigned char>* out) {
+  if (nq0 == 16 && nq1 == 12) return fill_force_block<real, 16, 12>(ax, out);
+  if (nq0 == 8 && nq1 == 4) return fill_force_block<real, 8, 4>(ax, out);
+  return false;
 }
-static inline void host_tf32_split(double x, uint32_t* hi, uint32_t* lo) {
-  const float f = float(x);
-  *hi = host_tf32(f);
-  float h;
-  memcpy(&h, hi, 4);
-  *lo = host_tf32(f - h);
+
+template <typename real>
+size_t channel_smem_bytes(ChanVariant, int nq0, int nq1, int* per_sm) {
+  if (nq0 == 16 && nq1 == 12) return *per_sm = ChanSmem<real, 16, 12>::min_ctas, ChanSmem<real, 16, 12>::bytes;
+  if (nq0 == 8 && nq1 == 4) return *per_sm = ChanSmem<real, 8, 4>::min_ctas, ChanSmem<real, 8, 4>::bytes;
+  return 0;
 }
 
 // Axis moment vector of the truncated equilibrium at rest (u = 0), in double.
@@ -317,47 +323,23 @@ static void rest_moment_vector(int kind, int N, double T, double* m) {
 }
 
 template <typename real, int Q0, int Q1>
-static void fill_chan_tables(const AxisTables* ax, const ModelArgs& m, double T0, std::vector<unsigned char>* out) {
+static void fill_chan_tables(const ModelArgs& m, double T0, std::vector<unsigned char>* out) {
   using Tab = ChanTables<real, Q0, Q1>;
-  using S = ChanShape<Q0, Q1>;
   out->assign(sizeof(Tab), 0);
   Tab& t = *reinterpret_cast<Tab*>(out->data());
-  const std::vector<double>&K0 = ax[0].K, &Kt0 = ax[0].Kt, &K1 = ax[1].K, &Kt1 = ax[1].Kt;
-  for (int k = 0; k < Q0 * Q0; ++k) t.K0[k] = real(K0[k]), t.Kt0[k] = real(Kt0[k]);
-  for (int k = 0; k < Q1 * Q1; ++k) t.K1[k] = real(K1[k]), t.Kt1[k] = real(Kt1[k]);
-  // lambda A fragments: a0 = K0[8t+g][8kk+tq], a1 = Kt0[..][8kk+tq], a2 = K0[..][8kk+tq+4], a3 = Kt0[..][8kk+tq+4]
-  for (int mt = 0; mt < S::MT; ++mt)
-    for (int kk = 0; kk < S::KKL; ++kk)
-      for (int lane = 0; lane < 32; ++lane) {
-        const int g = lane >> 2, tq = lane & 3, r = 8 * mt + g;
-        const double v4[4] = {K0[r * Q0 + 8 * kk + tq], Kt0[r * Q0 + 8 * kk + tq], K0[r * Q0 + 8 * kk + tq + 4],
-                              Kt0[r * Q0 + 8 * kk + tq + 4]};
-        for (int q = 0; q < 4; ++q) host_tf32_split(v4[q], &t.fl[mt][kk][0][lane][q], &t.fl[mt][kk][1][lane][q]);
-      }
-  // xi B fragments: b0 = B[8kk+tq][8nn+g], b1 = B[8kk+tq+4][8nn+g], B[j'][2j+e] = (e ? Kt1 : K1)[j][j']
-  for (int kk = 0; kk < S::KKX; ++kk)
-    for (int nn = 0; nn < S::NN; ++nn)
-      for (int lane = 0; lane < 32; ++lane) {
-        const int g = lane >> 2, tq = lane & 3;
-        const int jj = 4 * nn + (g >> 1), e = g & 1;
-        const std::vector<double>& M = e ? Kt1 : K1;
-        for (int q = 0; q < 2; ++q) {
-          const int jp = 8 * kk + tq + 4 * q;
-          const double x = jp < Q1 ? M[jj * Q1 + jp] : 0.0;
-          host_tf32_split(x, &t.fx[kk][nn][0][lane][q], &t.fx[kk][nn][1][lane][q]);
-        }
-      }
   for (int k = 0; k < Q0; ++k) {
     t.p0[k] = real(m.p0[k]);
-    t.iw0[k] = real(m.iw0[k]);
     t.w0[k] = real(m.w0[k]);
-    for (int s = 0; s < MAXN; ++s) t.tab0[k * MAXN + s] = real(m.tab0[k * MAXN + s]);
+    t.sc0[k] = real(weno_pow2(m.iw0[k]));
+    t.isc0[k] = real(1) / t.sc0[k];
+    for (int s = 0; s <= m.N0; ++s) t.tab[s * (Q0 + Q1) + k] = real(m.tab0[k * MAXN + s]);
   }
   for (int k = 0; k < Q1; ++k) {
     t.p1[k] = real(m.p1[k]);
-    t.iw1[k] = real(m.iw1[k]);
     t.w1[k] = real(m.w1[k]);
-    for (int s = 0; s < MAXN; ++s) t.tab1[k * MAXN + s] = real(m.tab1[k * MAXN + s]);
+    t.sc1[k] = real(weno_pow2(m.iw1[k]));
+    t.isc1[k] = real(1) / t.sc1[k];
+    for (int s = 0; s <= m.N1; ++s) t.tab[s * (Q0 + Q1) + Q0 + k] = real(m.tab1[k * MAXN + s]);
   }
   // f_eq(1, 0, T0): factors and the incoming wall flux (the denominator of Eq. nw)
   double mv0[MAXN], mv1[MAXN], g0[Q0], g1[Q1];
@@ -383,26 +365,27 @@ static void fill_chan_tables(const AxisTables* ax, const ModelArgs& m, double T0
     t.ref_hi[k] = real(refs[k]);
     t.ref_lo[k] = real(refs[k] - double(t.ref_hi[k]));
   }
-  t.N0 = m.N0, t.N1 = m.N1, t.kind0 = m.kind0, t.kind1 = m.kind1;
+  t.ref_sum[0] = real(sizeof(real) == 4 ? m.ref_sum_f : m.ref_n);
+  t.ref_sum[1] = real(sizeof(real) == 4 ? m.ref_sum_f - double(t.ref_sum[0]) : 0.0);
+  t.nmax = std::max(m.N0, m.N1), t.kind1 = m.kind1;
 }
 
 template <typename real>
-bool channel_tables(int nq0, int nq1, const AxisTables* ax, const ModelArgs& m, double T0,
-                    std::vector<unsigned char>* out) {
-  if (nq0 == 16 && nq1 == 12) return fill_chan_tables<real, 16, 12>(ax, m, T0, out), true;
-  if (nq0 == 8 && nq1 == 4) return fill_chan_tables<real, 8, 4>(ax, m, T0, out), true;
+bool channel_tables(int nq0, int nq1, const ModelArgs& m, double T0, std::vector<unsigned char>* out) {
+  if (nq0 == 16 && nq1 == 12) return fill_chan_tables<real, 16, 12>(m, T0, out), true;
+  if (nq0 == 8 && nq1 == 4) return fill_chan_tables<real, 8, 4>(m, T0, out), true;
   return false;
 }
 
 template <typename real>
-cudaError_t launch_channel(ChanVariant v, const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int grid,
+cudaError_t launch_channel(const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int kind1, int grid,
                            cudaStream_t s, bool clb) {
-#define VLB_CH(q0, q1, TP_)                                                                  \
-  if (nq0 == q0 && nq1 == q1 && v.tp == TP_)                                                 \
-    return clb ? go_channel<real, q0, q1, TP_, false, true>(a, kp, grid, s)                  \
-               : (sizeof(real) == 4 && v.tc) ? go_channel<real, q0, q1, TP_, sizeof(real) == 4>(a, kp, grid, s) \
-                                             : go_channel<real, q0, q1, TP_, false>(a, kp, grid, s);
-  VLB_CH(16, 12, 4) VLB_CH(8, 4, 4) VLB_CH(8, 4, 8)
+#define VLB_CH(q0, q1)                                                                             \
+  if (nq0 == q0 && nq1 == q1)                                                                      \
+    return clb ? go_channel<real, q0, q1, true, false>(a, kp, grid, s)                             \
+               : kind1 == 1 ? go_channel<real, q0, q1, false, true>(a, kp, grid, s)                \
+                            : go_channel<real, q0, q1, false, false>(a, kp, grid, s);
+  VLB_CH(16, 12) VLB_CH(8, 4)
 #undef VLB_CH
   return cudaErrorInvalidValue;
 }
@@ -934,11 +917,11 @@ template cudaError_t launch_stage<VLB_REAL>(StageVariant, const StageArgs<VLB_RE
                                             const KArgs<VLB_REAL>&, int, cudaStream_t, bool);
 template cudaError_t launch_init_equilibrium<VLB_REAL>(VLB_REAL*, long long, int, const ModelArgs&, double, double,
                                                        double, double, cudaStream_t);
-template size_t channel_smem_bytes<VLB_REAL>(ChanVariant, int, int);
-template cudaError_t launch_channel<VLB_REAL>(ChanVariant, const ChanArgs<VLB_REAL>&, const void*, int, int, int,
+template size_t channel_smem_bytes<VLB_REAL>(ChanVariant, int, int, int*);
+template cudaError_t launch_channel<VLB_REAL>(const ChanArgs<VLB_REAL>&, const void*, int, int, int, int,
                                               cudaStream_t, bool);
-template bool channel_tables<VLB_REAL>(int, int, const AxisTables*, const ModelArgs&, double,
-                                       std::vector<unsigned char>*);
+template bool channel_force_pairs<VLB_REAL>(int, int, const AxisTables*, std::vector<unsigned char>*);
+template bool channel_tables<VLB_REAL>(int, int, const ModelArgs&, double, std::vector<unsigned char>*);
 template cudaError_t launch_seed<VLB_REAL>(VLB_REAL*, long long, int, const ModelArgs&, const double*,
                                            const double*, const double*, const double*, const double*, cudaStream_t,
                                            CellMap);

@@ -47,32 +47,30 @@ cudaError_t launch_stage(StageVariant v, const StageArgs<real>& a, const ModelAr
 
 // Launch shapes of the channel stage kernel: ts lambda rows per segment of a
 // CTA's march (0: chosen by the host from the SM count; at least n_lambda: one
-// segment), tp xi-columns per strip, nt threads ((tp + 1) x velocities).
+// segment), tp xi-columns per strip, nt threads (one per velocity).
 struct ChanVariant {
   int ts, tp, nt;
-  int tc;  // single precision: force contraction on the tensor cores (1) or the CUDA cores (0)
 };
 template <typename real>
 struct ChanArgs;
 
 // Channel launch shapes for a model shape (at most 8); 0 if the shape has no channel kernel.
 int channel_variants(int nq0, int nq1, ChanVariant* out);
+// Shared memory of a CTA and (per_sm) the CTAs a SM holds; 0 if the shape has no channel kernel.
 template <typename real>
-size_t channel_smem_bytes(ChanVariant v, int nq0, int nq1);
-// The ChanTables block of a model shape (bytes, bulk-copied by every CTA) for the
-// axis tables, the model arguments and the reservoir / wall temperature T0; false
-// if the shape has no channel kernel.
+size_t channel_smem_bytes(ChanVariant v, int nq0, int nq1, int* per_sm);
+// The ChanTables block of a model shape (bytes, copied by every CTA) for the model arguments
+// and the reservoir / wall temperature T0; false if the shape has no channel kernel.
 template <typename real>
-bool channel_tables(int nq0, int nq1, const AxisTables* ax, const ModelArgs& m, double T0,
-                    std::vector<unsigned char>* out);
-// One channel stage on `grid` CTAs (a.nx / v.tp strips x a.nseg segments).
-// The split force block (ChanKP) of a model shape from the full matrices of the two
-// axes; false if the shape has no channel kernel or a matrix lacks the reflection
-// symmetry the split relies on.
+bool channel_tables(int nq0, int nq1, const ModelArgs& m, double T0, std::vector<unsigned char>* out);
+// The force block (ChanKP) of a model shape from the full matrices of the two axes; false if
+// the shape has no channel kernel or a matrix lacks the structure the block relies on.
+template <typename real>
 bool channel_force_pairs(int nq0, int nq1, const AxisTables* ax, std::vector<unsigned char>* out);
+// One channel stage on `grid` CTAs (a.nx / tp strips x a.nseg segments); kind1: axis 1 is half range (1).
 // clb: the Cartesian-split formulation on the same march (a.geo then holds its geometry records)
 template <typename real>
-cudaError_t launch_channel(ChanVariant v, const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int grid,
+cudaError_t launch_channel(const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int kind1, int grid,
                            cudaStream_t s, bool clb = false);
 
 // Order of a context's cells in device buffers against the caller's order.
