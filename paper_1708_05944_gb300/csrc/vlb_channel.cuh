@@ -117,13 +117,17 @@ struct ChanArgs {
 // reconstruction and the combine, s+1 for the force, s+2 and s+3 for the lambda windows and the
 // moments, s+4 in flight (issued when step s begins, after the barrier that ends the use of row s-1).  Cells are padded so that the force tasks of neighbouring cells fall on consecutive
 // banks: cell stride = Q1 pairs modulo 128 bytes.
-template <typename real, int Q0, int Q1>
+//
+// XW: warps beside the NW that own velocities.  Small velocity sets (one warp) take three for the
+// roles of the rows ahead where the grid leaves SMs idle: a step then takes the time of its longest
+// part, not of their sum.
+template <typename real, int Q0, int Q1, int XW>
 struct ChanSmem {
   using S = ChanShape<Q0, Q1>;
   using Tab = ChanTables<real, Q0, Q1>;
   static constexpr bool F32 = sizeof(real) == 4;
   static constexpr int TP = S::TP;
-  static constexpr int NT = S::V;
+  static constexpr int NT = S::V + 32 * XW;
   static constexpr int NRING = 5;
   static constexpr int RC = TP + 6;  // cells of a ring row
   static constexpr int NEQ = 4;      // equilibrium records (rows s .. s+3)
@@ -155,32 +159,6 @@ struct ChanSmem {
   static constexpr int fit = int((228 * 1024) / (bytes + 1024));
   static constexpr int min_ctas = sizeof(real) == 8 ? 1 : (fit * NT * 168 <= 65536 ? fit : 65536 / (NT * 168));
 };
-
-// Moment vector of the truncated equilibrium on one axis (the recurrences of eq_moment_vector),
-// every entry up to order nmax, with the 1/l factors as constants and one reciprocal of T.
-template <typename R>
-__device__ __forceinline__ void eq_moments_fast(int kind, int nmax, R u, R T, R* m) {
-  R a, b, c;  // m_l = (u m_{l-1} + h c m_{l-2}) f: h = 1, f = 1 / l (full range) or h = l - 1, f = 1
-  if (kind == 0) {
-    a = R(1), b = u, c = T - R(1);
-  } else {
-    const R is2T = rsqrt_t(R(2) * T);
-    const R x = u * is2T;
-    const R g0 = exp_t(-x * x) * is2T * R(0.56418958354775628695);  // N(0; u, T) = e^.. / sqrt(2 pi T)
-    a = R(0.5) * (R(1) + erf_t<R>(x));
-    b = u * a + T * g0, c = T;
-  }
-  m[0] = a;
-  m[1] = b;
-#pragma unroll
-  for (int l = 2; l < MAXN; ++l) {
-    if (l > nmax) break;
-    const R x = (u * b + (kind == 0 ? R(1) : R(l - 1)) * c * a) * (kind == 0 ? R(1.0 / l) : R(1));
-    m[l] = x;
-    a = b;
-    b = x;
-  }
-}
 
 // Coefficients of a packed contraction: single precision holds each duplicated into a pair, the
 // operand of a packed fma over (f', f''); double precision holds them once.
@@ -374,17 +352,19 @@ __device__ __forceinline__ void channel_equilibrium(const ChanTables<real, Q0, Q
 // (c = 0).  The lambda upwind side and the wall's incoming half-plane (Eq. canalie_coord_nw)
 // then depend on the column and the interface: the lambda window holds the six cells around an
 // interface and the walk's terms are formed per interface from the five of the upwind side.
-template <typename real, int Q0, int Q1, bool CLB, bool HX>
-__global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0, Q1>::min_ctas)
+template <typename real, int Q0, int Q1, int XW, bool CLB, bool HX>
+__global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real, Q0, Q1, XW>::min_ctas)
     channel_stage_kernel(const __grid_constant__ ChanArgs<real> a, const __grid_constant__ ChanKP<real, Q0, Q1> kp) {
   using S = ChanShape<Q0, Q1>;
-  using L = ChanSmem<real, Q0, Q1>;
+  using L = ChanSmem<real, Q0, Q1, XW>;
   using Tab = ChanTables<real, Q0, Q1>;
   using P = pair_t<real>;
   constexpr int V = S::V, ROW = S::ROW, EQW = S::EQW, TP = S::TP, NW = S::NW;
   constexpr int NRING = L::NRING, RC = L::RC, CS = L::CS, XS = L::XS;
   extern __shared__ __align__(128) unsigned char smem[];
-  const int v = threadIdx.x, lane = v & 31, warp = v >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool col = XW == 0 || tid < V;  // owns a velocity of the four columns
+  const int v = col ? tid : lane;
   const int i = v / Q1, j = v - i * Q1;
 
   const int nl = a.nl, nx = a.nx;
@@ -428,14 +408,14 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
   auto row_wait = [&](int r) -> bool { return mbar_wait(bar + slot(r), unsigned((r - sA) / NRING) & 1u, a.max_polls); };
 
   // ---- prologue: tables and rows sA .. sA+3
-  if (v == 0) {
+  if (tid == 0) {
     for (int k = 0; k < NRING; ++k) mbar_init(bar + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   {
     const uint4* src = reinterpret_cast<const uint4*>(a.tables);
     uint4* dst = reinterpret_cast<uint4*>(smem + L::tab_off);
-    for (int x = v; x < int(sizeof(Tab) / 16); x += V) dst[x] = src[x];
+    for (int x = tid; x < int(sizeof(Tab) / 16); x += L::NT) dst[x] = src[x];
   }
   __syncthreads();
   if (warp == 0)
@@ -458,7 +438,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
   bool good = true;  // every wait of this thread so far ended in time
   // a wait ran out: let the copies in flight land (bounded), then leave together
   auto give_up = [&]() {
-    if (v == 0) {
+    if (tid == 0) {
       atomicOr(a.err, ERR_TIMEOUT);
       for (int r = max(sA, issued - NRING + 1); r <= issued; ++r) row_wait(r);
     }
@@ -470,9 +450,13 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
     return;
   }
 
-  // ---- the roles of the rows ahead.  With at least six warps: warps 0 and 1 contract along
-  // lambda, 2 and 3 along xi, 4 takes the equilibria, 5 the inflow factors; fewer take all in turn.
+  // ---- the roles of the rows ahead, by warp: with six warps, 0 and 1 contract along lambda, 2 and 3
+  // along xi, 4 takes the equilibria, 5 the inflow factors; with extra warps they share the same;
+  // else the one warp takes all in turn.
   constexpr bool SPLIT = NW >= 6;
+  static_assert(XW == 0 || XW == 3, "extra warps: lambda, xi, equilibria and inflow");
+  constexpr int WL = SPLIT ? 0 : XW ? NW : 0, WX = SPLIT ? 2 : XW ? NW + 1 : 0, WE = SPLIT ? 4 : XW ? NW + 2 : 0,
+                WR = SPLIT ? 5 : WE, FW = SPLIT ? 2 : 1;  // their first warps; warps of a contraction
   auto force_row = [&](int r) {
     if constexpr (!CLB) {
       const int k = slot(r);
@@ -480,8 +464,8 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
       real* ox = lbx + (r & 1) * TP * Q0 * XS;
       // Eq. (canalie_boltz): G_lxx (p^xi)^2 K0 f + G_lxl p^xi Kt0 f along lambda,
       // -G_lxl (p^lambda)^2 K1 f - G_lxx p^lambda Kt1 f along xi
-      if (!SPLIT || warp < 2)
-        for (int t = v; t < TP * Q1; t += SPLIT ? 64 : V) {
+      if (warp >= WL && warp < WL + FW)
+        for (int t = tid - 32 * WL; t < TP * Q1; t += 32 * FW) {
           const int cc = t / Q1, jj = t - cc * Q1;
           const ChanCell<real>& g = gring[k * TP + cc];
           const real pj = tb.p1[jj];
@@ -490,8 +474,8 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
           force_line<real, Q0 / 2, true>(kp.P0, kp.M0, kp.p0, kp.v0, kp.z0, F, F + Q0 * Q1, 2 * Q1, 2 * Q1,
                                          g.glxx * pj * pj, g.glxl * pj, O, O + Q0 * Q1, 2 * Q1, 2 * Q1);
         }
-      if (!SPLIT || (warp & ~1) == 2)
-        for (int t = SPLIT ? v - 64 : v; t < TP * Q0; t += SPLIT ? 64 : V) {
+      if (warp >= WX && warp < WX + FW)
+        for (int t = tid - 32 * WX; t < TP * Q0; t += 32 * FW) {
           const int cc = t / Q0, ii = t - cc * Q0;
           const ChanCell<real>& g = gring[k * TP + cc];
           const real pi = tb.p0[ii];
@@ -504,7 +488,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
     }
   };
   auto eq_row = [&](int r) {
-    if (warp != (SPLIT ? 4 : 0)) return;
+    if (warp != WE) return;
     const int cc = lane >> 3;
     channel_equilibrium<real, Q0, Q1>(tb, cell(slot(r), cc), mvs + cc * 4 * MAXN,
                                       eqr + ((r & (L::NEQ - 1)) * TP + cc) * EQW, a.ikn);
@@ -550,7 +534,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
     }
   };
   auto res_row = [&](int r) {
-    if (!(inlet || outlet) || warp != (SPLIT ? 5 : 0)) return;
+    if (!(inlet || outlet) || warp != WR) return;
 #pragma unroll 1
     for (int end = 0; end < 2; ++end)
       if (end == 0 ? inlet : outlet) res_job(r, end);
@@ -590,6 +574,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
   WenoWin<real, !L::F32> win[CLB ? 1 : TP];
   P raw[CLB ? TP : 1][6];
   P flo[TP];  // lambda interface s - 1/2 (scaled)
+  if (col)
 #pragma unroll
   for (int c = 0; c < TP; ++c) {
     if constexpr (CLB) {
@@ -636,6 +621,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
   // The wall's n_w, and its ghost rows into the ring slots of rows nl and nl + 1 (rows nl-5 and
   // nl-4 have left them; row nl + 2 reads as nl + 1): each thread its own velocity
   auto wall_density = [&]() {
+    if (col)
 #pragma unroll 1
     for (int c = 0; c < TP; ++c) {
       real fl = real(0), fd = real(0);
@@ -665,7 +651,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
       if (lane == 0) wred[c * NW + warp] = fl, wred[(TP + c) * NW + warp] = fd;
     }
     __syncthreads();
-    if (v < TP) {
+    if (tid < TP) {
       double num = CLB ? 0.0 : tb.ref_flux_pos;  // vielbein: the outgoing flux of R, then of D
       double den = CLB ? 0.0 : tb.wall_den;
       for (int w = 0; w < NW; ++w) {
@@ -678,6 +664,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
       if (!isfinite(nwc)) atomicOr(a.err, ERR_NONFINITE);
     }
     __syncthreads();
+    if (col)
 #pragma unroll 1
     for (int c = 0; c < TP; ++c) {
       P G1, G2;
@@ -700,7 +687,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
 #pragma unroll
   for (int c = 0; c < TP; ++c) {
     flr[c] = p_set(real(0));
-    if (need_fl) flr[c] = p_load(Fl + c * ROW);
+    if (need_fl && col) flr[c] = p_load(Fl + c * ROW);
   }
   __syncthreads();
 
@@ -713,6 +700,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
     if (full && warp == 0 && s + 4 <= rlast) row_issue(s + 4);
     if (s > sA && s + 3 <= rlast) good = row_wait(s + 3) && good;
     if (s == nl - 3) wall_density();
+    if (col) {
     const int k0 = full ? slot(s) : 0;
     const int k3 = slot(min(s + 2 + (CLB ? 1 : off), nl + 1));  // the row that joins the lambda windows
     const ChanCell<real>* geo = gring + k0 * TP;
@@ -844,12 +832,13 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1>::NT, ChanSmem<real, Q0,
 #pragma unroll
     for (int c = 0; c < TP; ++c) flo[c] = fhi[c];
     }
+    }
     // ---- the rows ahead
     if (s + 3 < sB) eq_row(s + 3);
     if (s + 2 >= sA && s + 2 < sB) res_row(s + 2);
     if (s + 1 >= sA && s + 1 < sB) {
       force_row(s + 1);
-      if (inlet || outlet) fill_ghosts(s + 1);
+      if (col && (inlet || outlet)) fill_ghosts(s + 1);
     }
     if (!__syncthreads_and(good)) {
       give_up();

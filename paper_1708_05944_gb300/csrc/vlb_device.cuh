@@ -369,6 +369,14 @@ inline double weno_pow2(double inv_w) {
   return ldexp(1.0, e);
 }
 
+// The same from 1 / w on the device, at most 2^62 (a product of two axes' stays in single precision)
+__device__ __forceinline__ float weno_pow2_dev(float inv_w) {
+  return fminf(__int_as_float(__float_as_int(inv_w) & 0x7f800000), 4.6116860e18f);
+}
+__device__ __forceinline__ double weno_pow2_dev(double inv_w) {
+  return __hiloint2double(__double2hiint(inv_w) & 0x7ff00000, 0);
+}
+
 // 2^-e with e the exponent of x >= 0 (0, Inf and the top binade give values the caller's test
 // of the weight sum rejects)
 __device__ __forceinline__ float inv_pow2(float x) {
@@ -532,6 +540,14 @@ struct WenoWin {
     weno_corr<real, false>(terms(), sm, sm, sm, w, den);
     return weno_in_range(den);
   }
+  // the value, checked at once
+  __device__ __forceinline__ P face_checked(const WenoSide<real>& w) const {
+    P den, corr;
+    if constexpr (K) corr = weno_corr<real, true>(terms(), km, k0, kp, w, den);
+    else corr = weno_corr<real, false>(terms(), sm, sm, sm, w, den);
+    if (__builtin_expect(!weno_in_range(den), 0)) corr = weno_corr_slow<real>(terms(), w.hs.x > real(0));
+    return p_add(g0, corr);
+  }
   // the value in any case
   __device__ __forceinline__ P face_any(bool up) const { return p_add(g0, weno_corr_slow<real>(terms(), up)); }
 };
@@ -570,6 +586,32 @@ __device__ __forceinline__ void eq_moment_vector(int kind, int N, R u, R T, R* m
   }
 }
 
+// Moment vector of the truncated equilibrium on one axis (the recurrences of eq_moment_vector),
+// every entry up to order nmax, with the 1/l factors as constants and one reciprocal of T.
+template <typename R>
+__device__ __forceinline__ void eq_moments_fast(int kind, int nmax, R u, R T, R* m) {
+  R a, b, c;  // m_l = (u m_{l-1} + h c m_{l-2}) f: h = 1, f = 1 / l (full range) or h = l - 1, f = 1
+  if (kind == 0) {
+    a = R(1), b = u, c = T - R(1);
+  } else {
+    const R is2T = rsqrt_t(R(2) * T);
+    const R x = u * is2T;
+    const R g0 = exp_t(-x * x) * is2T * R(0.56418958354775628695);  // N(0; u, T) = e^.. / sqrt(2 pi T)
+    a = R(0.5) * (R(1) + erf_t<R>(x));
+    b = u * a + T * g0, c = T;
+  }
+  m[0] = a;
+  m[1] = b;
+#pragma unroll
+  for (int l = 2; l < MAXN; ++l) {
+    if (l > nmax) break;
+    const R x = (u * b + (kind == 0 ? R(1) : R(l - 1)) * c * a) * (kind == 0 ? R(1.0 / l) : R(1));
+    m[l] = x;
+    a = b;
+    b = x;
+  }
+}
+
 // Rescale the axis-0 equilibrium factor (which carries n) so that the stored
 // factors reproduce the cell density exactly: sum_i gn_i sum_j g1_j = n.  In
 // exact arithmetic the truncated equilibrium already has this sum (Sec. IV.D);
@@ -583,6 +625,13 @@ __device__ __forceinline__ void normalise_equilibrium(R* gn, const R* g1, int nq
   for (int k = 0; k < nq1; ++k) s1 += double(g1[k]);
   const R sc = R(n / (s0 * s1));
   for (int k = 0; k < nq0; ++k) gn[k] *= sc;
+}
+
+// 1 / tau of the same conventions, ikn = 1 / Kn
+template <typename R>
+__device__ __forceinline__ R relaxation_rate(int mode, R ikn, R n, R T) {
+  const R r = n * ikn;
+  return mode == 0 ? r * T : mode == 1 ? r * R(1.5957691216057307117) : r;  // sqrt(8 / pi)
 }
 
 template <typename R>

@@ -205,10 +205,10 @@ cudaError_t stage_config(StageVariant v, const ModelArgs& m, int Vp, int* nbuf, 
 }
 
 // ---------------------------------------------------------------- channel dispatch
-template <typename real, int Q0, int Q1, bool CLB, bool HX>
+template <typename real, int Q0, int Q1, int XW, bool CLB, bool HX>
 static cudaError_t go_channel(const ChanArgs<real>& a, const void* kpb, int grid, cudaStream_t s) {
-  using L = ChanSmem<real, Q0, Q1>;
-  auto kern = channel_stage_kernel<real, Q0, Q1, CLB, HX>;
+  using L = ChanSmem<real, Q0, Q1, XW>;
+  auto kern = channel_stage_kernel<real, Q0, Q1, XW, CLB, HX>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(L::bytes));
   if (e != cudaSuccess) return e;
   ChanKP<real, Q0, Q1> kp;
@@ -304,8 +304,8 @@ bool channel_force_pairs(int nq0, int nq1, const AxisTables* ax, std::vector<uns
 
 template <typename real>
 size_t channel_smem_bytes(ChanVariant, int nq0, int nq1, int* per_sm) {
-  if (nq0 == 16 && nq1 == 12) return *per_sm = ChanSmem<real, 16, 12>::min_ctas, ChanSmem<real, 16, 12>::bytes;
-  if (nq0 == 8 && nq1 == 4) return *per_sm = ChanSmem<real, 8, 4>::min_ctas, ChanSmem<real, 8, 4>::bytes;
+  if (nq0 == 16 && nq1 == 12) return *per_sm = ChanSmem<real, 16, 12, 0>::min_ctas, ChanSmem<real, 16, 12, 0>::bytes;
+  if (nq0 == 8 && nq1 == 4) return *per_sm = ChanSmem<real, 8, 4, 0>::min_ctas, ChanSmem<real, 8, 4, 0>::bytes;
   return 0;
 }
 
@@ -380,12 +380,17 @@ bool channel_tables(int nq0, int nq1, const ModelArgs& m, double T0, std::vector
 template <typename real>
 cudaError_t launch_channel(const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int kind1, int grid,
                            cudaStream_t s, bool clb) {
-#define VLB_CH(q0, q1)                                                                             \
-  if (nq0 == q0 && nq1 == q1)                                                                      \
-    return clb ? go_channel<real, q0, q1, true, false>(a, kp, grid, s)                             \
-               : kind1 == 1 ? go_channel<real, q0, q1, false, true>(a, kp, grid, s)                \
-                            : go_channel<real, q0, q1, false, false>(a, kp, grid, s);
-  VLB_CH(16, 12) VLB_CH(8, 4)
+#define VLB_CH(q0, q1, xw)                                                                  \
+  return clb ? go_channel<real, q0, q1, xw, true, false>(a, kp, grid, s)                    \
+             : kind1 == 1 ? go_channel<real, q0, q1, xw, false, true>(a, kp, grid, s)       \
+                          : go_channel<real, q0, q1, xw, false, false>(a, kp, grid, s);
+  if (nq0 == 16 && nq1 == 12) VLB_CH(16, 12, 0)
+  // one-warp velocity set: extra warps while every CTA with them is resident at once (16 x 128
+  // cells, 12 steps: 812 us against 929 with one warp); beyond that more CTAs of one warp fill the SMs
+  if (nq0 == 8 && nq1 == 4) {
+    if (grid <= 152 * ChanSmem<real, 8, 4, 3>::min_ctas) VLB_CH(8, 4, 3)
+    VLB_CH(8, 4, 0)
+  }
 #undef VLB_CH
   return cudaErrorInvalidValue;
 }
