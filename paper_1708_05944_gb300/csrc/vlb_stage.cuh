@@ -13,6 +13,12 @@
 // Every distribution buffer holds the deviation D = F - R from the rest state
 // (ModelArgs): the operator is linear in R's part, which it leaves unchanged.
 // A cell row holds Vp velocity pairs (f', f'') interleaved (see pair_t).
+//
+// What bounds it: issue slots and latency (48 % of the issue slots, 35 % of the FP32 pipe, 20 warps
+// a SM).  The walk of phase D takes WENO-5 on shared differences (WenoWin), phase A sums a row of
+// nodes per lane: 285 -> 236 instructions per warp and cell-velocity row.  Single precision, 16 x
+// 20 velocities, a step: 256 instances of 64 .. 1024 cells 1.90 -> 1.57 ms, 5 x 1024 cells 89 ->
+// 76 us; double precision 5 x 1024 cells 2.6 -> 2.3 ms.
 #pragma once
 #include <type_traits>
 
@@ -67,7 +73,7 @@ struct StageSmem {
   // doubles: p0, p1 (MAXQ each), reduction (NW*4), wall equilibrium factors (2*MAXQ), scalars (16)
   static constexpr size_t n_dbl = 2 * MAXQ + NW * 4 + 2 * MAXQ + 16;
   __host__ __device__ static size_t real_off(int Vp, int nbuf) { return dbl_off(Vp, nbuf) + n_dbl * sizeof(double); }
-  // reals: p0, p1, 1/w0, 1/w1 (MAXQ each), tab0, tab1 (MAXQ*MAXN each), then pairs: n g_R and g_phi
+  // reals: p0, p1, the two WENO scales (MAXQ each), tab0, tab1 (MAXQ*MAXN each), then pairs: n g_R and g_phi
   // (TC*MAXQ each), (1, T), -1/tau, cp, -cm, 1/Rbar (TC each); then moment vectors (TC*4*MAXN),
   // w0, w1 (MAXQ each)
   static constexpr size_t n_real = 4 * MAXQ + 2 * MAXQ * MAXN + 4 * TC * MAXQ + 10 * TC + TC * 4 * MAXN + 2 * MAXQ;
@@ -117,9 +123,9 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
   double* mw = gw1 + MAXQ;     // [0] incoming equilibrium flux, [1] n_w
   real* p0r = reinterpret_cast<real*>(smem + L::real_off(Vp, nbuf));
   real* p1r = p0r + MAXQ;
-  real* iw0 = p1r + MAXQ;  // 1 / w_i
-  real* iw1 = iw0 + MAXQ;  // 1 / w_j
-  real* tabr0 = iw1 + MAXQ;  // equilibrium tables in the bulk type
+  real* iw0 = p1r + MAXQ;  // powers of two next to 1 / w_i and 1 / w_j: the scale of the WENO walk
+  real* iw1 = iw0 + MAXQ;
+  real* tabr0 = iw1 + MAXQ;  // equilibrium tables in the bulk type, [s][k]
   real* tabr1 = tabr0 + MAXQ * MAXN;
   // per-cell values of phase D as ready pairs (both lanes of a packed operand)
   using P2 = pair_t<real>;
@@ -146,22 +152,23 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     if constexpr (F32) {
       p0r[x] = m.p0f[x];
       p1r[x] = m.p1f[x];
-      iw0[x] = m.iw0f[x];
-      iw1[x] = m.iw1f[x];
+      iw0[x] = x < nq0 ? weno_pow2_dev(m.iw0f[x]) : 1.0f;
+      iw1[x] = x < nq1 ? weno_pow2_dev(m.iw1f[x]) : 1.0f;
       w0r[x] = m.w0f[x];
       w1r[x] = m.w1f[x];
     } else {
       p0r[x] = m.p0[x];
       p1r[x] = m.p1[x];
-      iw0[x] = m.iw0[x];
-      iw1[x] = m.iw1[x];
+      iw0[x] = x < nq0 ? weno_pow2_dev(m.iw0[x]) : 1.0;
+      iw1[x] = x < nq1 ? weno_pow2_dev(m.iw1[x]) : 1.0;
       w0r[x] = m.w0[x];
       w1r[x] = m.w1[x];
     }
   }
   for (int x = tid; x < MAXQ * MAXN; x += NT) {
-    tabr0[x] = sizeof(real) == 4 ? real(m.tab0f[x]) : real(m.tab0[x]);
-    tabr1[x] = sizeof(real) == 4 ? real(m.tab1f[x]) : real(m.tab1[x]);
+    const int y = (x % MAXN) * MAXQ + x / MAXN;
+    tabr0[y] = sizeof(real) == 4 ? real(m.tab0f[x]) : real(m.tab0[x]);
+    tabr1[y] = sizeof(real) == 4 ? real(m.tab1f[x]) : real(m.tab1[x]);
   }
   __syncthreads();
   const bool need_fl = a.caf != 0.0f;
@@ -226,15 +233,35 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     const int t = has ? tc : TCe - 1;  // it repeats the lower half's and writes nothing
     const real* F = tile + (t + 3) * row;
     real sn = 0, sr = 0, sp = 0, se = 0;  // per-lane partial sums over a sixteenth of the velocities
+    if constexpr (EXACT && 16 % Q0MAX == 0 && Q1MAX % (32 / Q0MAX) == 0) {
+      // lane hl sums the nodes j of row i = hl mod Q0 (all, or its share of them): the p^phi weights
+      // are uniform operands and p^R enters once (a third of the instructions of the general form)
+      constexpr int JN = Q1MAX * Q0MAX / 16;
+      const int jb = (hl / Q0MAX) * JN;
+      const real* f = F + 2 * ((hl % Q0MAX) * Q1MAX + jb);
+      const real pr = p0r[hl % Q0MAX];
+#pragma unroll
+      for (int j = 0; j < JN; j += 2) {
+        const pair_t<real> f0 = p_load(f + 2 * j), f1 = p_load(f + 2 * j + 2);
+        const real pa = JN == Q1MAX ? (F32 ? real(m.p1f[j]) : real(m.p1[j])) : p1r[jb + j];
+        const real pb = JN == Q1MAX ? (F32 ? real(m.p1f[j + 1]) : real(m.p1[j + 1])) : p1r[jb + j + 1];
+        const real ta = pa * f0.x, tb = pb * f1.x;
+        sn += f0.x, sp += ta, se += pa * ta + f0.y;
+        sn += f1.x, sp += tb, se += pb * tb + f1.y;
+      }
+      sr = pr * sn;
+      se += pr * sr;
+    } else {
 #pragma unroll 4
-    for (int v = hl; v < V; v += 16) {
-      const int i = v / nq1, j = v - i * nq1;
-      const pair_t<real> f = p_load(F + 2 * v);
-      const real f1 = f.x, f2 = f.y, pr = p0r[i], pp = p1r[j];
-      sn += f1;
-      sr += pr * f1;
-      sp += pp * f1;
-      se += (pr * pr + pp * pp) * f1 + f2;
+      for (int v = hl; v < V; v += 16) {
+        const int i = v / nq1, j = v - i * nq1;
+        const pair_t<real> f = p_load(F + 2 * v);
+        const real f1 = f.x, f2 = f.y, pr = p0r[i], pp = p1r[j];
+        sn += f1;
+        sr += pr * f1;
+        sp += pp * f1;
+        se += (pr * pr + pp * pp) * f1 + f2;
+      }
     }
     // sums over the half-warp; then the sums of D plus those of R and the derived fields
     real nn, u0, u1, T;
@@ -252,25 +279,27 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       float nh, nl;
       two_sum(sn, m.ref_nf[0], nh, nl);
       nn = nh + (nl + (en + m.ref_nf[1]));
-      const float inv = 1.0f / nn;
+      const float inv = rcp_rn(nn);
       u0 = (sr + (er + m.ref_rf)) * inv;
       u1 = (sp + (ep + m.ref_pf)) * inv;
       T = ((se + (ee + m.ref_ef)) * inv - (u0 * u0 + u1 * u1)) * (1.0f / 3.0f);
     } else {
       dn = half_sum(double(sn));
       const double dr = half_sum(double(sr)), dpp = half_sum(double(sp)), de = half_sum(double(se));
-      nn = real(dn + m.ref_n), u0 = real(dr + m.ref_r) / nn, u1 = real(dpp + m.ref_p) / nn;
-      T = (real(de + m.ref_e) - nn * (u0 * u0 + u1 * u1)) / (real(3) * nn);
+      nn = real(dn + m.ref_n);
+      const real inv = rcp_rn(nn);
+      u0 = real(dr + m.ref_r) * inv, u1 = real(dpp + m.ref_p) * inv;
+      T = (real(de + m.ref_e) * inv - (u0 * u0 + u1 * u1)) * (real(1) / real(3));
     }
     if (hl == 0 && has) {
       cT1[t] = p_make(real(1), T);
-      cNtau[t] = p_set(-(real(1) / relaxation_time<real>(in.tau_mode, F32 ? real(in.kn_f) : real(in.kn), nn, T)));
+      cNtau[t] = p_set(-relaxation_rate<real>(in.tau_mode, rcp_rn(F32 ? real(in.kn_f) : real(in.kn)), nn, T));
     }
     real* mt = mv + t * 4 * MAXN;  // moment vectors [axis * 2 + side][s]
     if (hl < 4 && has) {
       const int ax = hl >> 1, side = hl & 1;
       const real u = (ax ? u1 : u0) * (side ? real(-1) : real(1));
-      eq_moment_vector<real>(ax ? m.kind1 : m.kind0, ax ? m.N1 : m.N0, u, T, mt + hl * MAXN);
+      eq_moments_fast<real>(ax ? m.kind1 : m.kind0, ax ? m.N1 : m.N0, u, T, mt + hl * MAXN);
     }
     __syncwarp();
     // equilibrium factors: lane hl takes g_R[k] and g_phi[k] for k = hl and hl + 16
@@ -280,12 +309,12 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       const int k = hl + 16 * q;
       if (16 * q < Q0MAX && k < nq0) {
         const real* mm = mt + ((m.kind0 == 1 && p0r[k] < real(0)) ? 1 : 0) * MAXN;
-        for (int s2 = 0; s2 <= m.N0; ++s2) gr[q] += tabr0[k * MAXN + s2] * mm[s2];
+        for (int s2 = 0; s2 <= m.N0; ++s2) gr[q] += tabr0[s2 * MAXQ + k] * mm[s2];
         gr[q] *= nn;
       }
       if (16 * q < Q1MAX && k < nq1) {
         const real* mm = mt + (2 + ((m.kind1 == 1 && p1r[k] < real(0)) ? 1 : 0)) * MAXN;
-        for (int s2 = 0; s2 <= m.N1; ++s2) gp[q] += tabr1[k * MAXN + s2] * mm[s2];
+        for (int s2 = 0; s2 <= m.N1; ++s2) gp[q] += tabr1[s2 * MAXQ + k] * mm[s2];
       }
     }
     // rescale g_R so that sum_i g_R sum_j g_phi is exactly the target sum D + sum R (f_eq - R
@@ -305,7 +334,7 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       float th, tl;
       two_sum(sn, m.ref_sumf[0], th, tl);
       tl = tl + (en + m.ref_sumf[1]);
-      delta = (__fsub_rn(Ah, th) + (Al - tl)) / Ah;
+      delta = (__fsub_rn(Ah, th) + (Al - tl)) * rcp_rn(Ah);
       scale0 = real(0);
     } else {
       const double a0 = half_sum(double(gr[0]) + double(gr[1])), a1 = half_sum(double(gp[0]) + double(gp[1]));
@@ -548,7 +577,15 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       }
       const pair_t<real> G0 = p_fma(F1, p_set(real(-3)), p_fma(F0, p_set(real(3)), F2));
       const pair_t<real> G1 = p_fma(F1, p_set(real(-8)), p_fma(F0, p_set(real(6)), p_mul(F2, p_set(real(3)))));
-      num += double(weno5p<real>(F2, F1, F0, G0, G1, iw0[i] * iw1[j]).x) * p0d[i];
+      // (bit for bit phase D's value: the same cell, side and order)
+      const real sc = iw0[i] * iw1[j];
+      const pair_t<real> SC = p_set(sc);
+      WenoWin<real, false> w;
+      WenoSide<real> ws;
+      ws.set(wall != 0);
+      w.start(p_mul(wall ? F2 : G1, SC), p_mul(wall ? F1 : G0, SC), p_mul(F0, SC), p_mul(wall ? G0 : F1, SC),
+              p_mul(wall ? G1 : F2, SC));
+      num += double(w.face_checked(ws).x * rcp_rn(sc)) * p0d[i];
     }
     num = warp_sum<real>(num);
     if (lane == 0) red[warp] = num;
@@ -620,22 +657,26 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     const bool up = pr >= real(0);
     const real sc = iw0[i] * iw1[j];
     const P nrij = p_set(-(w0r[i] * w1r[j]));
-    const P npr = p_set(-pr);
+    const P SC = p_set(sc);
+    const P npr = p_set(-pr * rcp_rn(sc));  // interface values carry the scale sc (a power of two)
+    WenoSide<real> side;
+    side.set(up);
     real* S = tile + 2 * v;
     const real* Fl = a.Fl + size_t(in.cell0 + c0) * row + 2 * v;  // F_l of the owned cells, read once
-    // the advected value of slot q: D (chi), F~ - R = (D + R) sqrt(g) - R (f~)
+    // the advected value of slot q, scaled: D (chi), F~ - R = (D + R) sqrt(g) - R (f~)
     const real Rr = w0r[i] * w1r[j];
-    auto adv_val = [&](const real* x, int q) -> P {
-      if constexpr (FT) return p_fma(p_load(x), p_set(sgs[q]), p_set(Rr * (sgs[q] - real(1))));
-      else return p_load(x);
+    auto adv_val = [&](int q) -> P {
+      const P x = p_load(S + q * row);
+      if constexpr (FT) return p_mul(p_fma(x, p_set(sgs[q]), p_set(Rr * (sgs[q] - real(1)))), SC);
+      else return p_mul(x, SC);
     };
     P FRv = p_set(real(0));  // f~: the inertial term of R for this velocity
     if constexpr (FT) FRv = p_set(a.forceR[v]);
-    P w0 = adv_val(S, 0), w1 = adv_val(S + row, 1), w2 = adv_val(S + 2 * row, 2), w3 = adv_val(S + 3 * row, 3);
-    P w4 = adv_val(S + 4 * row, 4), w5 = adv_val(S + 5 * row, 5);
-    // upwind stencil: (w0..w4) for p^R >= 0, mirrored (w5..w1) otherwise
-    P fm = weno5p<real>(p_sel(up, w0, w5), p_sel(up, w1, w4), p_sel(up, w2, w3), p_sel(up, w3, w2),
-                        p_sel(up, w4, w1), sc);
+    // the upwind cell of interface s + 1/2 is s for p^R >= 0, s + 1 otherwise: the walk runs one cell ahead
+    const int o = up ? 0 : 1;
+    WenoWin<real, true> win;
+    win.start(adv_val(o), adv_val(o + 1), adv_val(o + 2), adv_val(o + 3), adv_val(o + 4));
+    P fm = win.face_checked(side);
     // F_l of the next cell is loaded one cell ahead (a global load, the only one of the walk)
     P fl_next = need_fl ? p_load(Fl) : p_set(real(0));
 #pragma unroll
@@ -643,16 +684,12 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       if (t < TCe) {
         const P fl = fl_next;
         if (need_fl && t + 1 < TCe) fl_next = p_load(Fl + (t + 1) * row);
-        const P w6 = adv_val(S + (t + 6) * row, t + 6);
-        const P fp = weno5p<real>(p_sel(up, w1, w6), p_sel(up, w2, w5), p_sel(up, w3, w4), p_sel(up, w4, w3),
-                                  p_sel(up, w5, w2), sc);
+        win.push(adv_val(t + 5 + o));
+        const P fp = win.face_checked(side);
         // -adv = -p^R (cp F_{s+1/2} - cm F_{s-1/2}); per-cell factors: shared-memory broadcasts
         P nadv = p_mul(p_fma(fp, ccp[t], p_mul(fm, cNcm[t])), npr);
-        P Dc = w3;  // the cell's D
-        if constexpr (FT) {
-          nadv = p_fma(p_mul(npr, p_set(Rr)), p_add(ccp[t], cNcm[t]), nadv);  // the advection of R
-          Dc = p_load(S + (t + 3) * row);
-        }
+        const P Dc = p_load(S + (t + 3) * row);  // the cell's D
+        if constexpr (FT) nadv = p_fma(p_set(-pr * Rr), p_add(ccp[t], cNcm[t]), nadv);  // the advection of R
         // f_eq - R for both fields: (g, T g) - R
         const P deq = p_fma(p_mul(gRn[t * MAXQ + i], gP[t * MAXQ + j]), cT1[t], nrij);
         P force = p_load(lbuf + t * row + 2 * v);
@@ -662,12 +699,6 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
         P o = p_fma(Lv, p_set(cc), Dc);
         if (need_fl) o = p_fma(p_sub(fl, Dc), p_set(ca), o);
         p_store(S + (t + 3) * row, o);  // in place: this column's slot t+3 is not read again
-        w0 = w1;
-        w1 = w2;
-        w2 = w3;
-        w3 = w4;
-        w4 = w5;
-        w5 = w6;
         fm = fp;
       }
     }
