@@ -186,28 +186,33 @@ namespace {
 // the tile list in rounds of `slots` CTAs, so the tile size s <= TC is chosen to
 // minimise rounds x (s + 3): the makespan in cell-times with the three halo
 // cells as the fixed cost of a tile (for 5 x 1024 cells on 456 CTAs: 6-cell
-// tiles in two rounds instead of 8-cell tiles in two).  CTA b takes the tiles
-// b, b + slots, ...; when the last round is not full, the tiles that reach a
-// wall (and so also fill its ghost cells, several times the work of an interior
-// tile's phase in between) are placed in the first round of the CTAs that have
-// no tile in the last round.
+// tiles in two rounds instead of 8-cell tiles in two).  Either takes smaller tiles
+// while they come to no more than one per SM: a stage is then the latency of its tile,
+// which grows with its cells (32 cells x 32 velocities in double precision, 12 steps:
+// 2215 us with tiles of eight, 900 us with one cell each; beyond one tile per SM they
+// only add halo work).  CTA b takes the tiles b, b + slots, ...; when the last round is
+// not full, the tiles that reach a wall (and so also fill its ghost cells, several
+// times the work of an interior tile's phase in between) are placed in the first round of the
+// CTAs that have no tile in the last round.
 void build_tiles(vlb_ctx* c) {
   const StageVariant& v = c->variants[c->variant];
+  auto tiles_of = [&](int cand) {
+    long long count = 0;
+    for (int i = 0; i < c->n_inst; ++i) count += (c->inst[i].n_cells + cand - 1) / cand;
+    return count;
+  };
   int s = v.tc;
-  int slots = 0;
-  if (v.persist) {
-    int nbuf = 1;
-    if (stage_launch_config(c, 1 << 30, &nbuf, &slots) != cudaSuccess) slots = 0;
-    if (slots > 0) {
-      long long best = -1;
-      for (int cand = v.tc; cand >= std::max(3, (v.tc + 1) / 2); --cand) {
-        long long count = 0;
-        for (int i = 0; i < c->n_inst; ++i) count += (c->inst[i].n_cells + cand - 1) / cand;
-        const long long cost = ((count + slots - 1) / slots) * (cand + 3);
-        if (best < 0 || cost < best) best = cost, s = cand;
-      }
+  int nbuf = 1, slots = 0;
+  if (stage_launch_config(c, 1 << 30, &nbuf, &slots) != cudaSuccess) slots = 0;
+  if (v.persist && slots > 0) {
+    long long best = -1;
+    for (int cand = v.tc; cand >= std::max(3, (v.tc + 1) / 2); --cand) {
+      const long long cost = ((tiles_of(cand) + slots - 1) / slots) * (cand + 3);
+      if (best < 0 || cost < best) best = cost, s = cand;
     }
   }
+  for (int cand = s - 1; cand >= 1 && tiles_of(cand) <= c->sms; --cand) s = cand;
+  if (!v.persist) slots = 0;
   c->tiles.clear();
   for (int i = 0; i < c->n_inst; ++i)
     for (int c0 = 0; c0 < c->inst[i].n_cells; c0 += s)

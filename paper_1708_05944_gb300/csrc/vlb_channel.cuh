@@ -262,29 +262,17 @@ __device__ __forceinline__ void channel_equilibrium(const ChanTables<real, Q0, Q
     sr += pr * n;
     se += pr * pr * n;
   }
-  auto sum8 = [](real x) -> real {
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-  };
-  sr = sum8(sr), sp = sum8(sp), se = sum8(se);
+  sr = group_sum<8>(sr), sp = group_sum<8>(sp), se = group_sum<8>(se);
   real nn, th, tl;  // th + tl: the cell's mass that f_eq - R has to carry
   if constexpr (F32) {
     float e = 0.f, nh, nlo;
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {  // as half_sum_comp
-      const float s2 = __shfl_xor_sync(0xffffffffu, sn, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
-      float t, er;
-      two_sum(sn, s2, t, er);
-      sn = t;
-      e = __fadd_rn(__fadd_rn(e, e2), er);
-    }
+    group_sum_comp<8>(sn, e);
     two_sum(sn, tb.ref_hi[0], nh, nlo);
     nn = nh + (nlo + (e + tb.ref_lo[0]));
     two_sum(sn, tb.ref_sum[0], th, tl);
     tl = tl + (e + tb.ref_sum[1]);
   } else {
-    nn = sum8(sn) + tb.ref_hi[0];
+    nn = group_sum<8>(sn) + tb.ref_hi[0];
     th = nn, tl = 0.0;
   }
   const real inv = rcp_rn(nn);
@@ -313,7 +301,7 @@ __device__ __forceinline__ void channel_equilibrium(const ChanTables<real, Q0, Q
     if (q < RP) g[q] *= nn, a0 += g[q];
     else a1 += g[q];
   }
-  a0 = sum8(a0), a1 = sum8(a1);
+  a0 = group_sum<8>(a0), a1 = group_sum<8>(a1);
   // g0 <- g0 target / (sum g0 sum g1); single precision: g0 (1 - delta), the target in float-float
   real scale;
   if constexpr (F32) {

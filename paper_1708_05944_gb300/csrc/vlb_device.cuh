@@ -377,13 +377,17 @@ __device__ __forceinline__ double weno_pow2_dev(double inv_w) {
   return __hiloint2double(__double2hiint(inv_w) & 0x7ff00000, 0);
 }
 
-// 2^-e with e the exponent of x >= 0 (0, Inf and the top binade give values the caller's test
-// of the weight sum rejects)
-__device__ __forceinline__ float inv_pow2(float x) {
-  return __int_as_float(0x7f000000 - (__float_as_int(x) & 0x7f800000));
+// 2^-e with e the exponent of the largest of three numbers >= 0 (Inf and the top binade give values
+// the caller's test of the weight sum rejects; zeros a large power).  Integer compares in double
+// precision: the comparison instructions of the FP64 pipe run at its 1/64 rate.
+__device__ __forceinline__ float inv_pow2_max(float a, float b, float c) {
+  float m;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+  return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
 }
-__device__ __forceinline__ double inv_pow2(double x) {
-  return __hiloint2double(0x7fe00000 - (__double2hiint(x) & 0x7ff00000), 0);
+__device__ __forceinline__ double inv_pow2_max(double a, double b, double c) {
+  const int m = max(__double2hiint(a), max(__double2hiint(b), __double2hiint(c)));
+  return __hiloint2double(0x7fe00000 - (m & 0x7ff00000), 0);
 }
 __device__ __forceinline__ float2 p_rcp(float2 x) {  // 1 / x of normal numbers, about 1 ulp
   float2 r;
@@ -391,17 +395,24 @@ __device__ __forceinline__ float2 p_rcp(float2 x) {  // 1 / x of normal numbers,
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(x.y));
   return r;
 }
-// one division for both: x.x x.y must be a normal number
+// One reciprocal for both, x.x x.y a normal number: the hardware's approximation (20 bits) and two
+// steps of Newton's iteration, r <- r + r (1 - x r), to about 1 ulp.  Seven operations of the FP64
+// pipe in place of two divisions.
 __device__ __forceinline__ double2 p_rcp(double2 x) {
-  const double r = __drcp_rn(__dmul_rn(x.x, x.y));
+  const double y = __dmul_rn(x.x, x.y);
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(y));
+  r = fma(r, fma(-y, r, 1.0), r);
+  r = fma(r, fma(-y, r, 1.0), r);
   return make_double2(__dmul_rn(r, x.y), __dmul_rn(r, x.x));
 }
 // sums of weights the fast path accepts: their reciprocals (and, in double, the product of two) are normal
 __device__ __forceinline__ bool weno_in_range(float2 d) {
   return (d.x > 1e-30f) & (d.x < 1e30f) & (d.y > 1e-30f) & (d.y < 1e30f);
 }
-__device__ __forceinline__ bool weno_in_range(double2 d) {
-  return (d.x > 1e-140) & (d.x < 1e140) & (d.y > 1e-140) & (d.y < 1e140);
+__device__ __forceinline__ bool weno_in_range(double2 d) {  // 2^-465 (1e-140) .. 2^465, by the high words
+  const unsigned lo = 0x22e00000u, n = 0x5d000000u - 0x22e00000u;
+  return (unsigned(__double2hiint(d.x)) - lo < n) & (unsigned(__double2hiint(d.y)) - lo < n);
 }
 
 // 156 S^2, an exact zero raised to a constant that no other indicator comes near
@@ -472,13 +483,6 @@ struct WenoRange<double> {
   __device__ __forceinline__ void add(double2 d) { good = good && weno_in_range(d); }
   __device__ __forceinline__ bool ok() const { return good; }
 };
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-__device__ __forceinline__ double max3(double a, double b, double c) { return fmax(a, fmax(b, c)); }
-
 // The correction of a face from its terms by the fast weights, whose sum den tells whether they
 // hold; K = false: k* are not read, 156 S^2 is formed here.
 template <typename real, bool K>
@@ -490,7 +494,7 @@ __device__ __forceinline__ pair_t<real> weno_corr(const WenoTerms<real>& t, pair
   auto sq = [](P s) { return weno_sq<real>(s); };
   const P bm = p_fma(um, um, K ? km : sq(t.sm)), b0 = p_fma(u0, u0, K ? k0 : sq(t.s0)),
           bp = p_fma(up, up, K ? kp : sq(t.sp));
-  const P r = p_make(inv_pow2(max3(bm.x, b0.x, bp.x)), inv_pow2(max3(bm.y, b0.y, bp.y)));
+  const P r = p_make(inv_pow2_max(bm.x, b0.x, bp.x), inv_pow2_max(bm.y, b0.y, bp.y));
   const P xm = p_mul(bm, r), x0 = p_mul(b0, r), xp = p_mul(bp, r);  // the largest in [1, 2)
   const P A = p_mul(x0, xp), B = p_mul(xm, xp), C = p_mul(xm, x0);
   const P wm = p_mul(p_mul(A, A), w.dm), w0 = p_mul(p_mul(B, B), p_set(real(0.6))), wp = p_mul(p_mul(C, C), w.dp);
@@ -725,33 +729,27 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& err) 
   err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
 }
 
-// Compensated butterfly sum over each half-warp (lanes 0-15 and 16-31
-// separately) in single precision.  Each step adds the partner's value with
-// TwoSum, and the errors accumulate in e.  On return every lane of a half holds
-// the same (s, e), whose sum s + e carries about twice the float precision, so a
+// Compensated butterfly sum over each group of W neighbouring lanes in single precision.  Each step
+// adds the partner's value with TwoSum, and the errors accumulate in e.  On return every lane of a
+// group holds the same (s, e), whose sum s + e carries about twice the float precision, so a
 // reduction that would otherwise need the 1/64-rate FP64 pipe stays on FP32.
-__device__ __forceinline__ void half_sum_comp(float& s, float& e) {
+template <int W>
+__device__ __forceinline__ void group_sum_comp(float& s, float& e) {
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) {
+  for (int o = W / 2; o > 0; o >>= 1) {
     const float s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
-    const float t = __fadd_rn(s, s2);
-    const float bp = __fsub_rn(t, s);
-    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(s2, bp));
+    float t, err;
+    two_sum(s, s2, t, err);
     s = t;
     e = __fadd_rn(__fadd_rn(e, e2), err);
   }
 }
 
-// Plain double sum over each half-warp.
-__device__ __forceinline__ double half_sum(double v) {
+// Plain sum over each group of W neighbouring lanes.
+template <int W, typename T>
+__device__ __forceinline__ T group_sum(T v) {
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ float half_sum(float v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 

@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     tabr0[y] = sizeof(real) == 4 ? real(m.tab0f[x]) : real(m.tab0[x]);
     tabr1[y] = sizeof(real) == 4 ? real(m.tab1f[x]) : real(m.tab1[x]);
   }
+  TileDesc td_next = blockIdx.x < a.n_tiles ? a.tiles[blockIdx.x] : TileDesc{0, 0, 0};
   __syncthreads();
   const bool need_fl = a.caf != 0.0f;
   using Geo = typename L::Geo;
@@ -189,8 +190,6 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     if (lane == 0) bulk_g2s(dst + L::geo_off(Vp) / sizeof(real), geo_src + i.cell0 + t.c0, gbytes, bar + b);
   };
   unsigned phase = 0;  // bit b: parity of buffer b's next completion
-  // the next tile's descriptor is read during the current tile (its load latency hidden)
-  TileDesc td_next = blockIdx.x < a.n_tiles ? a.tiles[blockIdx.x] : TileDesc{0, 0, 0};
   if (nbuf == 2 && warp == 0 && blockIdx.x < a.n_tiles) stage_tile(td_next, 0);
   // one tile per iteration: a launch with one CTA per tile runs the body once, a persistent
   // launch (grid sized by occupancy) walks the tile list, with two buffers staging the next
@@ -221,39 +220,52 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     }
   }
 
-  // ==== phase A: per cell, one half-warp (16 lanes) with no CTA barrier: moments (Eq.
-  // macro_red), tau, the equilibrium moment vectors and factors (Sec. IV.D) and their mass
-  // normalisation.  A warp takes two cells, so each shuffle level and each per-cell scalar
-  // step serves both; warps without a cell go on to the force contractions below.
-  const int NA = (TCe + 1) >> 1;  // warps with cells
+  // ==== phase A: per cell, LPC lanes of a warp with no CTA barrier: moments (Eq. macro_red), tau,
+  // the equilibrium moment vectors and factors (Sec. IV.D) and their mass normalisation.  Each
+  // shuffle level and each per-cell scalar step serves all the warp's cells (eight lanes and four
+  // cells where the node counts are fixed, else a half-warp and two); warps without a cell go on
+  // to the force contractions below.
+  // (single-precision tiles of four cells and less keep two cells a warp: with one warp for all
+  // four, the f~ stage's critical path grew by 3 %)
+  constexpr bool BYROW = EXACT && 16 % Q0MAX == 0 && Q0MAX >= 8 && Q1MAX % 2 == 0;
+  constexpr int LPC = BYROW && !(F32 && TC < 8) ? 8 : 16, CPW = 32 / LPC;
+  constexpr int NF0 = (Q0MAX + LPC - 1) / LPC, NF1 = (Q1MAX + LPC - 1) / LPC;  // factors per lane and axis
+  const int NA = (TCe + CPW - 1) / CPW;  // warps with cells
   for (int wa = warp; wa < NA; wa += NW) {
-    const int hl = lane & 15;
-    const int tc = 2 * wa + (lane >> 4);
-    const bool has = tc < TCe;         // the upper half of the last warp of an odd tile has no cell:
-    const int t = has ? tc : TCe - 1;  // it repeats the lower half's and writes nothing
+    const int hl = lane & (LPC - 1);
+    const int tc = CPW * wa + lane / LPC;
+    const bool has = tc < TCe;         // the last warp's groups beyond the tile have no cell: they
+    const int t = has ? tc : TCe - 1;  // repeat the last one's and write nothing
     const real* F = tile + (t + 3) * row;
-    real sn = 0, sr = 0, sp = 0, se = 0;  // per-lane partial sums over a sixteenth of the velocities
-    if constexpr (EXACT && 16 % Q0MAX == 0 && Q1MAX % (32 / Q0MAX) == 0) {
-      // lane hl sums the nodes j of row i = hl mod Q0 (all, or its share of them): the p^phi weights
-      // are uniform operands and p^R enters once (a third of the instructions of the general form)
-      constexpr int JN = Q1MAX * Q0MAX / 16;
-      const int jb = (hl / Q0MAX) * JN;
-      const real* f = F + 2 * ((hl % Q0MAX) * Q1MAX + jb);
-      const real pr = p0r[hl % Q0MAX];
+    real sn = 0, sr = 0, sp = 0, se = 0;  // the lane's partial sums
+    if constexpr (BYROW) {
+      // lane hl sums nodes j of its rows i (all of them, or its share where a row has several lanes):
+      // the p^phi weights are uniform operands and p^R enters once per row (a third of the
+      // instructions of the general form); row by row, for the rounding of short sums
+      constexpr int PARTS = LPC / Q0MAX > 0 ? LPC / Q0MAX : 1, JN = Q1MAX / PARTS, RP = Q0MAX * PARTS / LPC;
 #pragma unroll
-      for (int j = 0; j < JN; j += 2) {
-        const pair_t<real> f0 = p_load(f + 2 * j), f1 = p_load(f + 2 * j + 2);
-        const real pa = JN == Q1MAX ? (F32 ? real(m.p1f[j]) : real(m.p1[j])) : p1r[jb + j];
-        const real pb = JN == Q1MAX ? (F32 ? real(m.p1f[j + 1]) : real(m.p1[j + 1])) : p1r[jb + j + 1];
-        const real ta = pa * f0.x, tb = pb * f1.x;
-        sn += f0.x, sp += ta, se += pa * ta + f0.y;
-        sn += f1.x, sp += tb, se += pb * tb + f1.y;
+      for (int r = 0; r < RP; ++r) {
+        const int i = hl % Q0MAX + LPC * r, jb = (hl / Q0MAX) * JN;
+        const real* f = F + 2 * (i * Q1MAX + jb);
+        const real pr = p0r[i];
+        real n = 0, q = 0, e = 0;
+#pragma unroll
+        for (int j = 0; j < JN; ++j) {
+          const pair_t<real> x = p_load(f + 2 * j);
+          const real pj = PARTS > 1 ? p1r[jb + j] : F32 ? real(m.p1f[j]) : real(m.p1[j]), u = pj * x.x;
+          n += x.x;
+          q += u;
+          e += pj * u + x.y;
+        }
+        const real u = pr * n;
+        sn += n;
+        sr += u;
+        sp += q;
+        se += pr * u + e;
       }
-      sr = pr * sn;
-      se += pr * sr;
     } else {
 #pragma unroll 4
-      for (int v = hl; v < V; v += 16) {
+      for (int v = hl; v < V; v += LPC) {
         const int i = v / nq1, j = v - i * nq1;
         const pair_t<real> f = p_load(F + 2 * v);
         const real f1 = f.x, f2 = f.y, pr = p0r[i], pp = p1r[j];
@@ -263,19 +275,19 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
         se += (pr * pr + pp * pp) * f1 + f2;
       }
     }
-    // sums over the half-warp; then the sums of D plus those of R and the derived fields
+    // sums over the cell's lanes; then the sums of D plus those of R and the derived fields
     real nn, u0, u1, T;
     double dn = 0.0;  // FP64 path: sum of D (n - sum R)
     float en = 0.f;   // FP32 path: rounding error of the mass sum sn (float-float sn + en)
     if constexpr (F32) {
-      // compensated FP32 butterflies leave the same sums on every lane of the half; n in
+      // compensated FP32 butterflies leave the same sums on every lane of the cell; n in
       // float-float, the other fields in FP32 through one reciprocal: no FP64 and no
       // broadcast on the dependency chain
       float er = 0.f, ep = 0.f, ee = 0.f;
-      half_sum_comp(sn, en);
-      half_sum_comp(sr, er);
-      half_sum_comp(sp, ep);
-      half_sum_comp(se, ee);
+      group_sum_comp<LPC>(sn, en);
+      group_sum_comp<LPC>(sr, er);
+      group_sum_comp<LPC>(sp, ep);
+      group_sum_comp<LPC>(se, ee);
       float nh, nl;
       two_sum(sn, m.ref_nf[0], nh, nl);
       nn = nh + (nl + (en + m.ref_nf[1]));
@@ -284,8 +296,8 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       u1 = (sp + (ep + m.ref_pf)) * inv;
       T = ((se + (ee + m.ref_ef)) * inv - (u0 * u0 + u1 * u1)) * (1.0f / 3.0f);
     } else {
-      dn = half_sum(double(sn));
-      const double dr = half_sum(double(sr)), dpp = half_sum(double(sp)), de = half_sum(double(se));
+      dn = group_sum<LPC>(double(sn));
+      const double dr = group_sum<LPC>(double(sr)), dpp = group_sum<LPC>(double(sp)), de = group_sum<LPC>(double(se));
       nn = real(dn + m.ref_n);
       const real inv = rcp_rn(nn);
       u0 = real(dr + m.ref_r) * inv, u1 = real(dpp + m.ref_p) * inv;
@@ -302,17 +314,23 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       eq_moments_fast<real>(ax ? m.kind1 : m.kind0, ax ? m.N1 : m.N0, u, T, mt + hl * MAXN);
     }
     __syncwarp();
-    // equilibrium factors: lane hl takes g_R[k] and g_phi[k] for k = hl and hl + 16
-    real gr[2] = {real(0), real(0)}, gp[2] = {real(0), real(0)};
+    // equilibrium factors: lane hl takes g_R[k] and g_phi[k] for k = hl, hl + LPC, ...
+    real gr[NF0], gp[NF1], sgr = real(0), sgp = real(0);
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int k = hl + 16 * q;
-      if (16 * q < Q0MAX && k < nq0) {
+    for (int q = 0; q < NF0; ++q) {
+      const int k = hl + LPC * q;
+      gr[q] = real(0);
+      if (k < nq0) {
         const real* mm = mt + ((m.kind0 == 1 && p0r[k] < real(0)) ? 1 : 0) * MAXN;
         for (int s2 = 0; s2 <= m.N0; ++s2) gr[q] += tabr0[s2 * MAXQ + k] * mm[s2];
         gr[q] *= nn;
       }
-      if (16 * q < Q1MAX && k < nq1) {
+    }
+#pragma unroll
+    for (int q = 0; q < NF1; ++q) {
+      const int k = hl + LPC * q;
+      gp[q] = real(0);
+      if (k < nq1) {
         const real* mm = mt + (2 + ((m.kind1 == 1 && p1r[k] < real(0)) ? 1 : 0)) * MAXN;
         for (int s2 = 0; s2 <= m.N1; ++s2) gp[q] += tabr1[s2 * MAXQ + k] * mm[s2];
       }
@@ -324,11 +342,13 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     if constexpr (F32) {
       // A = sum g_R sum g_phi and the target sum D + sum R, both in float-float;
       // delta = (A - target) / A, where A_hi - target_hi is exact (the two are close)
-      float a0, a0e, a1, a1e;
-      two_sum(gr[0], gr[1], a0, a0e);
-      two_sum(gp[0], gp[1], a1, a1e);
-      half_sum_comp(a0, a0e);
-      half_sum_comp(a1, a1e);
+      float a0 = gr[0], a0e = 0.f, a1 = gp[0], a1e = 0.f, t1, er;
+#pragma unroll
+      for (int q = 1; q < NF0; ++q) two_sum(a0, gr[q], t1, er), a0 = t1, a0e += er;
+#pragma unroll
+      for (int q = 1; q < NF1; ++q) two_sum(a1, gp[q], t1, er), a1 = t1, a1e += er;
+      group_sum_comp<LPC>(a0, a0e);
+      group_sum_comp<LPC>(a1, a1e);
       const float Ah = a0 * a1;
       const float Al = fmaf(a0, a1e, fmaf(a0e, a1, fmaf(a0, a1, -Ah)));
       float th, tl;
@@ -337,16 +357,22 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       delta = (__fsub_rn(Ah, th) + (Al - tl)) * rcp_rn(Ah);
       scale0 = real(0);
     } else {
-      const double a0 = half_sum(double(gr[0]) + double(gr[1])), a1 = half_sum(double(gp[0]) + double(gp[1]));
-      scale0 = real((dn + m.ref_n) / (a0 * a1));
+#pragma unroll
+      for (int q = 0; q < NF0; ++q) sgr += gr[q];
+#pragma unroll
+      for (int q = 0; q < NF1; ++q) sgp += gp[q];
+      scale0 = real((dn + m.ref_n) / (group_sum<LPC>(double(sgr)) * group_sum<LPC>(double(sgp))));
     }
     if (has) {
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int k = hl + 16 * q;
-        if (16 * q < Q0MAX && k < nq0)
-          gRn[t * MAXQ + k] = p_set(F32 ? real(fmaf(-float(gr[q]), delta, float(gr[q]))) : gr[q] * scale0);
-        if (16 * q < Q1MAX && k < nq1) gP[t * MAXQ + k] = p_set(gp[q]);
+      for (int q = 0; q < NF0; ++q) {
+        const int k = hl + LPC * q;
+        if (k < nq0) gRn[t * MAXQ + k] = p_set(F32 ? real(fmaf(-float(gr[q]), delta, float(gr[q]))) : gr[q] * scale0);
+      }
+#pragma unroll
+      for (int q = 0; q < NF1; ++q) {
+        const int k = hl + LPC * q;
+        if (k < nq1) gP[t * MAXQ + k] = p_set(gp[q]);
       }
     }
   }
@@ -679,7 +705,9 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     P fm = win.face_checked(side);
     // F_l of the next cell is loaded one cell ahead (a global load, the only one of the walk)
     P fl_next = need_fl ? p_load(Fl) : p_set(real(0));
-#pragma unroll
+// (two cells a pass: fully unrolled, the walk outruns the instruction cache -- batch of 256
+// instances 5.18 ms a call, 4.99 ms so)
+#pragma unroll 2
     for (int t = 0; t < TC; ++t) {
       if (t < TCe) {
         const P fl = fl_next;
