@@ -395,7 +395,9 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
   };
   auto row_wait = [&](int r) -> bool { return mbar_wait(bar + slot(r), unsigned((r - sA) / NRING) & 1u, a.max_polls); };
 
-  // ---- prologue: tables and rows sA .. sA+3
+  // ---- prologue: tables and rows sA .. sA+3 (the tables are no kernel's output; the rows and
+  // everything below are read and written once the launch before this one is complete)
+  grid_launch_dependents();
   if (tid == 0) {
     for (int k = 0; k < NRING; ++k) mbar_init(bar + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -406,6 +408,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
     for (int x = tid; x < int(sizeof(Tab) / 16); x += L::NT) dst[x] = src[x];
   }
   __syncthreads();
+  grid_dependency_wait();
   if (warp == 0)
     for (int r = sA; r <= min(sA + 3, rlast); ++r) row_issue(r);
 

@@ -45,9 +45,8 @@ static cudaError_t stage_buffers(int Vp, int persist, int* nbuf, int* per_sm) {
 template <typename real, int TC, int NT, int Q0, int Q1, bool EXACT, bool FT = false>
 static cudaError_t go_stage(const StageArgs<real>& a, const ModelArgs& m, const KArgs<real>& k, int grid,
                             cudaStream_t s) {
-  couette_stage_kernel<real, TC, Q0, Q1, NT, EXACT, FT>
-      <<<grid, NT, StageSmem<real, TC, NT>::bytes(a.Vp, a.nbuf), s>>>(a, m, k);
-  return cudaGetLastError();
+  return launch_dependent(couette_stage_kernel<real, TC, Q0, Q1, NT, EXACT, FT>, dim3(grid), NT,
+                          StageSmem<real, TC, NT>::bytes(a.Vp, a.nbuf), s, a, m, k);
 }
 
 enum Shape { SH_16x20 = 0, SH_16x12 = 1, SH_8x4 = 2, SH_SMALL = 3, SH_GENERIC = 4 };
@@ -213,8 +212,7 @@ static cudaError_t go_channel(const ChanArgs<real>& a, const void* kpb, int grid
   if (e != cudaSuccess) return e;
   ChanKP<real, Q0, Q1> kp;
   memcpy(&kp, kpb, sizeof(kp));
-  kern<<<grid, L::NT, L::bytes, s>>>(a, kp);
-  return cudaGetLastError();
+  return launch_dependent(kern, dim3(grid), L::NT, L::bytes, s, a, kp);
 }
 
 #ifdef VLB_DEFINE_SHARED
@@ -647,7 +645,9 @@ __global__ void __launch_bounds__(128) shakhov_kernel(real* Fout, const real* Fp
   __shared__ ModelSmem<real> ms;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int V = m.nq0 * m.nq1;
+  grid_launch_dependents();
   stage_model<real>(m, ms);
+  grid_dependency_wait();
   auto wsum = [&](real x) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -712,9 +712,9 @@ cudaError_t launch_shakhov(real* Fout, const real* Fprev, long long cells, int V
                            cudaStream_t s) {
   long long blocks = (cells + 3) / 4;
   if (blocks > 152 * 16) blocks = 152 * 16;
-  shakhov_kernel<real><<<int(blocks > 0 ? blocks : 1), 128, 0, s>>>(Fout, Fprev, cells, Vp, m, inst, n_inst, cc,
-                                                                    one_minus_pr, kn_fixed);
-  return cudaGetLastError();
+  const dim3 g(static_cast<unsigned>(blocks > 0 ? blocks : 1));
+  return launch_dependent(shakhov_kernel<real>, g, 128, 0, s, Fout, Fprev, cells, Vp,
+                          m, inst, n_inst, cc, one_minus_pr, kn_fixed);
 }
 
 // ---------------------------------------------------------------- caller layout <-> device layout

@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
   real* w0r = mv + TC * 4 * MAXN;  // weights: R_ij = w0_i w1_j in the bulk type
   real* w1r = w0r + MAXQ;
 
+  grid_launch_dependents();
   if (tid == 0) {
     mbar_init(bar, 1);
     mbar_init(bar + 1, 1);
@@ -170,8 +171,14 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     tabr0[y] = sizeof(real) == 4 ? real(m.tab0f[x]) : real(m.tab0[x]);
     tabr1[y] = sizeof(real) == 4 ? real(m.tab1f[x]) : real(m.tab1[x]);
   }
+  // the next tile's descriptor is read during the current tile (its load latency hidden); it and the
+  // instances are no kernel's output
   TileDesc td_next = blockIdx.x < a.n_tiles ? a.tiles[blockIdx.x] : TileDesc{0, 0, 0};
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(a.inst + td_next.inst));
   __syncthreads();
+  // what the launch before this one wrote is read and what it read is written from here on
+  // (dependent launches, see launch_dependent)
+  grid_dependency_wait();
   const bool need_fl = a.caf != 0.0f;
   using Geo = typename L::Geo;
   const Geo* geo_src =
