@@ -298,7 +298,7 @@ vlb_status do_large_stage(vlb_ctx* c, int k, int prev, int out) {
                                  c->d_lwall, c->d_nw, static_cast<real*>(c->d_lrec), static_cast<real*>(c->d_lforce),
                                  c->d_lpart, ca[k - 1], cc[k - 1], c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "large-set stage launch");
-  c->launches += 5;
+  c->launches += 3;
   return VLB_OK;
 }
 

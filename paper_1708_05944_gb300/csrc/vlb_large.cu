@@ -1,13 +1,15 @@
 // Circular Couette stage for velocity sets beyond the fused stage kernel's 32 nodes per
 // axis (the high-order half-range models of Sec. VI.D, e.g. HH(4;200) x HH(4;10), 8000
 // velocities).  A cell row no longer fits a tile in shared memory, so the stage runs as
-// four kernels over device memory (L2-resident at these sizes):
+// three kernels over device memory (L2-resident at these sizes), each launched as dependent on the
+// one before (launch_dependent):
 //
 //   sums   -- per cell and chunk of 1024 velocities the sums of the moments (Eqs.
 //             macro_red, mom_quad), and per wall and chunk the outgoing WENO-5 flux of the
 //             extrapolated populations (Eqs. extrapol, nw), FP64, spread over many CTAs;
 //   cell   -- per cell n, u, T from its chunk sums (in a fixed order), tau and the
-//             truncated equilibrium factors (Sec. IV.D) normalised to sum n;
+//             truncated equilibrium factors (Sec. IV.D) normalised to sum n; beside it, on
+//             other CTAs of the same launch (neither needs the other),
 //   force  -- the radial part of the inertial term -(1/R)(p^phi)^2 K^R f (Eq.
 //             boltz_couette_kom): per cell the contraction over the nq0 radial nodes is
 //             a dense (nq0 x nq0) x (nq0 x 2 nq1) product, run as a shared-memory tiled
@@ -18,7 +20,9 @@
 //             wall equilibrium for the incoming half, built in place), the chi flux
 //             difference, the azimuthal part of the inertial term (nq1 terms), BGK and
 //             the RK3 combine, both fields as a pair.
-// Every sum is taken in a fixed order, so results do not depend on scheduling.
+// Every sum is taken in a fixed order, so results do not depend on scheduling.  What bounds it at
+// the sizes it is run at (16 cells): the latency of the three kernels' chains.  16 cells x 1600
+// velocities, single precision, a stage: 40.7 us in five launches, 33.3 us in three.
 //
 // The same kernels run the f~ formulation (LargeModel::ftilde, Sec. VI.B): the stencils and
 // the wall construction act on F~ = sqrt(g) f, whose flux difference e_{s+1/2} F~_{s+1/2} -
@@ -71,6 +75,14 @@ __device__ __forceinline__ real weno_scale(double iw) {
   else return real(iw);
 }
 
+// The power-of-two scale of the WENO walk, at most 2^100 in single precision (tail populations below
+// ~1e-38 are zero there, and for the others the weights do not see the scale).
+template <typename real>
+__device__ __forceinline__ real walk_scale(double iw0, double iw1) {
+  const double sc = weno_pow2_dev(iw0) * weno_pow2_dev(iw1);
+  return real(sizeof(real) == 4 ? fmin(sc, 0x1p100) : fmin(sc, 0x1p996));
+}
+
 // Equilibrium factors of (n, u0, u1, T) into g0 (carrying n, normalised so that
 // sum_ij g0_i g1_j = n, reading of Sec. IV.D) and g1: shared arrays, whole block.
 __device__ void eq_factors(const LargeModel& m, double n, double u0, double u1, double T, double* g0, double* g1,
@@ -106,10 +118,8 @@ __device__ void eq_factors(const LargeModel& m, double n, double u0, double u1, 
 // part[(c NP + p) 4 + k]: over the velocities p kChunk .. (p + 1) kChunk of cell c, the sums
 // of f', p^0 f', p^1 f' and (p^0^2 + p^1^2) f' + f'' (F = D + R), FP64
 template <typename real>
-__global__ void __launch_bounds__(256) lm_partial_kernel(const LargeModel m, const real* F, double* part) {
+__device__ void lm_partial(const LargeModel& m, const real* F, double* part, long long c, int p, int NP) {
   __shared__ double red[4][8];
-  const long long c = blockIdx.x;
-  const int p = blockIdx.y, NP = gridDim.y;
   const real* f = F + c * 2 * m.Vp;
   double q[4] = {0, 0, 0, 0};
 #pragma unroll
@@ -142,11 +152,10 @@ __global__ void __launch_bounds__(256) lm_partial_kernel(const LargeModel m, con
 // wpart[(ii 2 + wall) NP + p]: the outgoing particle flux at the wall of the WENO-5 interface
 // values of the extrapolated populations (Eqs. extrapol, nw) over one chunk of velocities
 template <typename real>
-__global__ void __launch_bounds__(256) lm_wallpart_kernel(const LargeModel m, const real* F, const InstDesc* inst,
-                                                          double* wpart) {
+__device__ void lm_wallpart(const LargeModel& m, const real* F, const InstDesc* inst, double* wpart, int ii, int wall,
+                            int p, int NP) {
   __shared__ double red[8];
   using P = pair_t<real>;
-  const int ii = blockIdx.x, wall = blockIdx.y, p = blockIdx.z, NP = gridDim.z;
   const InstDesc d = inst[ii];
   const long long edge = d.cell0 + (wall == 0 ? 0 : d.n_cells - 1);
   const int dir = wall == 0 ? 1 : -1;
@@ -169,7 +178,15 @@ __global__ void __launch_bounds__(256) lm_wallpart_kernel(const LargeModel m, co
     }
     const P G0 = p_fma(F1, p_set(real(-3)), p_fma(F0, p_set(real(3)), F2));
     const P G1 = p_fma(F1, p_set(real(-8)), p_fma(F0, p_set(real(6)), p_mul(F2, p_set(real(3)))));
-    num += double(weno5p<real>(F2, F1, F0, G0, G1, weno_scale<real>(m.iw0[i] * m.iw1[j])).x) * m.p0[i];
+    // (the update kernel's value: the same cell, side and order)
+    const real sc = walk_scale<real>(m.iw0[i], m.iw1[j]);
+    const P SC = p_set(sc);
+    WenoWin<real, false> w;
+    WenoSide<real> ws;
+    ws.set(wall != 0);
+    w.start(p_mul(wall ? F2 : G1, SC), p_mul(wall ? F1 : G0, SC), p_mul(F0, SC), p_mul(wall ? G0 : F1, SC),
+            p_mul(wall ? G1 : F2, SC));
+    num += double(w.face_checked(ws).x * rcp_rn(sc)) * m.p0[i];
   }
   num = warp_sum<double>(num);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = num;
@@ -181,12 +198,26 @@ __global__ void __launch_bounds__(256) lm_wallpart_kernel(const LargeModel m, co
   }
 }
 
+// blocks 0 .. cells NP - 1: the moment sums of (cell, chunk); then those of (instance, wall, chunk)
+template <typename real>
+__global__ void __launch_bounds__(256) lm_sums_kernel(const LargeModel m, const real* F, long long cells, int NP,
+                                                      const InstDesc* inst, double* part, double* wpart) {
+  grid_launch_dependents();
+  grid_dependency_wait();
+  const long long b = blockIdx.x, nc = cells * NP;
+  if (b < nc) {
+    lm_partial<real>(m, F, part, b / NP, int(b % NP), NP);
+  } else {
+    const int x = int(b - nc), p = x % NP, y = x / NP;
+    lm_wallpart<real>(m, F, inst, wpart, y >> 1, y & 1, p, NP);
+  }
+}
+
 // ---------------------------------------------------------------- cell kernel
 // rec per cell: g0 (nq0, carrying n), g1 (nq1), T, 1/tau; moments from the partial sums
 template <typename real>
-__global__ void __launch_bounds__(kCellThreads) lm_cell_kernel(const LargeModel m, long long cells, int NP,
-                                                               const double* part, const InstDesc* inst, int n_inst,
-                                                               real* rec) {
+__device__ void lm_cell(const LargeModel& m, long long cells, int NP, const double* part, const InstDesc* inst,
+                        int n_inst, real* rec, int block, int blocks) {
   extern __shared__ double sh[];
   double* g0 = sh;
   double* g1 = g0 + m.nq0;
@@ -194,7 +225,7 @@ __global__ void __launch_bounds__(kCellThreads) lm_cell_kernel(const LargeModel 
   double* red = mv + 4 * MAXN;  // 33 entries
   double* q = red + 33;         // 4 entries
   const int stride = m.nq0 + m.nq1 + 2;
-  for (long long c = blockIdx.x; c < cells; c += gridDim.x) {
+  for (long long c = block; c < cells; c += blocks) {
     if (threadIdx.x < 4) {
       double t = 0.0;
       for (int p = 0; p < NP; ++p) t += part[(c * NP + p) * 4 + threadIdx.x];
@@ -224,12 +255,12 @@ __global__ void __launch_bounds__(kCellThreads) lm_cell_kernel(const LargeModel 
 // one cell and one k part, k in chunks of TK; 128 threads, each 2 rows x 5 columns.
 constexpr int TI = 32, TJ = 40, TK = 32, FT = 128, KS = 4;
 template <typename real>
-__global__ void __launch_bounds__(FT) lm_force_kernel(const LargeModel m, const real* F, const GeoCell* geo, real* out) {
+__device__ void lm_force(const LargeModel& m, const real* F, const GeoCell* geo, real* out, long long cells, long long c,
+                         int by, int bz) {
   __shared__ real Ks[TI][TK + 1];
   __shared__ real Ds[TK][TJ];
-  const long long c = blockIdx.x;
   const int ncol = 2 * m.nq1, ntj = (ncol + TJ - 1) / TJ;
-  const int i0 = blockIdx.y * TI, c0 = (blockIdx.z % ntj) * TJ, h = blockIdx.z / ntj;
+  const int i0 = by * TI, c0 = (bz % ntj) * TJ, h = bz / ntj;
   const int kchunks = (m.nq0 + TK - 1) / TK, per = (kchunks + KS - 1) / KS;
   const int kbeg = h * per * TK, kend = min(m.nq0, (h + 1) * per * TK);
   const real* D = F + c * 2 * m.Vp;  // [i][jd], row stride ncol
@@ -273,24 +304,44 @@ __global__ void __launch_bounds__(FT) lm_force_kernel(const LargeModel m, const 
       const int col = c0 + tj + 8 * r;
       if (col >= ncol) continue;
       const real pj = real(m.p1[col >> 1]);
-      out[(size_t(h) * gridDim.x + c) * 2 * m.Vp + size_t(i) * ncol + col] = -irb * pj * pj * (si * acc[q][r]);
+      out[(size_t(h) * cells + c) * 2 * m.Vp + size_t(i) * ncol + col] = -irb * pj * pj * (si * acc[q][r]);
     }
   }
 }
 
-// ---------------------------------------------------------------- update kernel
+// blocks 0 .. cblocks - 1: the cells (a long serial chain, so first); then the force tiles of every cell
 template <typename real>
-__global__ void lm_update_kernel(const LargeModel m, const real* Fprev, const real* Fl, real* Fout, long long cells,
+__global__ void __launch_bounds__(FT) lm_cell_force_kernel(const LargeModel m, const real* F, const GeoCell* geo,
+                                                           real* out, long long cells, int NP, const double* part,
+                                                           const InstDesc* inst, int n_inst, real* rec, int cblocks,
+                                                           int ny, int nz) {
+  grid_launch_dependents();
+  grid_dependency_wait();
+  if (int(blockIdx.x) < cblocks) {
+    lm_cell<real>(m, cells, NP, part, inst, n_inst, rec, int(blockIdx.x), cblocks);
+  } else {
+    const long long b = (long long)blockIdx.x - cblocks;
+    const int t = int(b % (ny * nz));
+    lm_force<real>(m, F, geo, out, cells, b / (ny * nz), t % ny, t / ny);
+  }
+}
+
+// ---------------------------------------------------------------- update kernel
+constexpr int UT = 128;  // velocities per CTA
+template <typename real>
+__global__ void __launch_bounds__(UT) lm_update_kernel(const LargeModel m, const real* Fprev, const real* Fl, real* Fout, long long cells,
                                  const InstDesc* inst, int n_inst, const GeoCell* geo, const real* rec,
                                  const real* force, const double* walls, const double* wpart, int NP, double* nw,
                                  double ca, double cc) {
   using P = pair_t<real>;
   constexpr bool F32 = sizeof(real) == 4;
-  const long long total = cells * m.V;
-  const int stride = m.nq0 + m.nq1 + 2;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < total; x += (long long)gridDim.x * blockDim.x) {
-    const long long c = x / m.V;
-    const int v = int(x - c * m.V);
+  const int stride = m.nq0 + m.nq1 + 2, per = (m.V + UT - 1) / UT;  // CTAs per cell
+  grid_launch_dependents();
+  grid_dependency_wait();
+  for (long long x = blockIdx.x; x < cells * per; x += gridDim.x) {
+    const long long c = x / per;
+    const int v = int(x - c * per) * UT + int(threadIdx.x);
+    if (v >= m.V) continue;
     const int i = v / m.nq1, j = v - i * m.nq1;
     const int ii = instance_of(inst, n_inst, c);
     const InstDesc& d = inst[ii];
@@ -334,22 +385,24 @@ __global__ void lm_update_kernel(const LargeModel m, const real* Fprev, const re
           nw[ii * 2 + wall] = nwv;
           if (!isfinite(nwv)) atomicOr(m.err, ERR_NONFINITE);
         }
-    const P Fm3 = at(-3), Fm2 = at(-2), Fm1 = at(-1), S0 = at(0), Fp1 = at(1), Fp2 = at(2), Fp3 = at(3);
     const P F0 = p_load(Fprev + c * 2 * m.Vp + 2 * v);  // the cell's own D
-    const real sc = weno_scale<real>(m.iw0[i] * m.iw1[j]);
+    // both interfaces by the walk of the fused kernel: the upwind cells are s - 1, s for p^R >= 0 and
+    // s, s + 1 otherwise
+    const real sc = walk_scale<real>(m.iw0[i], m.iw1[j]);
+    const P SC = p_set(sc);
     const real pr = real(m.p0[i]);
-    P fm, fp;
-    if (pr >= real(0)) {
-      fm = weno5p<real>(Fm3, Fm2, Fm1, S0, Fp1, sc);
-      fp = weno5p<real>(Fm2, Fm1, S0, Fp1, Fp2, sc);
-    } else {
-      fm = weno5p<real>(Fp2, Fp1, S0, Fm1, Fm2, sc);
-      fp = weno5p<real>(Fp3, Fp2, Fp1, S0, Fm1, sc);
-    }
+    const int up = pr >= real(0) ? 0 : 1;
+    WenoSide<real> side;
+    side.set(up == 0);
+    WenoWin<real, true> win;
+    win.start(p_mul(at(up - 3), SC), p_mul(at(up - 2), SC), p_mul(at(up - 1), SC), p_mul(at(up), SC), p_mul(at(up + 1), SC));
+    const P fm = win.face_checked(side);
+    win.push(p_mul(at(up + 2), SC));
+    const P fp = win.face_checked(side);
     const GeoCell g = geo[c];
     // -adv = -p^R (cp F_{s+1/2} - cm F_{s-1/2}); f~: the factors e_{s+-1/2} / (d eta sqrt(g_s))
     const real cp = real(m.ftilde ? m.advp[c] : g.cp), cm = real(m.ftilde ? m.advm[c] : g.cm);
-    const P nadv = p_mul(p_sub(p_mul(fp, p_set(cp)), p_mul(fm, p_set(cm))), p_set(-pr));
+    const P nadv = p_mul(p_sub(p_mul(fp, p_set(cp)), p_mul(fm, p_set(cm))), p_set(-pr * rcp_rn(sc)));
     // the azimuthal part of the inertial term, +inv_rbar p0_i sum_l Kt1[j][l] D[c][i][l]
     const real* Drow = Fprev + c * 2 * m.Vp + size_t(i) * 2 * m.nq1;
     P e = p_set(real(0));
@@ -636,15 +689,18 @@ cudaError_t lm_stage(const LargeModel& m, const real* Fprev, const real* Fl, rea
                      real* rec, real* force, double* part, double ca, double cc, cudaStream_t s) {
   const int NP = chunks(m);
   double* wpart = part + cells * NP * 4;
-  lm_partial_kernel<real><<<dim3(unsigned(cells), unsigned(NP)), 256, 0, s>>>(m, Fprev, part);
-  lm_wallpart_kernel<real><<<dim3(unsigned(n_inst), 2, unsigned(NP)), 256, 0, s>>>(m, Fprev, inst, wpart);
-  const int cgrid = int(cells < 152 * 8 ? cells : 152 * 8);
-  lm_cell_kernel<real><<<cgrid, kCellThreads, cell_smem(m), s>>>(m, cells, NP, part, inst, n_inst, rec);
-  const dim3 fg(unsigned(cells), unsigned((m.nq0 + TI - 1) / TI), unsigned((2 * m.nq1 + TJ - 1) / TJ) * KS);
-  lm_force_kernel<real><<<fg, FT, 0, s>>>(m, Fprev, geo, force);
-  lm_update_kernel<real><<<grid_for(cells * m.V, 256), 256, 0, s>>>(m, Fprev, Fl, Fout, cells, inst, n_inst, geo,
-                                                                   rec, force, walls, wpart, NP, nw, ca, cc);
-  return cudaGetLastError();
+  const int cb = int(cells < 152 * 8 ? cells : 152 * 8);
+  const int ny = (m.nq0 + TI - 1) / TI, nz = (2 * m.nq1 + TJ - 1) / TJ * KS;
+  const long long ub = cells * ((m.V + UT - 1) / UT);
+  cudaError_t e = launch_dependent(lm_sums_kernel<real>, dim3(unsigned(cells * NP + 2ll * n_inst * NP)), 256, 0, s, m,
+                                   Fprev, cells, NP, inst, part, wpart);
+  if (e == cudaSuccess)
+    e = launch_dependent(lm_cell_force_kernel<real>, dim3(unsigned(cb + cells * ny * nz)), FT, cell_smem(m), s, m, Fprev,
+                         geo, force, cells, NP, part, inst, n_inst, rec, cb, ny, nz);
+  if (e == cudaSuccess)
+    e = launch_dependent(lm_update_kernel<real>, dim3(unsigned(ub < 152 * 64 ? ub : 152 * 64)), UT, 0, s, m, Fprev, Fl,
+                         Fout, cells, inst, n_inst, geo, rec, force, walls, wpart, NP, nw, ca, cc);
+  return e;
 }
 
 template <typename real>
