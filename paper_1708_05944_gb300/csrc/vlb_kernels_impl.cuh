@@ -64,8 +64,10 @@ template <typename real>
 struct VariantTable;
 template <>
 struct VariantTable<float> {
-  static constexpr StageVariant v16x20[] = {{4, 256, 0},  {8, 256, 0},  {4, 320, 0}, {8, 320, 0},
-                                            {16, 320, 0}, {10, 320, 0}, {9, 320, 0}};
+  // (the first is the default: a thread per velocity and two CTAs of ten cells a SM; with 256 threads
+  // a second pass over 64 of the 320 velocities leaves most of them idle)
+  static constexpr StageVariant v16x20[] = {{10, 320, 0}, {8, 256, 0},  {4, 320, 0}, {8, 320, 0},
+                                            {16, 320, 0}, {4, 256, 0}, {9, 320, 0}};
   static constexpr StageVariant v16x12[] = {{16, 256, 0}, {8, 256, 0}, {16, 384, 0}};
   static constexpr StageVariant v8x4[] = {{16, 64, 0}, {8, 64, 0}};
   static constexpr StageVariant vsmall[] = {{16, 64, 0}};
@@ -122,7 +124,7 @@ cudaError_t launch_stage(StageVariant v, const StageArgs<real>& a, const ModelAr
 #define VLB_FT(SH, TC_, NT_, q0, q1, ex) \
   if (sh == SH && v.tc == TC_ && v.nt == NT_) return go_stage<real, TC_, NT_, q0, q1, ex, true>(a, m, k, grid, s);
     if constexpr (sizeof(real) == 4) {
-      VLB_FT(SH_16x20, 4, 256, 16, 20, true) VLB_FT(SH_16x12, 16, 256, 16, 12, true)
+      VLB_FT(SH_16x20, 10, 320, 16, 20, true) VLB_FT(SH_16x12, 16, 256, 16, 12, true)
       VLB_FT(SH_8x4, 16, 64, 8, 4, true) VLB_FT(SH_SMALL, 16, 64, MAXQ, MAXQ, false)
       VLB_FT(SH_GENERIC, 16, 256, MAXQ, MAXQ, false)
     } else {
@@ -165,7 +167,7 @@ cudaError_t stage_config(StageVariant v, const ModelArgs& m, int Vp, int* nbuf, 
 #define VLB_FT(SH, TC_, NT_, q0, q1, ex) \
   if (sh == SH && v.tc == TC_ && v.nt == NT_) return stage_buffers<real, TC_, NT_, q0, q1, ex, true>(Vp, v.persist, nbuf, per_sm);
     if constexpr (sizeof(real) == 4) {
-      VLB_FT(SH_16x20, 4, 256, 16, 20, true) VLB_FT(SH_16x12, 16, 256, 16, 12, true)
+      VLB_FT(SH_16x20, 10, 320, 16, 20, true) VLB_FT(SH_16x12, 16, 256, 16, 12, true)
       VLB_FT(SH_8x4, 16, 64, 8, 4, true) VLB_FT(SH_SMALL, 16, 64, MAXQ, MAXQ, false)
       VLB_FT(SH_GENERIC, 16, 256, MAXQ, MAXQ, false)
     } else {
@@ -894,6 +896,10 @@ template <typename real, int NV, int CH>
 __global__ void __launch_bounds__(256) deviation_kernel(const real* src, real* dst, long long cells, int Vp,
                                                         const __grid_constant__ ModelArgs m, int to_dev, CellMap map) {
   using P = pair_t<real>;
+  // (the weights by way of shared memory: an index per lane into the parameters is serialised)
+  __shared__ double sw[2][MAXQ];
+  if (threadIdx.x < 2 * MAXQ) sw[threadIdx.x / MAXQ][threadIdx.x % MAXQ] = (threadIdx.x < MAXQ ? m.w0 : m.w1)[threadIdx.x % MAXQ];
+  __syncthreads();
   const int lane = threadIdx.x & 31;
   const int V = m.nq0 * m.nq1;
   RestValue<real> R[CH][NV];
@@ -903,7 +909,7 @@ __global__ void __launch_bounds__(256) deviation_kernel(const real* src, real* d
     for (int q = 0; q < NV; ++q) {
       const int v = (32 * k + lane) * NV + q;
       const int i = v < V ? v / m.nq1 : 0, j = v < V ? v - i * m.nq1 : 0;
-      R[k][q] = rest_value<real>(m.w0[i] * m.w1[j]);
+      R[k][q] = rest_value<real>(sw[0][i] * sw[1][j]);
     }
   const real sgn = to_dev ? real(-1) : real(1);
   const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
