@@ -337,32 +337,34 @@ __device__ __forceinline__ pair_t<real> weno5p(pair_t<real> a, pair_t<real> b, p
 // ---------------------------------------------------------------- WENO-5 on shared differences
 // The same reconstruction for kernels that walk along a line of cells, in the form whose terms
 // neighbouring interfaces share.  With G a cell value times an exact power of two close to
-// 2 / (w_i w_j) (see weno_scale), D = G_{k+1} - G_k, S_k = (D_{k+1/2} - D_{k-1/2}) / 12 and the
-// three stencils of the upwind cell c centred on c - 1, c, c + 1:
-//   u_- = D_{c-1/2} + 6 S_{c-1},  u_0 = D_{c-1/2} + 6 S_c,  u_+ = D_{c+1/2} - 6 S_{c+1},
-//   sigma_q = 156 S_q^2 + u_q^2   (Eq. weno_sigma, times a constant the weights do not see),
-//   candidate_q = G_c + side u_q / 2 + S_q,
+// 1 / (w_i w_j), D = G_{k+1} - G_k, S_k = D_{k+1/2} - D_{k-1/2} and the three stencils of the
+// upwind cell c centred on c - 1, c, c + 1:
+//   u_- = 2 D_{c-1/2} + S_{c-1},  u_0 = D_{c-1/2} + D_{c+1/2},  u_+ = 2 D_{c+1/2} - S_{c+1},
+//   sigma_q = 13/3 S_q^2 + u_q^2   (Eq. weno_sigma, times 4, which the weights do not see),
+//   candidate_q = G_c + (3 side u_q + S_q) / 12,
 // side = +1 for the value at c + 1/2 (velocity >= 0, ideal weights 1/10, 6/10, 3/10 on -, 0, +)
 // and -1 for the value at c - 1/2 (velocity < 0, the mirrored weights).  So one cell-centred
-// formula serves both upwind sides with three constants per velocity, a new cell of the walk
-// adds one difference, one S and one 156 S^2, and the value is the cell's own plus a correction.
-// (A constant far below any non-zero indicator stands for an exact zero in 156 S^2, so that a
+// formula serves both upwind sides with three constants per velocity (the ideal weights relative
+// to the middle one), a new cell of the walk adds one difference, one S and one 13/3 S^2, and the
+// value is the cell's own plus a correction.
+// (A constant far below any non-zero indicator stands for an exact zero in 13/3 S^2, so that a
 // uniform stretch, all three indicators zero, takes the ideal weights and the value of its cells
 // on the fast path; one zero then gets all the weight there, two take weno_corr_slow.)
 // Power-of-two scaling keeps the scaled values exact; a face value is scaled back by its inverse.
-// 33 packed operations per interface against 52 of weno5p, whose bound (the FP32 pipe, 128 fma
-// per clock and SM, packed or not) it shares.
+// 34 packed operations per interface against 52 of weno5p, whose bound (the FP32 pipe, 128 fma
+// per clock and SM, packed or not) it shares; written with few constants, since a packed operand
+// is a register pair, which the compiler rebuilds at every use once registers run out.
 template <typename real>
-struct WenoSide {  // per velocity: side / 2 and the ideal weights of the - and + stencils
-  pair_t<real> hs, dm, dp;
+struct WenoSide {  // per velocity: 3 side and the ideal weights of the - and + stencils over the middle one's
+  pair_t<real> h3, dm, dp;
   __device__ __forceinline__ void set(bool up) {
-    hs = p_set(up ? real(0.5) : real(-0.5));
-    dm = p_set(up ? real(0.1) : real(0.3));
-    dp = p_set(up ? real(0.3) : real(0.1));
+    h3 = p_set(up ? real(3) : real(-3));
+    dm = p_set(up ? real(1) / real(6) : real(0.5));
+    dp = p_set(up ? real(0.5) : real(1) / real(6));
   }
 };
 
-// Power of two with the exponent of 2 / w (w a positive normal number), and its inverse by flipping sign.
+// A power of two next to 1 / w.
 inline double weno_pow2(double inv_w) {
   int e = 0;
   frexp(inv_w, &e);
@@ -415,10 +417,10 @@ __device__ __forceinline__ bool weno_in_range(double2 d) {  // 2^-465 (1e-140) .
   return (unsigned(__double2hiint(d.x)) - lo < n) & (unsigned(__double2hiint(d.y)) - lo < n);
 }
 
-// 156 S^2, an exact zero raised to a constant that no other indicator comes near
+// 13/3 S^2, an exact zero raised to a constant that no other indicator comes near
 template <typename real>
 __device__ __forceinline__ pair_t<real> weno_sq(pair_t<real> s) {
-  return p_fma(p_mul(s, p_set(real(156))), s, p_set(sizeof(real) == 4 ? real(1e-40) : real(1e-280)));
+  return p_fma(p_mul(s, p_set(real(13) / real(3))), s, p_set(sizeof(real) == 4 ? real(1e-40) : real(1e-280)));
 }
 
 // The five terms of a face (see above): S on the three stencils and the cell's two differences.
@@ -427,8 +429,6 @@ struct WenoTerms {
   pair_t<real> sm, s0, sp, dm, dc;
 };
 
-// sum_q w_q (candidate_q - G_c) / sum_q w_q, the correction of the cell value, in any case: Table
-// IV for vanishing indicators, delta_q (sigma_min / sigma_q)^2 where the fast weights leave their range.
 // num / s for 0 <= num <= s, s > 0 of any size (single precision: the reciprocal instruction wants a
 // normal operand; both are scaled by the same power of two)
 __device__ __forceinline__ float ratio_to(float num, float s) {
@@ -439,13 +439,16 @@ __device__ __forceinline__ float ratio_to(float num, float s) {
 }
 __device__ __forceinline__ double ratio_to(double num, double s) { return num / s; }
 
+// sum_q w_q (candidate_q - G_c) / sum_q w_q, the correction of the cell value, in any case: Table
+// IV for vanishing indicators, delta_q (sigma_min / sigma_q)^2 where the fast weights leave their range.
 template <typename real>
 __device__ __forceinline__ real weno_corr_slow1(real sm, real s0, real sp, real dm, real dc, bool up) {
-  const real um = rfma(sm, real(6), dm), u0 = rfma(s0, real(6), dm), uc = rfma(sp, real(-6), dc);
-  const real bm = rfma(um, um, rmul(rmul(sm, real(156)), sm)), b0 = rfma(u0, u0, rmul(rmul(s0, real(156)), s0)),
-             bp = rfma(uc, uc, rmul(rmul(sp, real(156)), sp));
-  const real hs = up ? real(0.5) : real(-0.5), lm = up ? real(0.1) : real(0.3), lp = up ? real(0.3) : real(0.1);
-  const real qm = rfma(um, hs, sm), q0 = rfma(u0, hs, s0), qp = rfma(uc, hs, sp);
+  const real k = real(13) / real(3);
+  const real um = radd(radd(dm, dm), sm), u0 = radd(dm, dc), uc = radd(radd(dc, dc), -sp);
+  const real bm = rfma(um, um, rmul(rmul(sm, k), sm)), b0 = rfma(u0, u0, rmul(rmul(s0, k), s0)),
+             bp = rfma(uc, uc, rmul(rmul(sp, k), sp));
+  const real h3 = up ? real(3) : real(-3), lm = up ? real(0.1) : real(0.3), lp = up ? real(0.3) : real(0.1);
+  const real qm = rfma(um, h3, sm), q0 = rfma(u0, h3, s0), qp = rfma(uc, h3, sp);
   const real mn = vmin(bm, vmin(b0, bp));
   real wm, w0, wp;
   if (mn == real(0)) {
@@ -456,7 +459,7 @@ __device__ __forceinline__ real weno_corr_slow1(real sm, real s0, real sp, real 
     const real rm = ratio_to(mn, bm), r0 = ratio_to(mn, b0), rp = ratio_to(mn, bp);
     wm = lm * rm * rm, w0 = real(0.6) * r0 * r0, wp = lp * rp * rp;
   }
-  return vdiv(rfma(wm, qm, rfma(w0, q0, rmul(wp, qp))), radd(radd(wm, w0), wp));
+  return vdiv(rfma(wm, qm, rfma(w0, q0, rmul(wp, qp))), radd(radd(wm, w0), wp)) * (real(1) / real(12));
 }
 template <typename real>
 __device__ __forceinline__ pair_t<real> weno_corr_slow(const WenoTerms<real>& t, bool up) {
@@ -483,74 +486,75 @@ struct WenoRange<double> {
   __device__ __forceinline__ void add(double2 d) { good = good && weno_in_range(d); }
   __device__ __forceinline__ bool ok() const { return good; }
 };
-// The correction of a face from its terms by the fast weights, whose sum den tells whether they
-// hold; K = false: k* are not read, 156 S^2 is formed here.
+// The value of a face from the cell's and its terms by the fast weights, whose sum den tells whether
+// they hold; K = false: k* are not read, 13/3 S^2 is formed here.
 template <typename real, bool K>
-__device__ __forceinline__ pair_t<real> weno_corr(const WenoTerms<real>& t, pair_t<real> km, pair_t<real> k0,
-                                                  pair_t<real> kp, const WenoSide<real>& w, pair_t<real>& den) {
+__device__ __forceinline__ pair_t<real> weno_face(pair_t<real> g0, const WenoTerms<real>& t, pair_t<real> km,
+                                                  pair_t<real> k0, pair_t<real> kp, const WenoSide<real>& w,
+                                                  pair_t<real>& den) {
   using P = pair_t<real>;
-  const P um = p_fma(t.sm, p_set(real(6)), t.dm), u0 = p_fma(t.s0, p_set(real(6)), t.dm),
-          up = p_fma(t.sp, p_set(real(-6)), t.dc);
+  const P um = p_add(p_add(t.dm, t.dm), t.sm), u0 = p_add(t.dm, t.dc), up = p_sub(p_add(t.dc, t.dc), t.sp);
   auto sq = [](P s) { return weno_sq<real>(s); };
   const P bm = p_fma(um, um, K ? km : sq(t.sm)), b0 = p_fma(u0, u0, K ? k0 : sq(t.s0)),
           bp = p_fma(up, up, K ? kp : sq(t.sp));
   const P r = p_make(inv_pow2_max(bm.x, b0.x, bp.x), inv_pow2_max(bm.y, b0.y, bp.y));
   const P xm = p_mul(bm, r), x0 = p_mul(b0, r), xp = p_mul(bp, r);  // the largest in [1, 2)
   const P A = p_mul(x0, xp), B = p_mul(xm, xp), C = p_mul(xm, x0);
-  const P wm = p_mul(p_mul(A, A), w.dm), w0 = p_mul(p_mul(B, B), p_set(real(0.6))), wp = p_mul(p_mul(C, C), w.dp);
+  const P wm = p_mul(p_mul(A, A), w.dm), w0 = p_mul(B, B), wp = p_mul(p_mul(C, C), w.dp);
   den = p_add(p_add(wm, w0), wp);
-  const P qm = p_fma(um, w.hs, t.sm), q0 = p_fma(u0, w.hs, t.s0), qp = p_fma(up, w.hs, t.sp);
+  const P qm = p_fma(um, w.h3, t.sm), q0 = p_fma(u0, w.h3, t.s0), qp = p_fma(up, w.h3, t.sp);
   const P num = p_fma(wm, qm, p_fma(w0, q0, p_mul(wp, qp)));
-  return p_mul(num, p_rcp(den));
+  const P i = p_rcp(den);
+  return p_fma(num, p_make(i.x * (real(1) / real(12)), i.y * (real(1) / real(12))), g0);
 }
 
 // The walk's state around the upwind cell: cell values g0 (the cell), g1, g2 (the next two), the
-// differences dm (c - 1/2), dc (c + 1/2), dn (c + 3/2), S on c - 1, c, c + 1, and with K also 156 S^2
+// differences dm (c - 1/2), dc (c + 1/2), dn (c + 3/2), S on c - 1, c, c + 1, and with K also 13/3 S^2
 // there (six registers more, four operations less).
 template <typename real, bool K>
 struct WenoWin {
   using P = pair_t<real>;
   P g0, g1, g2, dm, dc, dn, sm, s0, sp, km, k0, kp;
-  __device__ __forceinline__ static P sq(P s) { return weno_sq<real>(s); }
-  __device__ __forceinline__ static P second(P hi, P lo) { return p_mul(p_sub(hi, lo), p_set(real(1) / real(12))); }
   // five neighbouring cells in walk order, centred on c
   __device__ __forceinline__ void start(P a, P b, P c, P d, P e) {
     const P d0 = p_sub(b, a);
     g0 = c, g1 = d, g2 = e;
     dm = p_sub(c, b), dc = p_sub(d, c), dn = p_sub(e, d);
-    sm = second(dm, d0), s0 = second(dc, dm), sp = second(dn, dc);
-    if constexpr (K) km = sq(sm), k0 = sq(s0), kp = sq(sp);
+    sm = p_sub(dm, d0), s0 = p_sub(dc, dm), sp = p_sub(dn, dc);
+    if constexpr (K) km = weno_sq<real>(sm), k0 = weno_sq<real>(s0), kp = weno_sq<real>(sp);
   }
   __device__ __forceinline__ void push(P f) {  // one cell on
     g0 = g1, g1 = g2;
     dm = dc, dc = dn, dn = p_sub(f, g2);
     g2 = f;
-    sm = s0, s0 = sp, sp = second(dn, dc);
-    if constexpr (K) km = k0, k0 = kp, kp = sq(sp);
+    sm = s0, s0 = sp, sp = p_sub(dn, dc);
+    if constexpr (K) km = k0, k0 = kp, kp = weno_sq<real>(sp);
   }
   __device__ __forceinline__ WenoTerms<real> terms() const { return WenoTerms<real>{sm, s0, sp, dm, dc}; }
+  __device__ __forceinline__ P fast(const WenoSide<real>& w, P& den) const {
+    if constexpr (K) return weno_face<real, true>(g0, terms(), km, k0, kp, w, den);
+    else return weno_face<real, false>(g0, terms(), sm, sm, sm, w, den);
+  }
   // the interface value on the cell's side w (times the scale of G), where the range stays ok
   __device__ __forceinline__ P face(const WenoSide<real>& w, WenoRange<real>& range) const {
-    P den, corr;
-    if constexpr (K) corr = weno_corr<real, true>(terms(), km, k0, kp, w, den);
-    else corr = weno_corr<real, false>(terms(), sm, sm, sm, w, den);
+    P den;
+    const P f = fast(w, den);
     range.add(den);
-    return p_add(g0, corr);
+    return f;
   }
   __device__ __forceinline__ bool in_range(bool up) const {  // whether face() holds for this face
     P den;
     WenoSide<real> w;
     w.set(up);
-    weno_corr<real, false>(terms(), sm, sm, sm, w, den);
+    fast(w, den);
     return weno_in_range(den);
   }
   // the value, checked at once
   __device__ __forceinline__ P face_checked(const WenoSide<real>& w) const {
-    P den, corr;
-    if constexpr (K) corr = weno_corr<real, true>(terms(), km, k0, kp, w, den);
-    else corr = weno_corr<real, false>(terms(), sm, sm, sm, w, den);
-    if (__builtin_expect(!weno_in_range(den), 0)) corr = weno_corr_slow<real>(terms(), w.hs.x > real(0));
-    return p_add(g0, corr);
+    P den;
+    P f = fast(w, den);
+    if (__builtin_expect(!weno_in_range(den), 0)) f = face_any(w.h3.x > real(0));
+    return f;
   }
   // the value in any case
   __device__ __forceinline__ P face_any(bool up) const { return p_add(g0, weno_corr_slow<real>(terms(), up)); }

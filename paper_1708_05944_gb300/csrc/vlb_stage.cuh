@@ -74,9 +74,9 @@ struct StageSmem {
   static constexpr size_t n_dbl = 2 * MAXQ + NW * 4 + 2 * MAXQ + 16;
   __host__ __device__ static size_t real_off(int Vp, int nbuf) { return dbl_off(Vp, nbuf) + n_dbl * sizeof(double); }
   // reals: p0, p1, the two WENO scales (MAXQ each), tab0, tab1 (MAXQ*MAXN each), then pairs: n g_R and g_phi
-  // (TC*MAXQ each), (1, T), -1/tau, cp, -cm, 1/Rbar (TC each); then moment vectors (TC*4*MAXN),
+  // (TC*MAXQ each), six pairs of per-cell values (TC); then moment vectors (TC*4*MAXN),
   // w0, w1 (MAXQ each)
-  static constexpr size_t n_real = 4 * MAXQ + 2 * MAXQ * MAXN + 4 * TC * MAXQ + 10 * TC + TC * 4 * MAXN + 2 * MAXQ;
+  static constexpr size_t n_real = 4 * MAXQ + 2 * MAXQ * MAXN + 4 * TC * MAXQ + 12 * TC + TC * 4 * MAXN + 2 * MAXQ;
   __host__ __device__ static size_t bytes(int Vp, int nbuf) { return real_off(Vp, nbuf) + n_real * sizeof(real); }
 };
 
@@ -131,12 +131,10 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
   using P2 = pair_t<real>;
   P2* gRn = reinterpret_cast<P2*>(tabr1 + MAXQ * MAXN);  // [t][i] n_t g_{R,i} twice
   P2* gP = gRn + TC * MAXQ;                              // [t][j] g_{phi,j} twice
-  P2* cT1 = gP + TC * MAXQ;                              // (1, T)
-  P2* cNtau = cT1 + TC;                                  // -1/tau twice
-  P2* ccp = cNtau + TC;                                  // cp twice
-  P2* cNcm = ccp + TC;                                   // -cm twice
-  P2* cIR = cNcm + TC;                                   // 1/Rbar twice
-  real* mv = reinterpret_cast<real*>(cIR + TC);          // [t][axis*2 + side][s]
+  // per cell: cp twice, -cm twice, 1/Rbar twice, -1/tau twice, (1, T), pad (16-byte loads)
+  enum { C_CP = 0, C_NCM, C_IR, C_NTAU, C_1T, C_N = 6 };
+  P2* crec = gP + TC * MAXQ;
+  real* mv = reinterpret_cast<real*>(crec + C_N * TC);   // [t][axis*2 + side][s]
   real* w0r = mv + TC * 4 * MAXN;  // weights: R_ij = w0_i w1_j in the bulk type
   real* w1r = w0r + MAXQ;
 
@@ -221,9 +219,9 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
   {  // the cells' geometry as pairs for phase D
     const Geo* g = reinterpret_cast<const Geo*>(tile + L::geo_off(Vp) / sizeof(real));
     for (int t = tid; t < TCe; t += NT) {
-      ccp[t] = p_set(real(g[t].cp));
-      cNcm[t] = p_set(real(-g[t].cm));
-      cIR[t] = p_set(real(g[t].inv_rbar));
+      crec[C_N * t + C_CP] = p_set(real(g[t].cp));
+      crec[C_N * t + C_NCM] = p_set(real(-g[t].cm));
+      crec[C_N * t + C_IR] = p_set(real(g[t].inv_rbar));
     }
   }
 
@@ -311,8 +309,8 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       T = (real(de + m.ref_e) * inv - (u0 * u0 + u1 * u1)) * (real(1) / real(3));
     }
     if (hl == 0 && has) {
-      cT1[t] = p_make(real(1), T);
-      cNtau[t] = p_set(-relaxation_rate<real>(in.tau_mode, rcp_rn(F32 ? real(in.kn_f) : real(in.kn)), nn, T));
+      crec[C_N * t + C_1T] = p_make(real(1), T);
+      crec[C_N * t + C_NTAU] = p_set(-relaxation_rate<real>(in.tau_mode, rcp_rn(F32 ? real(in.kn_f) : real(in.kn)), nn, T));
     }
     real* mt = mv + t * 4 * MAXN;  // moment vectors [axis * 2 + side][s]
     if (hl < 4 && has) {
@@ -712,30 +710,38 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
     P fm = win.face_checked(side);
     // F_l of the next cell is loaded one cell ahead (a global load, the only one of the walk)
     P fl_next = need_fl ? p_load(Fl) : p_set(real(0));
-// (two cells a pass: fully unrolled, the walk outruns the instruction cache -- batch of 256
-// instances 5.18 ms a call, 4.99 ms so)
-#pragma unroll 2
+// (all cells in one body, left by a break at the last: two cells a pass under a guard issue 56e6 ALU
+// and 177e6 instructions a launch at a batch of 128 instances, this 34e6 and 145e6 -- the walk's state
+// changes its names, not its registers; 4.96 ms a call at a batch of 256, 4.82 ms so)
+#pragma unroll
     for (int t = 0; t < TC; ++t) {
-      if (t < TCe) {
-        const P fl = fl_next;
-        if (need_fl && t + 1 < TCe) fl_next = p_load(Fl + (t + 1) * row);
-        win.push(adv_val(t + 5 + o));
-        const P fp = win.face_checked(side);
-        // -adv = -p^R (cp F_{s+1/2} - cm F_{s-1/2}); per-cell factors: shared-memory broadcasts
-        P nadv = p_mul(p_fma(fp, ccp[t], p_mul(fm, cNcm[t])), npr);
-        const P Dc = p_load(S + (t + 3) * row);  // the cell's D
-        if constexpr (FT) nadv = p_fma(p_set(-pr * Rr), p_add(ccp[t], cNcm[t]), nadv);  // the advection of R
-        // f_eq - R for both fields: (g, T g) - R
-        const P deq = p_fma(p_mul(gRn[t * MAXQ + i], gP[t * MAXQ + j]), cT1[t], nrij);
-        P force = p_load(lbuf + t * row + 2 * v);
-        if constexpr (FT) force = p_sub(force, FRv);
-        // L = -adv + force / Rbar - (D - D_eq) / tau
-        const P Lv = p_fma(p_sub(Dc, deq), cNtau[t], p_fma(force, cIR[t], nadv));
-        P o = p_fma(Lv, p_set(cc), Dc);
-        if (need_fl) o = p_fma(p_sub(fl, Dc), p_set(ca), o);
-        p_store(S + (t + 3) * row, o);  // in place: this column's slot t+3 is not read again
-        fm = fp;
+      if (t >= TCe) break;
+      const P fl = fl_next;
+      if (need_fl && t + 1 < TCe) fl_next = p_load(Fl + (t + 1) * row);
+      win.push(adv_val(t + 5 + o));
+      const P fp = win.face_checked(side);
+      // -adv = -p^R (cp F_{s+1/2} - cm F_{s-1/2}); per-cell factors: shared-memory broadcasts
+      P cp, ncm, ir, ntau;
+      const P2* cr = crec + C_N * t;
+      if constexpr (F32) {
+        const float4 x = *reinterpret_cast<const float4*>(cr + C_CP), y = *reinterpret_cast<const float4*>(cr + C_IR);
+        cp = p_make(x.x, x.y), ncm = p_make(x.z, x.w), ir = p_make(y.x, y.y), ntau = p_make(y.z, y.w);
+      } else {
+        cp = cr[C_CP], ncm = cr[C_NCM], ir = cr[C_IR], ntau = cr[C_NTAU];
       }
+      P nadv = p_mul(p_fma(fp, cp, p_mul(fm, ncm)), npr);
+      const P Dc = p_load(S + (t + 3) * row);  // the cell's D
+      if constexpr (FT) nadv = p_fma(p_set(-pr * Rr), p_add(cp, ncm), nadv);  // the advection of R
+      // f_eq - R for both fields: (g, T g) - R
+      const P deq = p_fma(p_mul(gRn[t * MAXQ + i], gP[t * MAXQ + j]), cr[C_1T], nrij);
+      P force = p_load(lbuf + t * row + 2 * v);
+      if constexpr (FT) force = p_sub(force, FRv);
+      // L = -adv + force / Rbar - (D - D_eq) / tau
+      const P Lv = p_fma(p_sub(Dc, deq), ntau, p_fma(force, ir, nadv));
+      P o = p_fma(Lv, p_set(cc), Dc);
+      if (need_fl) o = p_fma(p_sub(fl, Dc), p_set(ca), o);
+      p_store(S + (t + 3) * row, o);  // in place: this column's slot t+3 is not read again
+      fm = fp;
     }
   }
   // ---- bulk store of the owned cells (generic-proxy writes made visible to the async proxy first)
