@@ -60,8 +60,7 @@ WORKLOAD = (f"gradually expanding channel: {CH_NX} (xi) x {CH_NL} (lambda) cells
 # DRAM bytes (read + write) per launch of the channel stage kernel from one ncu capture, keyed by
 # the SHA-256 of the kernel's code at the time of the capture (a changed kernel reports null):
 # see profiles/ for the command and the scaling to the full grid
-CH_TRAFFIC = {"2136950b3e5fe6b7": 4.449e9, "430a6d91e4dc5596": 4.397e9, "70feb0c42dc71e10": 4.385e9,
-              "26f60cccea2d0a70": 4.395e9}
+CH_TRAFFIC = {"75dd4185db98bef9": 4.227e9}
 
 
 def dist_env():
@@ -444,12 +443,11 @@ def bench_channel(args, torch, stream, vlb, world):
         "value": value, "ms_per_step": total_ms / args.steps, "units": units, "clocks": clocks,
         "launches": 3 * args.steps,
         "launch_shape": {"rows_per_segment": shape[0], "columns_per_strip": shape[1], "threads": shape[2],
-                         "force": "tensor cores (mma.sync TF32, hi/lo split)" if tensor_cores
+                         "force": "tensor cores" if tensor_cores
                                   else "CUDA cores (packed FP32x2, reflection-split matrices)",
                          "autotuned": True},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-                     "traffic": traffic, "kernel": f"channel_stage_kernel<float, 16, 12, {shape[1]}, "
-                                                   f"{'true' if tensor_cores else 'false'}>",
+                     "traffic": traffic, "kernel": "channel_stage_kernel<float, 16, 12, 0, false, false>",
                      "kernel_source_sha": sha, "peak_source": f"{kind} hbm_gbs",
                      "algorithmic_bytes_per_launch": bytes_per_launch, "launch_ms": launch_ms,
                      "launch_ms_by_stage": [float(stage_ms[k::3].mean()) for k in range(3)]},

@@ -160,9 +160,9 @@ vlb_status vlb_create_channel(const vlb_model* model, vlb_precision prec, const 
  * number (0 for Couette contexts, negative on error).  Arrays may be NULL. */
 int vlb_channel_variants(const vlb_ctx* ctx, int* ts, int* tp, int* nt, int max);
 
-/* Force contraction of channel launch shape v: 1 on the tensor cores (single
- * precision, TF32 with hi/lo operand splits), 0 on the CUDA cores (packed
- * FP32x2, or FP64 in double precision); negative on error. */
+/* Force contraction of channel launch shape v: 1 on the tensor cores, 0 on the
+ * CUDA cores (packed FP32x2, or FP64 in double precision), which every shape
+ * uses; negative on error. */
 int vlb_channel_variant_tensor_cores(const vlb_ctx* ctx, int v);
 
 /* Total number of cells over all instances, nodes per cell (nq0 * nq1), and

@@ -175,37 +175,6 @@ __device__ __noinline__ void weno5_weights_slow(real s1, real s2, real s3, real*
   }
 }
 
-template <typename real>
-__device__ __forceinline__ real weno5(real a, real b, real c, real d, real e, real sc) {
-  const real k1312 = real(13) / real(12), q = real(0.25);
-  const real d1 = real(0.1), d2 = real(0.6), d3 = real(0.3);
-  const real F1 = a * (real(1) / real(3)) - b * (real(7) / real(6)) + c * (real(11) / real(6));
-  const real F2 = -b * (real(1) / real(6)) + c * (real(5) / real(6)) + d * (real(1) / real(3));
-  const real F3 = c * (real(1) / real(3)) + d * (real(5) / real(6)) - e * (real(1) / real(6));
-  const real A = a * sc, B = b * sc, Cc = c * sc, D = d * sc, E = e * sc;
-  real t = A - real(2) * B + Cc;
-  real u = A - real(4) * B + real(3) * Cc;
-  real s1 = k1312 * t * t + q * u * u;
-  t = B - real(2) * Cc + D;
-  u = B - D;
-  real s2 = k1312 * t * t + q * u * u;
-  t = Cc - real(2) * D + E;
-  u = real(3) * Cc - real(4) * D + E;
-  real s3 = k1312 * t * t + q * u * u;
-  const real r = vdiv(real(1), vmax(s1, vmax(s2, s3)));
-  const real x1 = s1 * r, x2 = s2 * r, x3 = s3 * r;
-  const real P = x1 * x1, Qv = x2 * x2, R = x3 * x3;
-  real w1 = d1 * (Qv * R), w2 = d2 * (P * R), w3 = d3 * (P * Qv);
-  real den = w1 + w2 + w3;
-  if (!(den > real(0)) || !(den < real(1e30))) {
-    real w[3];
-    weno5_weights_slow<real>(s1, s2, s3, w);
-    w1 = w[0], w2 = w[1], w3 = w[2];
-    den = w1 + w2 + w3;
-  }
-  return vdiv(w1 * F1 + w2 * F2 + w3 * F3, den);
-}
-
 // ---------------------------------------------------------------- pairs (f', f'') of one velocity
 // Device rows interleave the two reduced distributions of Sec. II: element
 // (field d, velocity v) of a cell row sits at 2 v + d, so one 8- or 16-byte
@@ -269,12 +238,13 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// weno5 on a pair of fields: the candidate reconstructions, the indicators
+// The reconstruction on a pair of fields: the candidates, the indicators
 // (times 4, which the normalisation removes) and the weights run on the pair;
 // only the maxima, the reciprocals and the test for the slow path are per
 // field.  The weighted sum is normalised once at the end.  The weights are
 // products and sums of p_mul / p_add, so a cell gets the same bits at every
 // position of an unrolled walk and the result does not depend on the tile shape.
+//
 // The reconstruction of both fields from their indicators and candidates, as the
 // fast path of weno5p computes it, with the Table IV weights of weno5_weights_slow
 // for each field whose fast-path denominator den is out of range (fast holds the
@@ -352,8 +322,7 @@ __device__ __forceinline__ pair_t<real> weno5p(pair_t<real> a, pair_t<real> b, p
 // on the fast path; one zero then gets all the weight there, two take weno_corr_slow.)
 // Power-of-two scaling keeps the scaled values exact; a face value is scaled back by its inverse.
 // 34 packed operations per interface against 52 of weno5p, whose bound (the FP32 pipe, 128 fma
-// per clock and SM, packed or not) it shares; written with few constants, since a packed operand
-// is a register pair, which the compiler rebuilds at every use once registers run out.
+// per clock and SM, packed or not) it shares.
 template <typename real>
 struct WenoSide {  // per velocity: 3 side and the ideal weights of the - and + stencils over the middle one's
   pair_t<real> h3, dm, dp;
@@ -663,25 +632,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
                : "memory");
 }
 
-// Plain arrival (one of the counted arrivals of the current phase).
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Named CTA barrier `id` over `count` threads (a multiple of 32), and its AND reduction.
-__device__ __forceinline__ void named_bar(int id, int count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-__device__ __forceinline__ bool named_bar_and(int id, int count, bool v) {
-  unsigned r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"(unsigned(v)), "r"(id), "r"(count)
-      : "memory");
-  return r != 0;
-}
-
 // One-dimensional bulk copy global -> shared completing on the mbarrier (16-byte
 // aligned addresses, size a multiple of 16).
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
@@ -699,13 +649,7 @@ __device__ __forceinline__ void bulk_s2g(void* dst, const void* src, unsigned by
                : "memory");
 }
 
-// Commit the issued bulk stores and wait until their shared-memory sources have been read.
-__device__ __forceinline__ void bulk_commit_and_wait_read() {
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-
-// The same in parts: commit the issued bulk stores as a group; wait until every
+// Commit the issued bulk stores as a group; wait until every
 // committed group of this thread has read its shared-memory source; wait until
 // every committed group has completed.
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
