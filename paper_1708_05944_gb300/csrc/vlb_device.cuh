@@ -563,17 +563,29 @@ __device__ __forceinline__ void eq_moment_vector(int kind, int N, R u, R T, R* m
   }
 }
 
+// 1 / sqrt(2 pi T), the peak of the unit Gaussian of variance T.  Every half-range equilibrium factor
+// carries it, so a rounding that is the same in all cells would not average out: in single
+// precision 2 pi T is held as a pair (the constant alone rounds by 2.8e-8; 1 / sqrt(pi) by
+// 5.2e-8) and one step of Newton's iteration takes the rest of it and the instruction's error out.
+__device__ __forceinline__ float gauss_peak(float T) {
+  const float hi = 6.2831854820251464844f, lo = -1.7484555e-7f;  // 2 pi = hi + lo
+  const float y = __fmul_rn(hi, T), yl = __fmaf_rn(lo, T, __fmaf_rn(hi, T, -y));
+  const float r = rsqrtf(y), yr = __fmul_rn(y, r);
+  const float e = __fmaf_rn(-yr, r, 1.0f) - __fmaf_rn(__fmaf_rn(y, r, -yr), r, yl * (r * r));
+  return __fmaf_rn(0.5f * r, e, r);
+}
+__device__ __forceinline__ double gauss_peak(double T) { return rsqrt(6.28318530717958647692 * T); }
+
 // Moment vector of the truncated equilibrium on one axis (the recurrences of eq_moment_vector),
-// every entry up to order nmax, with the 1/l factors as constants and one reciprocal of T.
+// every entry up to order nmax, with the 1/l factors as constants.
 template <typename R>
 __device__ __forceinline__ void eq_moments_fast(int kind, int nmax, R u, R T, R* m) {
   R a, b, c;  // m_l = (u m_{l-1} + h c m_{l-2}) f: h = 1, f = 1 / l (full range) or h = l - 1, f = 1
   if (kind == 0) {
     a = R(1), b = u, c = T - R(1);
   } else {
-    const R is2T = rsqrt_t(R(2) * T);
-    const R x = u * is2T;
-    const R g0 = exp_t(-x * x) * is2T * R(0.56418958354775628695);  // N(0; u, T) = e^.. / sqrt(2 pi T)
+    const R x = u * rsqrt_t(R(2) * T);
+    const R g0 = exp_t(-x * x) * gauss_peak(T);  // N(0; u, T)
     a = R(0.5) * (R(1) + erf_t<R>(x));
     b = u * a + T * g0, c = T;
   }
