@@ -319,7 +319,7 @@ __device__ __forceinline__ pair_t<real> weno5p(pair_t<real> a, pair_t<real> b, p
 // value is the cell's own plus a correction.
 // (A constant far below any non-zero indicator stands for an exact zero in 13/3 S^2, so that a
 // uniform stretch, all three indicators zero, takes the ideal weights and the value of its cells
-// on the fast path; one zero then gets all the weight there, two take weno_corr_slow.)
+// on the fast path, and one or two zeros get all the weight.)
 // Power-of-two scaling keeps the scaled values exact; a face value is scaled back by its inverse.
 // 34 packed operations per interface against 52 of weno5p, whose bound (the FP32 pipe, 128 fma
 // per clock and SM, packed or not) it shares.
@@ -348,17 +348,22 @@ __device__ __forceinline__ double weno_pow2_dev(double inv_w) {
   return __hiloint2double(__double2hiint(inv_w) & 0x7ff00000, 0);
 }
 
-// 2^-e with e the exponent of the largest of three numbers >= 0 (Inf and the top binade give values
-// the caller's test of the weight sum rejects; zeros a large power).  Integer compares in double
-// precision: the comparison instructions of the FP64 pipe run at its 1/64 rate.
-__device__ __forceinline__ float inv_pow2_max(float a, float b, float c) {
-  float m;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
-  return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
+// A power of two close to 1 / sqrt(s1 s2), s1 and s2 the two largest of three positive numbers: half
+// the sum of their bit patterns is the bit pattern of about sqrt(s1 s2).  With it the largest product of
+// two scaled numbers lies in [1/4, 9/8], however far apart the three are, and the weights never leave
+// the range: over a resting field, where two of three indicators vanish at many faces, scaling by the
+// largest one sent whole warps to weno_corr_slow (2048 x 512 x 192 channel from rest, a step: 19.2 ms
+// with that, 10.1 so).  (Double precision: the high words; the comparison instructions of the FP64
+// pipe run at its 1/64 rate.)  Inf, NaN and two numbers in the top binade give a sum of weights of 0,
+// Inf or NaN, and so a face of NaN (0 * Inf).
+__device__ __forceinline__ unsigned inv_sqrt_bits(unsigned a, unsigned b, unsigned c, unsigned twice_inv, unsigned exponent) {
+  return ((twice_inv - (a + b + c) + min(a, min(b, c))) >> 1) & exponent;
 }
-__device__ __forceinline__ double inv_pow2_max(double a, double b, double c) {
-  const int m = max(__double2hiint(a), max(__double2hiint(b), __double2hiint(c)));
-  return __hiloint2double(0x7fe00000 - (m & 0x7ff00000), 0);
+__device__ __forceinline__ float inv_pow2_top(float a, float b, float c) {
+  return __uint_as_float(inv_sqrt_bits(__float_as_uint(a), __float_as_uint(b), __float_as_uint(c), 0xfe000000u, 0x7f800000u));
+}
+__device__ __forceinline__ double inv_pow2_top(double a, double b, double c) {
+  return __hiloint2double(int(inv_sqrt_bits(__double2hiint(a), __double2hiint(b), __double2hiint(c), 0xffc00000u, 0x7ff00000u)), 0);
 }
 __device__ __forceinline__ float2 p_rcp(float2 x) {  // 1 / x of normal numbers, about 1 ulp
   float2 r;
@@ -377,13 +382,15 @@ __device__ __forceinline__ double2 p_rcp(double2 x) {
   r = fma(r, fma(-y, r, 1.0), r);
   return make_double2(__dmul_rn(r, x.y), __dmul_rn(r, x.x));
 }
-// sums of weights the fast path accepts: their reciprocals (and, in double, the product of two) are normal
-__device__ __forceinline__ bool weno_in_range(float2 d) {
-  return (d.x > 1e-30f) & (d.x < 1e30f) & (d.y > 1e-30f) & (d.y < 1e30f);
+// Whether the fast weights gave both values of a face (see inv_pow2_top).  (Double precision: the
+// fields share a reciprocal, p_rcp, so that one tells for both; its high word, for the reason above.)
+__device__ __forceinline__ bool weno_holds(float2 f) {
+  unsigned nan;
+  asm("{\n .reg .pred p;\n setp.nan.f32 p, %1, %2;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(nan) : "f"(f.x), "f"(f.y));
+  return nan == 0;
 }
-__device__ __forceinline__ bool weno_in_range(double2 d) {  // 2^-465 (1e-140) .. 2^465, by the high words
-  const unsigned lo = 0x22e00000u, n = 0x5d000000u - 0x22e00000u;
-  return (unsigned(__double2hiint(d.x)) - lo < n) & (unsigned(__double2hiint(d.y)) - lo < n);
+__device__ __forceinline__ bool weno_holds(double2 f) {
+  return (unsigned(__double2hiint(f.x)) & 0x7fffffffu) < 0x7ff80000u;
 }
 
 // 13/3 S^2, an exact zero raised to a constant that no other indicator comes near
@@ -408,8 +415,8 @@ __device__ __forceinline__ float ratio_to(float num, float s) {
 }
 __device__ __forceinline__ double ratio_to(double num, double s) { return num / s; }
 
-// sum_q w_q (candidate_q - G_c) / sum_q w_q, the correction of the cell value, in any case: Table
-// IV for vanishing indicators, delta_q (sigma_min / sigma_q)^2 where the fast weights leave their range.
+// sum_q w_q (candidate_q - G_c) / sum_q w_q, the correction of the cell value, where the fast weights do not
+// hold: Table IV for vanishing indicators, delta_q (sigma_min / sigma_q)^2 otherwise.
 template <typename real>
 __device__ __forceinline__ real weno_corr_slow1(real sm, real s0, real sp, real dm, real dc, bool up) {
   const real k = real(13) / real(3);
@@ -436,41 +443,29 @@ __device__ __forceinline__ pair_t<real> weno_corr_slow(const WenoTerms<real>& t,
                 weno_corr_slow1<real>(t.sm.y, t.s0.y, t.sp.y, t.dm.y, t.dc.y, up));
 }
 
-// Range of the weight sums of several faces: the fast weights of all of them hold if ok().  (A test
-// and a rarely taken branch at every face cost registers, code and issue slots.)
+// Whether the fast weights hold for several faces.  (A test and a rarely taken branch at every face
+// cost registers, code and issue slots.)
 template <typename real>
-struct WenoRange;
-template <>
-struct WenoRange<float> {
-  float lo = 1.0f, hi = 1.0f;
-  __device__ __forceinline__ void add(float2 d) {
-    asm("min.NaN.f32 %0, %0, %1, %2;" : "+f"(lo) : "f"(d.x), "f"(d.y));
-    asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(hi) : "f"(d.x), "f"(d.y));
-  }
-  __device__ __forceinline__ bool ok() const { return (lo > 1e-30f) & (hi < 1e30f); }
-};
-template <>
-struct WenoRange<double> {
+struct WenoRange {
   bool good = true;
-  __device__ __forceinline__ void add(double2 d) { good = good && weno_in_range(d); }
+  __device__ __forceinline__ void add(pair_t<real> f) { good = good && weno_holds(f); }
   __device__ __forceinline__ bool ok() const { return good; }
 };
-// The value of a face from the cell's and its terms by the fast weights, whose sum den tells whether
-// they hold; K = false: k* are not read, 13/3 S^2 is formed here.
+// The value of a face from the cell's and its terms by the fast weights, NaN where they do not hold;
+// K = false: k* are not read, 13/3 S^2 is formed here.
 template <typename real, bool K>
 __device__ __forceinline__ pair_t<real> weno_face(pair_t<real> g0, const WenoTerms<real>& t, pair_t<real> km,
-                                                  pair_t<real> k0, pair_t<real> kp, const WenoSide<real>& w,
-                                                  pair_t<real>& den) {
+                                                  pair_t<real> k0, pair_t<real> kp, const WenoSide<real>& w) {
   using P = pair_t<real>;
   const P um = p_add(p_add(t.dm, t.dm), t.sm), u0 = p_add(t.dm, t.dc), up = p_sub(p_add(t.dc, t.dc), t.sp);
   auto sq = [](P s) { return weno_sq<real>(s); };
   const P bm = p_fma(um, um, K ? km : sq(t.sm)), b0 = p_fma(u0, u0, K ? k0 : sq(t.s0)),
           bp = p_fma(up, up, K ? kp : sq(t.sp));
-  const P r = p_make(inv_pow2_max(bm.x, b0.x, bp.x), inv_pow2_max(bm.y, b0.y, bp.y));
-  const P xm = p_mul(bm, r), x0 = p_mul(b0, r), xp = p_mul(bp, r);  // the largest in [1, 2)
+  const P r = p_make(inv_pow2_top(bm.x, b0.x, bp.x), inv_pow2_top(bm.y, b0.y, bp.y));
+  const P xm = p_mul(bm, r), x0 = p_mul(b0, r), xp = p_mul(bp, r);
   const P A = p_mul(x0, xp), B = p_mul(xm, xp), C = p_mul(xm, x0);
   const P wm = p_mul(p_mul(A, A), w.dm), w0 = p_mul(B, B), wp = p_mul(p_mul(C, C), w.dp);
-  den = p_add(p_add(wm, w0), wp);
+  const P den = p_add(p_add(wm, w0), wp);
   const P qm = p_fma(um, w.h3, t.sm), q0 = p_fma(u0, w.h3, t.s0), qp = p_fma(up, w.h3, t.sp);
   const P num = p_fma(wm, qm, p_fma(w0, q0, p_mul(wp, qp)));
   const P i = p_rcp(den);
@@ -500,29 +495,25 @@ struct WenoWin {
     if constexpr (K) km = k0, k0 = kp, kp = weno_sq<real>(sp);
   }
   __device__ __forceinline__ WenoTerms<real> terms() const { return WenoTerms<real>{sm, s0, sp, dm, dc}; }
-  __device__ __forceinline__ P fast(const WenoSide<real>& w, P& den) const {
-    if constexpr (K) return weno_face<real, true>(g0, terms(), km, k0, kp, w, den);
-    else return weno_face<real, false>(g0, terms(), sm, sm, sm, w, den);
+  __device__ __forceinline__ P fast(const WenoSide<real>& w) const {
+    if constexpr (K) return weno_face<real, true>(g0, terms(), km, k0, kp, w);
+    else return weno_face<real, false>(g0, terms(), sm, sm, sm, w);
   }
   // the interface value on the cell's side w (times the scale of G), where the range stays ok
   __device__ __forceinline__ P face(const WenoSide<real>& w, WenoRange<real>& range) const {
-    P den;
-    const P f = fast(w, den);
-    range.add(den);
+    const P f = fast(w);
+    range.add(f);
     return f;
   }
   __device__ __forceinline__ bool in_range(bool up) const {  // whether face() holds for this face
-    P den;
     WenoSide<real> w;
     w.set(up);
-    fast(w, den);
-    return weno_in_range(den);
+    return weno_holds(fast(w));
   }
   // the value, checked at once
   __device__ __forceinline__ P face_checked(const WenoSide<real>& w) const {
-    P den;
-    P f = fast(w, den);
-    if (__builtin_expect(!weno_in_range(den), 0)) f = face_any(w.h3.x > real(0));
+    P f = fast(w);
+    if (__builtin_expect(!weno_holds(f), 0)) f = face_any(w.h3.x > real(0));
     return f;
   }
   // the value in any case
