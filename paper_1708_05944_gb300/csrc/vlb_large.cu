@@ -8,7 +8,8 @@
 //             macro_red, mom_quad), and per wall and chunk the outgoing WENO-5 flux of the
 //             extrapolated populations (Eqs. extrapol, nw), FP64, spread over many CTAs;
 //   cell   -- per cell n, u, T from its chunk sums (in a fixed order), tau and the
-//             truncated equilibrium factors (Sec. IV.D) normalised to sum n; beside it, on
+//             truncated equilibrium factors (Sec. IV.D) normalised to sum n, and for the cell
+//             next to a wall that wall's n_w; beside it, on
 //             other CTAs of the same launch (neither needs the other),
 //   force  -- the radial part of the inertial term -(1/R)(p^phi)^2 K^R f (Eq.
 //             boltz_couette_kom): per cell the contraction over the nq0 radial nodes is
@@ -21,8 +22,11 @@
 //             difference, the azimuthal part of the inertial term (nq1 terms), BGK and
 //             the RK3 combine, both fields as a pair.
 // Every sum is taken in a fixed order, so results do not depend on scheduling.  What bounds it at
-// the sizes it is run at (16 cells): the latency of the three kernels' chains.  16 cells x 1600
-// velocities, single precision, a stage: 40.7 us in five launches, 33.3 us in three.
+// the sizes it is run at (16 cells): the latency of the three kernels' chains.  Single precision, an RK3
+// step from graph replay: 16 cells x 1600 velocities 114 us in five launches, 81 us in three; 16 x 8000
+// 200 us and 194 us (207 us with n_w summed anew by every incoming ghost, the walk's scale by
+// double-precision operations of every velocity, and 80 registers in the update, whose CTAs then take
+// a second round that is nearly empty).
 //
 // The same kernels run the f~ formulation (LargeModel::ftilde, Sec. VI.B): the stencils and
 // the wall construction act on F~ = sqrt(g) f, whose flux difference e_{s+1/2} F~_{s+1/2} -
@@ -76,11 +80,13 @@ __device__ __forceinline__ real weno_scale(double iw) {
 }
 
 // The power-of-two scale of the WENO walk, at most 2^100 in single precision (tail populations below
-// ~1e-38 are zero there, and for the others the weights do not see the scale).
+// ~1e-38 are zero there, and for the others the weights do not see the scale), from the exponents of
+// 1 / w_i and 1 / w_j.
 template <typename real>
 __device__ __forceinline__ real walk_scale(double iw0, double iw1) {
-  const double sc = weno_pow2_dev(iw0) * weno_pow2_dev(iw1);
-  return real(sizeof(real) == 4 ? fmin(sc, 0x1p100) : fmin(sc, 0x1p996));
+  const int e = (__double2hiint(iw0) >> 20) + (__double2hiint(iw1) >> 20) - 2046;
+  if constexpr (sizeof(real) == 4) return __int_as_float((min(e, 100) + 127) << 23);
+  else return __hiloint2double((min(e, 996) + 1023) << 20, 0);
 }
 
 // Equilibrium factors of (n, u0, u1, T) into g0 (carrying n, normalised so that
@@ -217,7 +223,8 @@ __global__ void __launch_bounds__(256) lm_sums_kernel(const LargeModel m, const 
 // rec per cell: g0 (nq0, carrying n), g1 (nq1), T, 1/tau; moments from the partial sums
 template <typename real>
 __device__ void lm_cell(const LargeModel& m, long long cells, int NP, const double* part, const InstDesc* inst,
-                        int n_inst, real* rec, int block, int blocks) {
+                        int n_inst, const double* walls, const double* wpart, double* nw, real* rec, int block,
+                        int blocks) {
   extern __shared__ double sh[];
   double* g0 = sh;
   double* g1 = g0 + m.nq0;
@@ -231,10 +238,23 @@ __device__ void lm_cell(const LargeModel& m, long long cells, int NP, const doub
       for (int p = 0; p < NP; ++p) t += part[(c * NP + p) * 4 + threadIdx.x];
       q[threadIdx.x] = t;
     }
+    const int ii = instance_of(inst, n_inst, c);
+    const InstDesc& d = inst[ii];
+    // the wall next to this cell: n_w of Eq. (nw) from its chunk sums, in a fixed order (one thread of another
+    // warp, beside the cell's own sums)
+    if (threadIdx.x == 32 || threadIdx.x == 64) {
+      const int wall = threadIdx.x == 32 ? 0 : 1;
+      if (c == d.cell0 + (wall == 0 ? 0 : d.n_cells - 1)) {
+        double t = m.ftilde ? 0.0 : (wall == 0 ? m.ref_flux_neg : m.ref_flux_pos);  // f~: no R split
+        for (int p = 0; p < NP; ++p) t += wpart[(size_t(ii) * 2 + wall) * NP + p];
+        const double nwv = -t / walls[(size_t(ii) * 2 + wall) * (m.nq0 + m.nq1 + 2) + m.nq0 + m.nq1];
+        nw[ii * 2 + wall] = nwv;
+        if (!isfinite(nwv)) atomicOr(m.err, ERR_NONFINITE);
+      }
+    }
     __syncthreads();
     const double n = q[0], u0 = q[1] / n, u1 = q[2] / n;
     const double T = (q[3] / n - u0 * u0 - u1 * u1) / 3.0;
-    const InstDesc& d = inst[instance_of(inst, n_inst, c)];
     const double tau = relaxation_time<double>(d.tau_mode, d.kn, n, T);
     eq_factors(m, n, u0, u1, T, g0, g1, mv, red);
     real* o = rec + c * stride;
@@ -313,12 +333,13 @@ __device__ void lm_force(const LargeModel& m, const real* F, const GeoCell* geo,
 template <typename real>
 __global__ void __launch_bounds__(FT) lm_cell_force_kernel(const LargeModel m, const real* F, const GeoCell* geo,
                                                            real* out, long long cells, int NP, const double* part,
-                                                           const InstDesc* inst, int n_inst, real* rec, int cblocks,
+                                                           const InstDesc* inst, int n_inst, const double* walls,
+                                                           const double* wpart, double* nw, real* rec, int cblocks,
                                                            int ny, int nz) {
   grid_launch_dependents();
   grid_dependency_wait();
   if (int(blockIdx.x) < cblocks) {
-    lm_cell<real>(m, cells, NP, part, inst, n_inst, rec, int(blockIdx.x), cblocks);
+    lm_cell<real>(m, cells, NP, part, inst, n_inst, walls, wpart, nw, rec, int(blockIdx.x), cblocks);
   } else {
     const long long b = (long long)blockIdx.x - cblocks;
     const int t = int(b % (ny * nz));
@@ -327,12 +348,12 @@ __global__ void __launch_bounds__(FT) lm_cell_force_kernel(const LargeModel m, c
 }
 
 // ---------------------------------------------------------------- update kernel
-constexpr int UT = 128;  // velocities per CTA
+constexpr int UT = 128;  // velocities per CTA (seven a SM: 16 cells x 8000 velocities are 1008 CTAs, one round)
 template <typename real>
-__global__ void __launch_bounds__(UT) lm_update_kernel(const LargeModel m, const real* Fprev, const real* Fl, real* Fout, long long cells,
-                                 const InstDesc* inst, int n_inst, const GeoCell* geo, const real* rec,
-                                 const real* force, const double* walls, const double* wpart, int NP, double* nw,
-                                 double ca, double cc) {
+__global__ void __launch_bounds__(UT, 7)
+    lm_update_kernel(const LargeModel m, const real* Fprev, const real* Fl, real* Fout, long long cells,
+                     const InstDesc* inst, int n_inst, const GeoCell* geo, const real* rec, const real* force,
+                     const double* walls, const double* nw, double ca, double cc) {
   using P = pair_t<real>;
   constexpr bool F32 = sizeof(real) == 4;
   const int stride = m.nq0 + m.nq1 + 2, per = (m.V + UT - 1) / UT;  // CTAs per cell
@@ -347,11 +368,6 @@ __global__ void __launch_bounds__(UT) lm_update_kernel(const LargeModel m, const
     const InstDesc& d = inst[ii];
     const int s = int(c - d.cell0), n = d.n_cells;
     const double Rd = m.w0[i] * m.w1[j];
-    auto wall_density = [&](int wall) {  // n_w of Eq. (nw) from the chunk sums, in a fixed order
-      double t = m.ftilde ? 0.0 : (wall == 0 ? m.ref_flux_neg : m.ref_flux_pos);  // f~: no R split
-      for (int p = 0; p < NP; ++p) t += wpart[(size_t(ii) * 2 + wall) * NP + p];
-      return -t / walls[(size_t(ii) * 2 + wall) * (m.nq0 + m.nq1 + 2) + m.nq0 + m.nq1];
-    };
     // the advected value of a cell: D (chi), or F~ = sqrt(g) (D + R) (f~)
     auto cell = [&](long long cc) -> P {
       const P x = p_load(Fprev + cc * 2 * m.Vp + 2 * v);
@@ -368,7 +384,7 @@ __global__ void __launch_bounds__(UT) lm_update_kernel(const LargeModel m, const
         return p_fma(F1, p_set(real(-8)), p_fma(F0, p_set(real(6)), p_mul(F2, p_set(real(3)))));
       }
       const double* wt = walls + (size_t(ii) * 2 + wall) * (m.nq0 + m.nq1 + 2);
-      const double e = wall_density(wall) * wt[i] * wt[m.nq0 + j];
+      const double e = nw[ii * 2 + wall] * wt[i] * wt[m.nq0 + j];
       const double r = m.ftilde ? 0.0 : Rd;  // f~ ghosts are F~ itself
       return p_make(real(e - r), real(e * wt[m.nq0 + m.nq1 + 1] - r));
     };
@@ -378,13 +394,6 @@ __global__ void __launch_bounds__(UT) lm_update_kernel(const LargeModel m, const
       if (t >= n) return ghost(1, t - n + 1);
       return cell(c + k);
     };
-    if (v == 0 && (s == 0 || s == n - 1))  // the wall densities of the stage, for vlb_wall_density
-      for (int wall = 0; wall < 2; ++wall)
-        if ((wall == 0 && s == 0) || (wall == 1 && s == n - 1)) {
-          const double nwv = wall_density(wall);
-          nw[ii * 2 + wall] = nwv;
-          if (!isfinite(nwv)) atomicOr(m.err, ERR_NONFINITE);
-        }
     const P F0 = p_load(Fprev + c * 2 * m.Vp + 2 * v);  // the cell's own D
     // both interfaces by the walk of the fused kernel: the upwind cells are s - 1, s for p^R >= 0 and
     // s, s + 1 otherwise
@@ -696,10 +705,10 @@ cudaError_t lm_stage(const LargeModel& m, const real* Fprev, const real* Fl, rea
                                    Fprev, cells, NP, inst, part, wpart);
   if (e == cudaSuccess)
     e = launch_dependent(lm_cell_force_kernel<real>, dim3(unsigned(cb + cells * ny * nz)), FT, cell_smem(m), s, m, Fprev,
-                         geo, force, cells, NP, part, inst, n_inst, rec, cb, ny, nz);
+                         geo, force, cells, NP, part, inst, n_inst, walls, wpart, nw, rec, cb, ny, nz);
   if (e == cudaSuccess)
     e = launch_dependent(lm_update_kernel<real>, dim3(unsigned(ub < 152 * 64 ? ub : 152 * 64)), UT, 0, s, m, Fprev, Fl,
-                         Fout, cells, inst, n_inst, geo, rec, force, walls, wpart, NP, nw, ca, cc);
+                         Fout, cells, inst, n_inst, geo, rec, force, walls, static_cast<const double*>(nw), ca, cc);
   return e;
 }
 
