@@ -355,34 +355,36 @@ vlb_status setup_large(vlb_ctx* c) {
   return VLB_OK;
 }
 
-// Rows per lambda segment and segments of a channel launch shape.  A fixed ts
-// is used as given (at least 3 rows per segment, the last one included); ts = 0
-// picks the segment count that minimises waves x (rows + 6) over the resident
-// CTAs of the device: the 6 rows are the warm-up of a segment (its first four
-// rows' loads, the windows below it and the equilibria of its first three rows).
-void channel_segments(const vlb_ctx* c, const ChanVariant& v, int* seglen, int* nseg) {
+// Rows per lambda segment, segments and kernel of a channel launch shape: those that minimise
+// waves x (rows + 6) x (time of a step) over the resident CTAs of the device, where the 6 rows are
+// the warm-up of a segment (its first four rows' loads, the windows below it and the equilibria of its
+// first three rows).  A fixed ts is used as given (at least 3 rows per segment, the last one
+// included); ts = 0 tries every segment count.
+void channel_segments(const vlb_ctx* c, const ChanVariant& v, bool clb, int* seglen, int* nseg, int* kernel) {
   const int nl = c->cdesc.nl, nstrips = c->cdesc.nx / v.tp;
   auto count = [&](int L) {  // segments of L rows, 0 if the last would be shorter than 3
     const int n = (nl + L - 1) / L;
     return nl - (n - 1) * L >= 3 ? n : 0;
   };
+  long long best = -1;
+  *seglen = nl, *nseg = 1, *kernel = 0;
+  auto offer = [&](int L, int n) {
+    for (int k = 0; k < c->n_chan_kernels; ++k) {
+      const ChanKernel& kn = c->chan_kernels[clb][k];
+      const long long slots = std::max(1, c->sms * kn.per_sm);
+      const long long cost = ((static_cast<long long>(nstrips) * n + slots - 1) / slots) * (L + 6) * kn.step;
+      if (best < 0 || cost < best) best = cost, *seglen = L, *nseg = n, *kernel = k;
+    }
+  };
   if (v.ts > 0) {
-    int L = std::max(3, std::min(v.ts, nl));
-    int n = count(L);
-    if (n == 0) L = nl, n = 1;
-    *seglen = L, *nseg = n;
+    const int L = std::max(3, std::min(v.ts, nl)), n = count(L);
+    offer(n == 0 ? nl : L, n == 0 ? 1 : n);
     return;
   }
-  const int sms = c->sms > 0 ? c->sms * c->chan_per_sm : 1;
-  long long best = -1;
-  *seglen = nl, *nseg = 1;
   for (int want = 1; want <= nl / 3; ++want) {
     const int L = (nl + want - 1) / want;
     const int n = count(L);
-    if (n == 0) continue;
-    const long long waves = (static_cast<long long>(nstrips) * n + sms - 1) / sms;
-    const long long cost = waves * (L + 6);
-    if (best < 0 || cost < best) best = cost, *seglen = L, *nseg = n;
+    if (n > 0) offer(L, n);
   }
 }
 
@@ -410,9 +412,10 @@ vlb_status do_chan_stage(vlb_ctx* c, int k, int prev, int out, bool clb = false)
   a.flow = c->cdesc.flow;
   a.qflow = static_cast<const real*>(c->d_qflow);
   const ChanVariant& v = c->cvariants[c->variant];
-  channel_segments(c, v, &a.seglen, &a.nseg);
+  int kernel = 0;
+  channel_segments(c, v, clb, &a.seglen, &a.nseg, &kernel);
   const int grid = (a.nx / v.tp) * a.nseg;
-  cudaError_t e = launch_channel<real>(a, c->chan_kp.data(), c->nq0, c->nq1, c->margs.kind1, grid, c->stream, clb);
+  cudaError_t e = launch_channel<real>(a, c->chan_kp.data(), c->nq0, c->nq1, c->margs.kind1, kernel, grid, c->stream, clb);
   if (e != cudaSuccess) return cuda_fail(c, e, "channel stage kernel launch");
   c->launches += 1;
   return VLB_OK;
@@ -978,16 +981,19 @@ vlb_status vlb_create_channel(const vlb_model* model, vlb_precision prec, const 
   c->Vp = (c->V + 3) / 4 * 4;
   c->esize = prec == VLB_FP64 ? 8 : 4;
   {
-    // launch shapes: shared memory within an SM's, whole strips of columns, the force block's structure
+    // launch shapes: whole strips of columns, the force block's structure
     const bool kp_ok = prec == VLB_FP64 ? channel_force_pairs<double>(nq0, nq1, c->ax, &c->chan_kp)
                                         : channel_force_pairs<float>(nq0, nq1, c->ax, &c->chan_kp);
     ChanVariant all[8];
     const int n = kp_ok ? channel_variants(nq0, nq1, all) : 0;
-    for (int i = 0; i < n; ++i) {
-      const size_t sm = prec == VLB_FP64 ? channel_smem_bytes<double>(all[i], nq0, nq1, &c->chan_per_sm)
-                                         : channel_smem_bytes<float>(all[i], nq0, nq1, &c->chan_per_sm);
-      if (!(sm > 0 && sm <= 227 * 1024 && nx % all[i].tp == 0)) continue;
-      c->cvariants[c->n_cvariants++] = all[i];
+    for (int i = 0; i < n; ++i)
+      if (nx % all[i].tp == 0) c->cvariants[c->n_cvariants++] = all[i];
+    for (int clb = 0; clb < 2 && c->n_cvariants > 0; ++clb) {
+      const int kind1 = model->kind[1] == VLB_HALF ? 1 : 0;
+      const cudaError_t e = prec == VLB_FP64
+                                ? channel_kernels<double>(nq0, nq1, kind1, clb, c->chan_kernels[clb], &c->n_chan_kernels)
+                                : channel_kernels<float>(nq0, nq1, kind1, clb, c->chan_kernels[clb], &c->n_chan_kernels);
+      if (e != cudaSuccess) return fail(nullptr, VLB_ERR_CUDA, std::string("channel kernel residency: ") + cudaGetErrorString(e));
     }
     // no vielbein kernel for this velocity set: the context can still run the Cartesian split
     if (c->n_cvariants == 0 && (nq0 > MAXQ || nq1 > MAXQ))
@@ -1871,8 +1877,8 @@ int vlb_channel_variants(const vlb_ctx* c, int* ts, int* tp, int* nt, int max) {
   if (!c) return VLB_ERR_INVALID;
   if (c->kind != 1) return 0;
   for (int v = 0; v < c->n_cvariants && v < max; ++v) {
-    int L = 0, n = 0;
-    channel_segments(c, c->cvariants[v], &L, &n);
+    int L = 0, n = 0, kernel = 0;
+    channel_segments(c, c->cvariants[v], c->clb_march, &L, &n, &kernel);
     if (ts) ts[v] = L;
     if (tp) tp[v] = c->cvariants[v].tp;
     if (nt) nt[v] = c->cvariants[v].nt;
@@ -1889,8 +1895,8 @@ int vlb_variants(const vlb_ctx* c, int* tc, int* nt, int* persistent, int max) {
   if (!c) return VLB_ERR_INVALID;
   if (c->kind == 1) {
     for (int v = 0; v < c->n_cvariants && v < max; ++v) {
-      int L = 0, n = 0;
-      channel_segments(c, c->cvariants[v], &L, &n);
+      int L = 0, n = 0, kernel = 0;
+      channel_segments(c, c->cvariants[v], c->clb_march, &L, &n, &kernel);
       if (tc) tc[v] = L * c->cvariants[v].tp;
       if (nt) nt[v] = c->cvariants[v].nt;
       if (persistent) persistent[v] = 0;

@@ -1,7 +1,7 @@
 // One TVD-RK3 stage of the gradually expanding channel in the vielbein frame
 // (Sec. VII.A-C, Eq. canalie_boltz), as a marching kernel: each CTA owns a
 // strip of TP = 4 adjacent xi-columns and walks up a segment of lambda rows
-// (wall-normal).  A thread owns one velocity on all four columns.  Step s of the march
+// (wall-normal).  A thread owns one velocity on all four columns (on one, see ChanSmem).  Step s of the march
 //
 //   - reconstructs the five xi interfaces of row s in one walk along the strip (the row and its
 //     halo come from a shared-memory ring that bulk copies fill) and the lambda interface of
@@ -118,16 +118,18 @@ struct ChanArgs {
 // moments, s+4 in flight (issued when step s begins, after the barrier that ends the use of row s-1).  Cells are padded so that the force tasks of neighbouring cells fall on consecutive
 // banks: cell stride = Q1 pairs modulo 128 bytes.
 //
-// XW: warps beside the NW that own velocities.  Small velocity sets (one warp) take three for the
-// roles of the rows ahead where the grid leaves SMs idle: a step then takes the time of its longest
-// part, not of their sum.
-template <typename real, int Q0, int Q1, int XW>
+// CG: groups of threads that share the strip's columns; XW: warps beside those that own velocities.  A
+// small velocity set (one warp) takes a warp per column and three for the roles of the rows ahead where
+// the grid leaves SMs idle: a step then takes the time of its longest part, not of their sum, and double
+// precision gets all of an SM's FP64 units.  The xi walk of a single column reconstructs two interfaces,
+// five for four columns, so it costs a sixth more arithmetic; the values are the same.
+template <typename real, int Q0, int Q1, int CG, int XW>
 struct ChanSmem {
   using S = ChanShape<Q0, Q1>;
   using Tab = ChanTables<real, Q0, Q1>;
   static constexpr bool F32 = sizeof(real) == 4;
   static constexpr int TP = S::TP;
-  static constexpr int NT = S::V + 32 * XW;
+  static constexpr int NT = S::V * CG + 32 * XW;
   static constexpr int NRING = 5;
   static constexpr int RC = TP + 6;  // cells of a ring row
   static constexpr int NEQ = 4;      // equilibrium records (rows s .. s+3)
@@ -155,9 +157,12 @@ struct ChanSmem {
   static_assert(ring_off % 16 == 0 && geo_off % 16 == 0 && lbl_off % 16 == 0 && lbx_off % 16 == 0, "alignment");
   static_assert(NRING * sizeof(uint64_t) <= tab_off, "mbarriers fit before the tables");
   static_assert((NEQ & (NEQ - 1)) == 0 && (NRES & (NRES - 1)) == 0, "record slots by mask");
-  // resident CTAs a SM the registers are sized for (228 KB of shared memory, 1 KB of it per CTA)
+  // CTAs a SM the registers are sized for (228 KB of shared memory, 1 KB of it per CTA; single
+  // precision: 168 registers a thread for four columns, 80 for one).  How many the device holds is
+  // asked of the driver (channel_kernels).
   static constexpr int fit = int((228 * 1024) / (bytes + 1024));
-  static constexpr int min_ctas = sizeof(real) == 8 ? 1 : (fit * NT * 168 <= 65536 ? fit : 65536 / (NT * 168));
+  static constexpr int regs = CG == 1 ? 168 : 96;
+  static constexpr int min_ctas = sizeof(real) == 8 ? 1 : (fit * NT * regs <= 65536 ? fit : 65536 / (NT * regs));
 };
 
 // Coefficients of a packed contraction: single precision holds each duplicated into a pair, the
@@ -340,19 +345,20 @@ __device__ __forceinline__ void channel_equilibrium(const ChanTables<real, Q0, Q
 // (c = 0).  The lambda upwind side and the wall's incoming half-plane (Eq. canalie_coord_nw)
 // then depend on the column and the interface: the lambda window holds the six cells around an
 // interface and the walk's terms are formed per interface from the five of the upwind side.
-template <typename real, int Q0, int Q1, int XW, bool CLB, bool HX>
-__global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real, Q0, Q1, XW>::min_ctas)
+template <typename real, int Q0, int Q1, int CG, int XW, bool CLB, bool HX>
+__global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, CG, XW>::NT, ChanSmem<real, Q0, Q1, CG, XW>::min_ctas)
     channel_stage_kernel(const __grid_constant__ ChanArgs<real> a, const __grid_constant__ ChanKP<real, Q0, Q1> kp) {
   using S = ChanShape<Q0, Q1>;
-  using L = ChanSmem<real, Q0, Q1, XW>;
+  using L = ChanSmem<real, Q0, Q1, CG, XW>;
   using Tab = ChanTables<real, Q0, Q1>;
   using P = pair_t<real>;
-  constexpr int V = S::V, ROW = S::ROW, EQW = S::EQW, TP = S::TP, NW = S::NW;
+  constexpr int V = S::V, ROW = S::ROW, EQW = S::EQW, TP = S::TP, NW = S::NW, CPT = TP / CG;
   constexpr int NRING = L::NRING, RC = L::RC, CS = L::CS, XS = L::XS;
   extern __shared__ __align__(128) unsigned char smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool col = XW == 0 || tid < V;  // owns a velocity of the four columns
-  const int v = col ? tid : lane;
+  const bool col = XW == 0 || tid < V * CG;  // owns a velocity of CPT columns, from c0
+  const int v = !col ? lane : CG == 1 ? tid : tid % V;
+  const int c0 = CG == 1 || !col ? 0 : tid / V * CPT;
   const int i = v / Q1, j = v - i * Q1;
 
   const int nl = a.nl, nx = a.nx;
@@ -445,8 +451,10 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
   // along xi, 4 takes the equilibria, 5 the inflow factors; with extra warps they share the same;
   // else the one warp takes all in turn.
   constexpr bool SPLIT = NW >= 6;
+  static_assert(CG == 1 || XW == 3, "column groups come with extra warps");
   static_assert(XW == 0 || XW == 3, "extra warps: lambda, xi, equilibria and inflow");
-  constexpr int WL = SPLIT ? 0 : XW ? NW : 0, WX = SPLIT ? 2 : XW ? NW + 1 : 0, WE = SPLIT ? 4 : XW ? NW + 2 : 0,
+  constexpr int CW = NW * CG;  // column warps
+  constexpr int WL = SPLIT ? 0 : XW ? CW : 0, WX = SPLIT ? 2 : XW ? CW + 1 : 0, WE = SPLIT ? 4 : XW ? CW + 2 : 0,
                 WR = SPLIT ? 5 : WE, FW = SPLIT ? 2 : 1;  // their first warps; warps of a contraction
   auto force_row = [&](int r) {
     if constexpr (!CLB) {
@@ -536,7 +544,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
     const int k = slot(r), rs = r & (L::NRES - 1);
 #pragma unroll
     for (int end = 0; end < 2; ++end) {
-      if (!(end == 0 ? inlet : outlet)) continue;
+      if (!(end == 0 ? inlet : outlet) || (CG > 1 && c0 != (end == 0 ? 0 : TP - CPT))) continue;
       const int ce = end == 0 ? 0 : TP - 1;
       const ChanCell<real>& g = gring[k * TP + ce];
       const real Vx = end == 0 ? g.bm * px - g.cm * pl : g.bp * px - g.cp * pl;
@@ -562,19 +570,20 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
   };
   // vielbein: the window centred on row s + off; Cartesian split: F(s-2 .. s+3) of step s (scaled).
   // Before the march's pass sA - 1, which brings in one row more and reconstructs interface sA - 1/2.
-  WenoWin<real, !L::F32> win[CLB ? 1 : TP];
-  P raw[CLB ? TP : 1][6];
-  P flo[TP];  // lambda interface s - 1/2 (scaled)
+  WenoWin<real, !L::F32> win[CLB ? 1 : CPT];
+  P raw[CLB ? CPT : 1][6];
+  P flo[CPT];  // lambda interface s - 1/2 (scaled)
   if (col)
 #pragma unroll
-  for (int c = 0; c < TP; ++c) {
+  for (int c = 0; c < CPT; ++c) {
+    const int cc = c0 + c;
     if constexpr (CLB) {
 #pragma unroll
-      for (int q = 1; q < 6; ++q) raw[c][q] = p_mul(low_row(sA - 4 + q, c), SC);
+      for (int q = 1; q < 6; ++q) raw[c][q] = p_mul(low_row(sA - 4 + q, cc), SC);
     } else {
       const int b = sA - 3 + off;
-      const P x = p_mul(low_row(b, c), SC);  // (its lower neighbour's terms leave the window at once)
-      win[c].start(x, x, p_mul(low_row(b + 1, c), SC), p_mul(low_row(b + 2, c), SC), p_mul(low_row(b + 3, c), SC));
+      const P x = p_mul(low_row(b, cc), SC);  // (its lower neighbour's terms leave the window at once)
+      win[c].start(x, x, p_mul(low_row(b + 1, cc), SC), p_mul(low_row(b + 2, cc), SC), p_mul(low_row(b + 3, cc), SC));
     }
     flo[c] = p_set(real(0));
   }
@@ -614,7 +623,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
   auto wall_density = [&]() {
     if (col)
 #pragma unroll 1
-    for (int c = 0; c < TP; ++c) {
+    for (int c = c0; c < c0 + CPT; ++c) {
       real fl = real(0), fd = real(0);
       const bool out = wall_out(c);
       real Vw = pl;
@@ -639,7 +648,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
         fl += __shfl_xor_sync(0xffffffffu, fl, o);
         if constexpr (CLB) fd += __shfl_xor_sync(0xffffffffu, fd, o);
       }
-      if (lane == 0) wred[c * NW + warp] = fl, wred[(TP + c) * NW + warp] = fd;
+      if (lane == 0) wred[c * NW + (v >> 5)] = fl, wred[(TP + c) * NW + (v >> 5)] = fd;
     }
     __syncthreads();
     if (tid < TP) {
@@ -657,7 +666,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
     __syncthreads();
     if (col)
 #pragma unroll 1
-    for (int c = 0; c < TP; ++c) {
+    for (int c = c0; c < c0 + CPT; ++c) {
       P G1, G2;
       if (wall_out(c)) {
         extrapolate(c, G1, G2);
@@ -671,12 +680,12 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
   };
 
   // this thread's F_l and F_out of the strip's first cell in row s; F_l is loaded one step ahead
-  const real* Fl = a.Fl + dcell(sA, p0) * ROW + 2 * v;
-  real* Fo = a.Fout + dcell(sA, p0) * ROW + 2 * v;
+  const real* Fl = a.Fl + dcell(sA, p0 + c0) * ROW + 2 * v;
+  real* Fo = a.Fout + dcell(sA, p0 + c0) * ROW + 2 * v;
   const size_t rstep = size_t(nx) * ROW;
-  P flr[TP];
+  P flr[CPT];
 #pragma unroll
-  for (int c = 0; c < TP; ++c) {
+  for (int c = 0; c < CPT; ++c) {
     flr[c] = p_set(real(0));
     if (need_fl && col) flr[c] = p_load(Fl + c * ROW);
   }
@@ -694,17 +703,17 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
     if (col) {
     const int k0 = full ? slot(s) : 0;
     const int k3 = slot(min(s + 2 + (CLB ? 1 : off), nl + 1));  // the row that joins the lambda windows
-    const ChanCell<real>* geo = gring + k0 * TP;
+    const ChanCell<real>* geo = gring + k0 * TP + c0;
     const P R2 = p_set(CLB ? Rij * SC.x : real(0));
 
     // ---- xi: V F (CLB: of F = D + R) at the five interfaces of the strip in one walk.  V^xi = b p^xi
     // - c p^lambda (Eq. canalie_V), times isc; an interface's upwind cell follows the last one's,
     // unless V^xi changes its sign between the two.
-    P dphi[TP];
+    P dphi[CPT];
     if (full) {
-      auto xi_load = [&](int cc) -> P { return p_mul(p_load(cell(k0, cc) + 2 * v), SC); };
+      auto xi_load = [&](int cc) -> P { return p_mul(p_load(cell(k0, c0 + cc) + 2 * v), SC); };
       auto xi_vel = [&](int c) -> real {
-        const P bc = p_load(c < TP ? &geo[c].bm : &geo[TP - 1].bp);
+        const P bc = p_load(c < CPT ? &geo[c].bm : &geo[CPT - 1].bp);
         return bc.x * pxI - bc.y * plI;
       };
       auto flux = [&](real V, P f) -> P { return p_mul(p_set(V), CLB ? p_add(f, R2) : f); };
@@ -714,13 +723,13 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
       real V = xi_vel(0);
       bool up = V >= real(0);
       sx.set(up);
-      const real* q = cell(k0, up ? -3 : -2) + 2 * v;
+      const real* q = cell(k0, c0 + (up ? -3 : -2)) + 2 * v;
       wx.start(p_mul(p_load(q), SC), p_mul(p_load(q + CS), SC), p_mul(p_load(q + 2 * CS), SC),
                p_mul(p_load(q + 3 * CS), SC), p_mul(p_load(q + 4 * CS), SC));
-      P phi[TP + 1];
+      P phi[CPT + 1];
       phi[0] = flux(V, wx.face(sx, range));
 #pragma unroll
-      for (int c = 1; c <= TP; ++c) {
+      for (int c = 1; c <= CPT; ++c) {
         V = xi_vel(c);
         if ((V >= real(0)) == up) {
           wx.push(p_mul(p_load(q + (4 + c) * CS), SC));
@@ -735,7 +744,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
       }
       if (__any_sync(0xffffffffu, !range.ok())) {  // some weights left their range
 #pragma unroll 1
-        for (int c = 0; c <= TP; ++c) {
+        for (int c = 0; c <= CPT; ++c) {
           V = xi_vel(c);
           up = V >= real(0);
           const int n = up ? c - 1 : c;
@@ -743,23 +752,23 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
           const P x = flux(V, wx.face_any(up));
           const int to = wx.in_range(up) ? -1 : c;
 #pragma unroll
-          for (int k = 0; k <= TP; ++k) phi[k] = p_sel(k == to, x, phi[k]);
+          for (int k = 0; k <= CPT; ++k) phi[k] = p_sel(k == to, x, phi[k]);
         }
       }
 #pragma unroll
-      for (int c = 0; c < TP; ++c) dphi[c] = p_mul(p_load(geo[c].idx), p_sub(phi[c + 1], phi[c]));
+      for (int c = 0; c < CPT; ++c) dphi[c] = p_mul(p_load(geo[c].idx), p_sub(phi[c + 1], phi[c]));
     }
 
     // ---- lambda interface s + 1/2 of every column
-    P fhi[TP];
+    P fhi[CPT];
     WenoRange<real> range;
     auto lam_up = [&](int c) -> bool {  // upwind side of interface s + 1/2, Cartesian split
       const ChanCell<real>& g = geo[c];
       return (full ? g.ap[0] * pl - g.glxx * px : -(g.nam[0] * pl + g.glxl * px)) >= real(0);
     };
 #pragma unroll
-    for (int c = 0; c < TP; ++c) {
-      const P fnew = p_mul(p_load(cell(k3, c) + 2 * v), SC);
+    for (int c = 0; c < CPT; ++c) {
+      const P fnew = p_mul(p_load(cell(k3, c0 + c) + 2 * v), SC);
       if constexpr (CLB) {
 #pragma unroll
         for (int q = 0; q < 5; ++q) raw[c][q] = raw[c][q + 1];
@@ -772,27 +781,27 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
     }
     if (__any_sync(0xffffffffu, !range.ok())) {
 #pragma unroll 1
-      for (int c = 0; c < TP; ++c) {
+      for (int c = 0; c < CPT; ++c) {
         // from memory: the windows' older terms are not kept
         const bool up = CLB ? lam_up(c) : lpos;
-        const int b = s + (up ? 0 : 1) - 2;
+        const int b = s + (up ? 0 : 1) - 2, cc = c0 + c;
         WenoWin<real, false> w;
-        w.start(p_mul(any_row(b, c), SC), p_mul(any_row(b + 1, c), SC), p_mul(any_row(b + 2, c), SC),
-                p_mul(any_row(b + 3, c), SC), p_mul(any_row(b + 4, c), SC));
+        w.start(p_mul(any_row(b, cc), SC), p_mul(any_row(b + 1, cc), SC), p_mul(any_row(b + 2, cc), SC),
+                p_mul(any_row(b + 3, cc), SC), p_mul(any_row(b + 4, cc), SC));
         const P x = w.face_any(up);
         const int to = w.in_range(up) ? -1 : c;
 #pragma unroll
-        for (int k = 0; k < TP; ++k) fhi[k] = p_sel(k == to, x, fhi[k]);
+        for (int k = 0; k < CPT; ++k) fhi[k] = p_sel(k == to, x, fhi[k]);
       }
     }
 
     // ---- the combine of row s
     if (full) {
-      const real* rec = eqr + (s & (L::NEQ - 1)) * TP * EQW;
-      const real* fb = lbl + (s & 1) * TP * CS + 2 * v;
-      const real* xb = lbx + ((s & 1) * TP * Q0 + i) * XS + 2 * j;
+      const real* rec = eqr + ((s & (L::NEQ - 1)) * TP + c0) * EQW;
+      const real* fb = lbl + ((s & 1) * TP + c0) * CS + 2 * v;
+      const real* xb = lbx + (((s & 1) * TP + c0) * Q0 + i) * XS + 2 * j;
 #pragma unroll
-      for (int c = 0; c < TP; ++c) {
+      for (int c = 0; c < CPT; ++c) {
         const ChanCell<real>& g = geo[c];
         P adv;
         if constexpr (CLB) {
@@ -807,7 +816,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
         // L = -advection + force - (F - f_eq) / tau
         const real* rc = rec + c * EQW;
         const P deq = p_fma(p_mul(p_load(rc + 2 * i), p_load(rc + 2 * (Q0 + j))), p_load(rc + 2 * (Q0 + Q1)), NR);
-        const P F = p_load(cell(k0, c) + 2 * v);
+        const P F = p_load(cell(k0, c0 + c) + 2 * v);
         P Lv = p_sub(p_mul(p_sub(F, deq), p_load(rc + 2 * (Q0 + Q1) + 2)), adv);
         if constexpr (!CLB) Lv = p_add(Lv, p_add(p_load(fb + c * CS), p_load(xb + c * Q0 * XS)));
         P o = p_fma(a.ccdt, Lv, F);
@@ -818,10 +827,10 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, XW>::NT, ChanSmem<real,
       Fo += rstep;
       if (need_fl && s + 1 < sB)
 #pragma unroll
-        for (int c = 0; c < TP; ++c) flr[c] = p_load(Fl + c * ROW);
+        for (int c = 0; c < CPT; ++c) flr[c] = p_load(Fl + c * ROW);
     }
 #pragma unroll
-    for (int c = 0; c < TP; ++c) flo[c] = fhi[c];
+    for (int c = 0; c < CPT; ++c) flo[c] = fhi[c];
     }
     }
     // ---- the rows ahead

@@ -87,7 +87,8 @@ struct vlb_ctx {
   ChanDesc cdesc{};
   ChanVariant cvariants[8];
   int n_cvariants = 0;
-  int chan_per_sm = 1;  // resident CTAs of the channel stage kernel per SM
+  ChanKernel chan_kernels[2][2];  // [Cartesian split][kernel]
+  int n_chan_kernels = 0;
   ChanCell<double>* d_cgeo = nullptr;
   ChanCell<float>* d_cgeof = nullptr;
   CellMap cmap;  // device cell order against the caller's (identity for Couette)

@@ -206,10 +206,10 @@ cudaError_t stage_config(StageVariant v, const ModelArgs& m, int Vp, int* nbuf, 
 }
 
 // ---------------------------------------------------------------- channel dispatch
-template <typename real, int Q0, int Q1, int XW, bool CLB, bool HX>
+template <typename real, int Q0, int Q1, int CG, int XW, bool CLB, bool HX>
 static cudaError_t go_channel(const ChanArgs<real>& a, const void* kpb, int grid, cudaStream_t s) {
-  using L = ChanSmem<real, Q0, Q1, XW>;
-  auto kern = channel_stage_kernel<real, Q0, Q1, XW, CLB, HX>;
+  using L = ChanSmem<real, Q0, Q1, CG, XW>;
+  auto kern = channel_stage_kernel<real, Q0, Q1, CG, XW, CLB, HX>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(L::bytes));
   if (e != cudaSuccess) return e;
   ChanKP<real, Q0, Q1> kp;
@@ -302,11 +302,38 @@ bool channel_force_pairs(int nq0, int nq1, const AxisTables* ax, std::vector<uns
   return false;
 }
 
+template <typename real, int Q0, int Q1, int CG, int XW>
+static cudaError_t channel_residency(int kind1, bool clb, int* per_sm) {
+  using L = ChanSmem<real, Q0, Q1, CG, XW>;
+  auto kern = clb ? channel_stage_kernel<real, Q0, Q1, CG, XW, true, false>
+                  : kind1 == 1 ? channel_stage_kernel<real, Q0, Q1, CG, XW, false, true>
+                               : channel_stage_kernel<real, Q0, Q1, CG, XW, false, false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(L::bytes));
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, L::NT, L::bytes);
+  return e;
+}
+
+// A march step of the one-warp kernel of the 8 x 4 set takes about 1.1 (single precision) and 1.8 (double)
+// times that of the kernel with a warp per column, with the CTAs that are resident on a busy SM; times of
+// an RK3 step, warp per column / one warp.  Single precision: 16 x 128 cells 39.8 / 52.7 us, 64 x 64 44.7 /
+// 52.9, 16 x 604 55.1 / 57.3, 30 x 200 51.7 / 47.5, 16 x 612 71 / 58, 64 x 512 162 / 119.  Double precision:
+// 16 x 128 268 / 633, 64 x 64 462 / 652, 30 x 200 559 / 545, 16 x 604 848 / 699, 64 x 512 3171 / 2467.
 template <typename real>
-size_t channel_smem_bytes(ChanVariant, int nq0, int nq1, int* per_sm) {
-  if (nq0 == 16 && nq1 == 12) return *per_sm = ChanSmem<real, 16, 12, 0>::min_ctas, ChanSmem<real, 16, 12, 0>::bytes;
-  if (nq0 == 8 && nq1 == 4) return *per_sm = ChanSmem<real, 8, 4, 0>::min_ctas, ChanSmem<real, 8, 4, 0>::bytes;
-  return 0;
+cudaError_t channel_kernels(int nq0, int nq1, int kind1, bool clb, ChanKernel* out, int* n) {
+  cudaError_t e = cudaSuccess;
+  *n = 0;
+  if (nq0 == 16 && nq1 == 12) {
+    *n = 1;
+    out[0].step = 10;
+    e = channel_residency<real, 16, 12, 1, 0>(kind1, clb, &out[0].per_sm);
+  } else if (nq0 == 8 && nq1 == 4) {
+    *n = 2;
+    out[0].step = sizeof(real) == 8 ? 18 : 11;
+    out[1].step = 10;
+    e = channel_residency<real, 8, 4, 1, 0>(kind1, clb, &out[0].per_sm);
+    if (e == cudaSuccess) e = channel_residency<real, 8, 4, 4, 3>(kind1, clb, &out[1].per_sm);
+  }
+  return e;
 }
 
 // Axis moment vector of the truncated equilibrium at rest (u = 0), in double.
@@ -378,18 +405,16 @@ bool channel_tables(int nq0, int nq1, const ModelArgs& m, double T0, std::vector
 }
 
 template <typename real>
-cudaError_t launch_channel(const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int kind1, int grid,
+cudaError_t launch_channel(const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int kind1, int kernel, int grid,
                            cudaStream_t s, bool clb) {
-#define VLB_CH(q0, q1, xw)                                                                  \
-  return clb ? go_channel<real, q0, q1, xw, true, false>(a, kp, grid, s)                    \
-             : kind1 == 1 ? go_channel<real, q0, q1, xw, false, true>(a, kp, grid, s)       \
-                          : go_channel<real, q0, q1, xw, false, false>(a, kp, grid, s);
-  if (nq0 == 16 && nq1 == 12) VLB_CH(16, 12, 0)
-  // one-warp velocity set: extra warps while every CTA with them is resident at once (16 x 128
-  // cells, 12 steps: 812 us against 929 with one warp); beyond that more CTAs of one warp fill the SMs
+#define VLB_CH(q0, q1, cg, xw)                                                                  \
+  return clb ? go_channel<real, q0, q1, cg, xw, true, false>(a, kp, grid, s)                    \
+             : kind1 == 1 ? go_channel<real, q0, q1, cg, xw, false, true>(a, kp, grid, s)       \
+                          : go_channel<real, q0, q1, cg, xw, false, false>(a, kp, grid, s);
+  if (nq0 == 16 && nq1 == 12) VLB_CH(16, 12, 1, 0)
   if (nq0 == 8 && nq1 == 4) {
-    if (grid <= 152 * ChanSmem<real, 8, 4, 3>::min_ctas) VLB_CH(8, 4, 3)
-    VLB_CH(8, 4, 0)
+    if (kernel == 1) VLB_CH(8, 4, 4, 3)
+    VLB_CH(8, 4, 1, 0)
   }
 #undef VLB_CH
   return cudaErrorInvalidValue;
@@ -1068,8 +1093,8 @@ template cudaError_t launch_stage<VLB_REAL>(StageVariant, const StageArgs<VLB_RE
                                             const KArgs<VLB_REAL>&, int, cudaStream_t, bool);
 template cudaError_t launch_init_equilibrium<VLB_REAL>(VLB_REAL*, long long, int, const ModelArgs&, double, double,
                                                        double, double, cudaStream_t);
-template size_t channel_smem_bytes<VLB_REAL>(ChanVariant, int, int, int*);
-template cudaError_t launch_channel<VLB_REAL>(const ChanArgs<VLB_REAL>&, const void*, int, int, int, int,
+template cudaError_t channel_kernels<VLB_REAL>(int, int, int, bool, ChanKernel*, int*);
+template cudaError_t launch_channel<VLB_REAL>(const ChanArgs<VLB_REAL>&, const void*, int, int, int, int, int,
                                               cudaStream_t, bool);
 template bool channel_force_pairs<VLB_REAL>(int, int, const AxisTables*, std::vector<unsigned char>*);
 template bool channel_tables<VLB_REAL>(int, int, const ModelArgs&, double, std::vector<unsigned char>*);

@@ -74,9 +74,14 @@ struct ChanArgs;
 
 // Channel launch shapes for a model shape (at most 8); 0 if the shape has no channel kernel.
 int channel_variants(int nq0, int nq1, ChanVariant* out);
-// Shared memory of a CTA and (per_sm) the CTAs a SM holds; 0 if the shape has no channel kernel.
+// The kernels of a model shape (n of them, at most 2, 0 if it has none; kind1, clb as for launch_channel):
+// the CTAs of each that a SM of the current device holds, and the time of a step of its march against
+// that of the others.
+struct ChanKernel {
+  int per_sm, step;
+};
 template <typename real>
-size_t channel_smem_bytes(ChanVariant v, int nq0, int nq1, int* per_sm);
+cudaError_t channel_kernels(int nq0, int nq1, int kind1, bool clb, ChanKernel* out, int* n);
 // The ChanTables block of a model shape (bytes, copied by every CTA) for the model arguments
 // and the reservoir / wall temperature T0; false if the shape has no channel kernel.
 template <typename real>
@@ -85,10 +90,11 @@ bool channel_tables(int nq0, int nq1, const ModelArgs& m, double T0, std::vector
 // the shape has no channel kernel or a matrix lacks the structure the block relies on.
 template <typename real>
 bool channel_force_pairs(int nq0, int nq1, const AxisTables* ax, std::vector<unsigned char>* out);
-// One channel stage on `grid` CTAs (a.nx / tp strips x a.nseg segments); kind1: axis 1 is half range (1).
+// One channel stage on `grid` CTAs (a.nx / tp strips x a.nseg segments) of the shape's kernel of that number;
+// kind1: axis 1 is half range (1).
 // clb: the Cartesian-split formulation on the same march (a.geo then holds its geometry records)
 template <typename real>
-cudaError_t launch_channel(const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int kind1, int grid,
+cudaError_t launch_channel(const ChanArgs<real>& a, const void* kp, int nq0, int nq1, int kind1, int kernel, int grid,
                            cudaStream_t s, bool clb = false);
 
 // Order of a context's cells in device buffers against the caller's order.
