@@ -84,9 +84,12 @@ struct StageSmem {
 // allow them but the compiler, left alone, takes too many registers a thread.  A
 // single-precision CTA of 256 to 384 threads needs at most about 64 KB of shared
 // memory for tiles up to 8 cells (three fit on an SM) and about 100 KB for 16
-// (two fit) with the model shapes that have fixed node counts.
+// (two fit) with the model shapes that have fixed node counts.  In double precision the sets of
+// up to 64 velocities run on CTAs of 64 threads, whose latency only other CTAs hide: left alone the
+// compiler takes 172 to 184 registers, four CTAs a SM where shared memory holds five to seven
+// (64 instances of 80 cells, 8 x 8 velocities, a step: 904 us, and 836 with five).
 constexpr int stage_min_ctas(int real_bytes, int tc, int nt) {
-  return (real_bytes == 4 && nt >= 256 && nt <= 384) ? (tc <= 8 ? 3 : 2) : 1;
+  return real_bytes == 8 ? (nt == 64 ? 6 : 1) : nt >= 256 && nt <= 384 ? (tc <= 8 ? 3 : 2) : 1;
 }
 
 // FT: the f~ formulation (Sec. VI.B, Eqs. boltz_couette_cons / boltz_couette_str_cons).  The

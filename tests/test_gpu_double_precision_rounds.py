@@ -1,0 +1,42 @@
+"""Double-precision Couette contexts of up to 64 velocities (CTAs of 64 threads): five CTAs stay resident on a
+SM, so that a context whose tiles come to between four and five a SM runs in one round."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+from paper_1708_05944_gb300 import vlb  # noqa: E402
+
+
+def step_ms(spec, n_inst, cells, collision=None, steps=10):
+    s = torch.cuda.Stream()
+    c = vlb.Couette(spec, vlb.VLB_FP64, [dict(n_cells=cells, r_in=1.0, r_out=2.0)] * n_inst, [(0.1, 1.0)] * n_inst,
+                    [(0.0, 1.0)] * n_inst, [0.1] * n_inst, [1] * n_inst, stream=s.cuda_stream)
+    if collision is not None:
+        c.set_collision(*collision)
+    c.set_dt([1e-5] * n_inst)
+    c.init_equilibrium(1.0, 0.0, 0.01, 1.1)
+    c.step(1e-5, 5)
+    best = np.inf
+    for _ in range(3):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record(s)
+        c.step(1e-5, steps)
+        b.record(s)
+        s.synchronize()
+        best = min(best, a.elapsed_time(b) / steps)
+    c.close()
+    return best
+
+
+# ten tiles of eight cells an instance: just under four tiles a SM, and four and a fifth.  In two rounds the
+# second costs 1.9 times the first; in one the SMs that take a fifth tile cost a little
+@pytest.mark.parametrize("spec", ["HH(3;4)xHH(3;4)", "H(4;6)xHH(3;5)"])
+def test_five_tiles_a_sm_are_one_round(spec):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 4 * sms // 10
+    assert step_ms(spec, n + sms // 50, 80) < 1.3 * step_ms(spec, n - 1, 80)
