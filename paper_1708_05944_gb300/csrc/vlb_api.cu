@@ -471,10 +471,10 @@ vlb_status run_stage(vlb_ctx* c, int k) {
         c->prec == VLB_FP64
             ? launch_shakhov<double>(static_cast<double*>(c->F[out]), static_cast<const double*>(c->F[prev]),
                                      c->total_cells, c->Vp, c->margs, c->d_inst, c->n_inst, ccw[k - 1],
-                                     1.0 - c->prandtl, knf, c->stream)
+                                     1.0 - c->prandtl, knf, c->sms, c->stream)
             : launch_shakhov<float>(static_cast<float*>(c->F[out]), static_cast<const float*>(c->F[prev]),
                                     c->total_cells, c->Vp, c->margs, c->d_inst, c->n_inst, ccw[k - 1],
-                                    1.0 - c->prandtl, knf, c->stream);
+                                    1.0 - c->prandtl, knf, c->sms, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "Shakhov correction launch");
     c->launches += 1;
   }

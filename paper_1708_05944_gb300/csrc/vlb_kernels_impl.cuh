@@ -667,12 +667,12 @@ __device__ inline void power_tables(const ModelArgs& m, const ModelSmem<R>& ms, 
 template <typename real>
 __global__ void __launch_bounds__(128) shakhov_kernel(real* Fout, const real* Fprev, long long cells, int Vp,
                                                       const __grid_constant__ ModelArgs m, const InstDesc* inst,
-                                                      int n_inst, double cc, double omp, double kn_fixed) {
+                                                      int n_inst, double cc, double omp, double kn_fixed, bool early) {
   __shared__ real A[4][4][MAXQ], B[4][4][MAXQ], M[4][4][MAXN + 3], OV[4][16][MAXN];  // per warp
   __shared__ ModelSmem<real> ms;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int V = m.nq0 * m.nq1;
-  grid_launch_dependents();
+  if (early) grid_launch_dependents();  // (see launch_shakhov)
   stage_model<real>(m, ms);
   grid_dependency_wait();
   auto wsum = [&](real x) {
@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(128) shakhov_kernel(real* Fout, const real* Fp
 template <typename real, int Q0, int Q1>
 __global__ void __launch_bounds__(128) shakhov_fixed_kernel(real* Fout, const real* Fprev, long long cells,
                                                             const __grid_constant__ ModelArgs m, const InstDesc* inst,
-                                                            int n_inst, double cc, double omp, double kn_fixed) {
+                                                            int n_inst, double cc, double omp, double kn_fixed, bool early) {
   using P = pair_t<real>;
   constexpr int V = Q0 * Q1, R = V / 32, NQ = Q0 + Q1;
   static_assert(V % 32 == 0, "whole warps of velocities");
@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(128) shakhov_fixed_kernel(real* Fout, const re
   __shared__ alignas(16) real PA[4][Q0][4], PB[4][Q1][4];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   constexpr bool F32 = sizeof(real) == 4;
-  grid_launch_dependents();
+  if (early) grid_launch_dependents();  // (see launch_shakhov)
   const int nmax = m.N0 > m.N1 ? m.N0 : m.N1;
   for (int x = threadIdx.x; x < MAXN * NQ; x += 128) {
     const int s = x / NQ, q = x - s * NQ, ax = q >= Q0, k = ax ? q - Q0 : q;
@@ -867,21 +867,28 @@ __global__ void __launch_bounds__(128) shakhov_fixed_kernel(real* Fout, const re
   }
 }
 
+// Launched as dependent on the stage, as the next stage is on it.  In double precision only where its CTAs
+// come to an eighth of the SMs at most: the device places a dependent grid's CTAs while the other's still
+// hold some SMs, and those that are free take more than their share, which a kernel of 1/64-rate
+// operations does not make up for (a step replayed from a graph, 8 x 8 velocities: 1600 cells 718 us
+// dependent, 471 not; 8 x 8, 2560 cells 784 and 603; 16 x 20, 608 cells 436 and 342; 8 x 4, 8 cells 98 and
+// 104).  From six CTAs a SM it evens out, and the correction is dependent again.
 template <typename real>
 cudaError_t launch_shakhov(real* Fout, const real* Fprev, long long cells, int Vp, const ModelArgs& m,
-                           const InstDesc* inst, int n_inst, double cc, double one_minus_pr, double kn_fixed,
+                           const InstDesc* inst, int n_inst, double cc, double one_minus_pr, double kn_fixed, int sms,
                            cudaStream_t s) {
   long long blocks = (cells + 3) / 4;
   if (blocks > 152 * 16) blocks = 152 * 16;
+  const bool early = sizeof(real) == 4 || blocks <= sms / 8, dependent = early || blocks > 6ll * sms;
   const dim3 g(static_cast<unsigned>(blocks > 0 ? blocks : 1));
 #define VLB_SHAKHOV(q0, q1)                                                                                          \
   if (m.nq0 == q0 && m.nq1 == q1)                                                                                    \
-    return launch_dependent(shakhov_fixed_kernel<real, q0, q1>, g, 128, 0, s, Fout, Fprev, cells, m, inst, n_inst, cc, \
-                            one_minus_pr, kn_fixed);
+    return launch_ordered(dependent, shakhov_fixed_kernel<real, q0, q1>, g, 128, 0, s, Fout, Fprev, cells, m, inst, \
+                          n_inst, cc, one_minus_pr, kn_fixed, early);
   VLB_SHAKHOV(16, 20) VLB_SHAKHOV(16, 12) VLB_SHAKHOV(8, 4)
 #undef VLB_SHAKHOV
-  return launch_dependent(shakhov_kernel<real>, g, 128, 0, s, Fout, Fprev, cells, Vp,
-                          m, inst, n_inst, cc, one_minus_pr, kn_fixed);
+  return launch_ordered(dependent, shakhov_kernel<real>, g, 128, 0, s, Fout, Fprev, cells, Vp, m, inst, n_inst, cc,
+                        one_minus_pr, kn_fixed, early);
 }
 
 // ---------------------------------------------------------------- caller layout <-> device layout
@@ -1107,6 +1114,6 @@ template cudaError_t launch_deviation<VLB_REAL>(const VLB_REAL*, VLB_REAL*, long
 template cudaError_t launch_moments<VLB_REAL>(const VLB_REAL*, long long, int, const ModelArgs&, double*,
                                               cudaStream_t, CellMap);
 template cudaError_t launch_shakhov<VLB_REAL>(VLB_REAL*, const VLB_REAL*, long long, int, const ModelArgs&,
-                                              const InstDesc*, int, double, double, double, cudaStream_t);
+                                              const InstDesc*, int, double, double, double, int, cudaStream_t);
 
 }  // namespace vlb

@@ -16,15 +16,20 @@ namespace vlb {
 // kernel's own start-up, about 2 us of a 12 us stage).  After a copy or another kernel it waits for
 // those as a plain launch does, and captures into a graph as such.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t s,
-                                    Args&&... args) {
+inline cudaError_t launch_ordered(bool dependent, void (*kern)(Params...), dim3 grid, int threads, size_t smem,
+                                  cudaStream_t s, Args&&... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid, cfg.blockDim = dim3(unsigned(threads)), cfg.dynamicSmemBytes = smem, cfg.stream = s;
-  cfg.attrs = &at, cfg.numAttrs = 1;
+  cfg.attrs = &at, cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <typename... Params, typename... Args>
+inline cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                                    Args&&... args) {
+  return launch_ordered(true, kern, grid, threads, smem, s, std::forward<Args>(args)...);
 }
 
 template <typename real>
@@ -138,10 +143,10 @@ cudaError_t launch_deviation(const real* src, real* dst, long long cells, int Vp
 // Shakhov correction of a stage (see shakhov_kernel): F_out += cc dt (1 - Pr) G[F_prev] / tau per
 // cell, the moments taken from F_prev by the same kernel (device cell order); kn_fixed > 0:
 // tau = kn_fixed / (n T) for every cell, else each cell's instance (Kn, tau convention); dt from
-// the instance.
+// the instance; sms: of the device.
 template <typename real>
 cudaError_t launch_shakhov(real* Fout, const real* Fprev, long long cells, int Vp, const ModelArgs& m,
-                           const InstDesc* inst, int n_inst, double cc, double one_minus_pr, double kn_fixed,
+                           const InstDesc* inst, int n_inst, double cc, double one_minus_pr, double kn_fixed, int sms,
                            cudaStream_t s);
 
 // Model tables of a Couette context beyond the fused kernels' 32 nodes per axis (device

@@ -1,5 +1,6 @@
-"""Double-precision Couette contexts of up to 64 velocities (CTAs of 64 threads): five CTAs stay resident on a
-SM, so that a context whose tiles come to between four and five a SM runs in one round."""
+"""How double-precision Couette contexts fill the device.  Sets of up to 64 velocities (CTAs of 64 threads):
+five CTAs stay resident on a SM, so that a context whose tiles come to between four and five a SM runs
+in one round.  The Shakhov correction: its CTAs are spread evenly, also when replayed from a graph."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,7 @@ if not torch.cuda.is_available():
 from paper_1708_05944_gb300 import vlb  # noqa: E402
 
 
-def step_ms(spec, n_inst, cells, collision=None, steps=10):
+def step_ms(spec, n_inst, cells, collision=None, graph=False, steps=12):
     s = torch.cuda.Stream()
     c = vlb.Couette(spec, vlb.VLB_FP64, [dict(n_cells=cells, r_in=1.0, r_out=2.0)] * n_inst, [(0.1, 1.0)] * n_inst,
                     [(0.0, 1.0)] * n_inst, [0.1] * n_inst, [1] * n_inst, stream=s.cuda_stream)
@@ -20,12 +21,13 @@ def step_ms(spec, n_inst, cells, collision=None, steps=10):
         c.set_collision(*collision)
     c.set_dt([1e-5] * n_inst)
     c.init_equilibrium(1.0, 0.0, 0.01, 1.1)
-    c.step(1e-5, 5)
+    step = c.step_graph if graph else c.step
+    step(1e-5, 6)
     best = np.inf
     for _ in range(3):
         a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
         a.record(s)
-        c.step(1e-5, steps)
+        step(1e-5, steps)
         b.record(s)
         s.synchronize()
         best = min(best, a.elapsed_time(b) / steps)
@@ -40,3 +42,10 @@ def test_five_tiles_a_sm_are_one_round(spec):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     n = 4 * sms // 10
     assert step_ms(spec, n + sms // 50, 80) < 1.3 * step_ms(spec, n - 1, 80)
+
+
+# 1600 cells are 400 CTAs of the correction.  Placed while the stage still held most SMs they doubled a step
+@pytest.mark.parametrize("spec", ["HH(3;4)xHH(3;4)", "H(4;6)xHH(3;5)"])
+def test_shakhov_correction_is_spread_evenly(spec):
+    bgk = step_ms(spec, 16, 100, graph=True)
+    assert step_ms(spec, 16, 100, (vlb.VLB_SHAKHOV, 2.0 / 3.0), graph=True) < 1.6 * bgk
