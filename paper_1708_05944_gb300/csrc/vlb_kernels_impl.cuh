@@ -900,50 +900,79 @@ cudaError_t launch_shakhov(real* Fout, const real* Fprev, long long cells, int V
 // velocities stays in registers over all rows of the warp.  A row is read whole before any of
 // it is written, so src and dst may be the same buffer when V == Vp and the map is the identity.
 //
-// F -/+ R in single precision takes R as a float pair (hi, lo) and TwoSum: the sum is exact to
-// about 2^-48 before its one rounding, where the earlier sum in double cost three operations
-// of the 1/64-rate FP64 pipe per value.  2048 x 512 x 192 channel (1.6 GB), both directions
-// together: 5.5 ms before, 1.27 ms now (6.4 GB moved: 0.75 of the measured copy bandwidth).
+// F -/+ R is rounded once.  In single precision R (53 bits) is a sum of three floats, and the sum with F
+// stays on the FP32 pipe, where one in double cost three operations of the 1/64-rate FP64 pipe per
+// value: its bounds from directed sums of the low parts round to the same value nearly always, and the
+// others (near rest, where F and R nearly cancel, or next to a tie) are gathered exactly.  (A pair of
+// floats alone would lose the last five bits of R, near rest a quarter of a unit in the deviation's last
+// place.)  In double precision R = w_i w_j is not rounded before the sum.  2048 x 512 x 192 channel
+// (1.6 GB), both directions together: 5.5 ms with the sum in double, 1.15 ms so (6.4 GB moved: 0.82 of
+// the measured copy bandwidth; 1.28 ms at rest).
 template <typename real>
-struct RestValue {  // R of one velocity
-  real hi, lo;
+struct RestValue;  // of one velocity, with the sign of the sum
+template <>
+struct RestValue<float> {
+  float hi, mid, lo;
+  __device__ __forceinline__ void set(double w0, double w1) {
+    const double R = w0 * w1;
+    hi = float(R);
+    mid = float(R - double(hi));
+    lo = float(R - double(hi) - double(mid));
+  }
 };
-template <typename real>
-__device__ __forceinline__ RestValue<real> rest_value(double R) {
-  RestValue<real> r;
-  r.hi = real(R);
-  r.lo = real(R - double(r.hi));
-  return r;
-}
-// x + sgn R, rounded once
-__device__ __forceinline__ float add_rest(float x, RestValue<float> r, float sgn) {
+template <>
+struct RestValue<double> {
+  double w0, w1;
+  __device__ __forceinline__ void set(double a, double b) { w0 = a, w1 = b; }
+};
+// x + R where both bounds round to the same value; else out is set
+__device__ __forceinline__ float add_rest(float x, RestValue<float> r, bool& out) {
   float s, e;
-  two_sum(x, sgn * r.hi, s, e);
-  const float t = __fadd_rn(s, __fadd_rn(e, sgn * r.lo));
-  return fabsf(s) <= 3.402823466e38f ? t : s;  // Inf and NaN stay what the plain sum gives
+  two_sum(x, r.hi, s, e);
+  const float d = __fadd_rn(s, __fadd_rd(__fadd_rd(e, r.mid), r.lo));
+  const float u = __fadd_rn(s, __fadd_ru(__fadd_ru(e, r.mid), r.lo));
+  out = out || !(d == u);
+  return d;
 }
-__device__ __forceinline__ double add_rest(double x, RestValue<double> r, double sgn) { return x + sgn * r.hi; }
+__device__ __forceinline__ double add_rest(double x, RestValue<double> r, bool&) { return fma(r.w0, r.w1, x); }
+// a + b rounded to odd: of the two neighbours of an inexact sum the one with the last bit set, so that a
+// further rounding to fewer bits sees which side of a tie the sum lies on
+__device__ __forceinline__ float add_odd(float a, float b) {
+  const float d = __fadd_rd(a, b), u = __fadd_ru(a, b);
+  return __float_as_uint(d) & 1u ? d : u;
+}
+__device__ __forceinline__ float add_rest_exact(float x, RestValue<float> r) {
+  float s, e, v, f, t, q;
+  two_sum(x, r.hi, s, e);
+  two_sum(e, r.mid, v, f);
+  two_sum(s, v, t, q);
+  const float z = __fadd_rn(t, add_odd(q, add_odd(f, r.lo)));
+  return fabsf(s) <= 3.402823466e38f ? z : s;  // Inf and NaN stay what the plain sum gives
+}
+__device__ __forceinline__ double add_rest_exact(double x, RestValue<double> r) { return fma(r.w0, r.w1, x); }
 
 template <typename real, int NV, int CH>
 __global__ void __launch_bounds__(256) deviation_kernel(const real* src, real* dst, long long cells, int Vp,
                                                         const __grid_constant__ ModelArgs m, int to_dev, CellMap map) {
   using P = pair_t<real>;
-  // (the weights by way of shared memory: an index per lane into the parameters is serialised)
+  // (the weights by way of shared memory: an index per lane into the parameters is serialised; then R,
+  // whose parts take FP64-pipe operations, once per CTA)
   __shared__ double sw[2][MAXQ];
+  __shared__ RestValue<real> sr[32 * CH * NV];
   if (threadIdx.x < 2 * MAXQ) sw[threadIdx.x / MAXQ][threadIdx.x % MAXQ] = (threadIdx.x < MAXQ ? m.w0 : m.w1)[threadIdx.x % MAXQ];
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int V = m.nq0 * m.nq1;
+  for (int v = threadIdx.x; v < 32 * CH * NV; v += blockDim.x) {
+    const int i = v < V ? v / m.nq1 : 0, j = v < V ? v - i * m.nq1 : 0;
+    sr[v].set(to_dev ? -sw[0][i] : sw[0][i], sw[1][j]);
+  }
+  __syncthreads();
   RestValue<real> R[CH][NV];
 #pragma unroll
   for (int k = 0; k < CH; ++k)
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      const int v = (32 * k + lane) * NV + q;
-      const int i = v < V ? v / m.nq1 : 0, j = v < V ? v - i * m.nq1 : 0;
-      R[k][q] = rest_value<real>(sw[0][i] * sw[1][j]);
-    }
-  const real sgn = to_dev ? real(-1) : real(1);
+    for (int q = 0; q < NV; ++q) R[k][q] = sr[(32 * k + lane) * NV + q];
   const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long c = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < cells; c += nw) {
     const long long cc = caller_cell(map, c);  // device cell c is the caller's cell cc
@@ -971,10 +1000,24 @@ __global__ void __launch_bounds__(256) deviation_kernel(const real* src, real* d
             x[k][0] = p_load(a + 2 * v);
           }
         }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < CH; ++k) {
+      if (32 * k * NV >= V) break;
+      P y[NV];
+      bool out = false;
+#pragma unroll
+      for (int q = 0; q < NV; ++q)
+        y[q] = p_make(add_rest(x[k][q].x, R[k][q], out), add_rest(x[k][q].y, R[k][q], out));
+      if (__any_sync(0xffffffffu, out)) {
 #pragma unroll
         for (int q = 0; q < NV; ++q)
-          x[k][q] = p_make(add_rest(x[k][q].x, R[k][q], sgn), add_rest(x[k][q].y, R[k][q], sgn));
+          y[q] = p_make(add_rest_exact(x[k][q].x, R[k][q]), add_rest_exact(x[k][q].y, R[k][q]));
       }
+#pragma unroll
+      for (int q = 0; q < NV; ++q)
+        if ((32 * k + lane) * NV < V) x[k][q] = y[q];  // (the padding velocities stay zero)
     }
     __syncwarp();
 #pragma unroll

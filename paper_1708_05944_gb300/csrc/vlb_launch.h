@@ -133,8 +133,7 @@ cudaError_t launch_seed(real* F, long long cells, int Vp, const ModelArgs& m, co
 // Caller layout F (per cell: f' then f'', V values each) to and from the device
 // layout (per cell: Vp interleaved (f', f'') pairs of the deviation D = F - R;
 // padding zero).  to_deviation = 1: caller -> device, 0: device -> caller; each
-// element is summed with R to twice its own precision and rounded once (single precision; in
-// double precision a plain sum).  src and dst may be the same buffer when V == Vp and
+// sum is rounded once.  src and dst may be the same buffer when V == Vp and
 // the cell map is the identity.
 template <typename real>
 cudaError_t launch_deviation(const real* src, real* dst, long long cells, int Vp, const ModelArgs& m,
