@@ -385,8 +385,10 @@ vlb_status vlb_autotune(vlb_ctx* ctx, double dt, int reps, int* chosen, double* 
  * loads the library holds it until the process exits), so
  * 2 x total_cells x 2 x nvel x sizeof(real) must not exceed 64 MiB, else
  * VLB_ERR_UNSUPPORTED; nvel must be a multiple of 4, else VLB_ERR_UNSUPPORTED;
- * a channel context gets VLB_ERR_UNSUPPORTED and nothing is launched.  The
- * context's device must be the current device (else VLB_ERR_INVALID).  The
+ * a channel context gets VLB_ERR_UNSUPPORTED and nothing is launched.  f_out
+ * must start on a 16-byte boundary (its rows are bulk-copied) and f_in on one
+ * of its type; the context's device must be the current device (else
+ * VLB_ERR_INVALID).  The
  * first call on a device looks up the array's device address
  * (cudaGetSymbolAddress), and a call whose dt differs from the context's
  * current time step copies the instance descriptors and synchronises the

@@ -8,6 +8,8 @@
 // call this entry point, which uses g_step_scratch below for F^(1) and F^(2).
 #include <cuda_runtime.h>
 
+#include <stdint.h>
+
 #include <atomic>
 #include <cmath>
 #include <string>
@@ -76,6 +78,9 @@ extern "C" vlb_status vlb_step_static_scratch(vlb_ctx* c, const void* f_in, void
   if (c->large || c->ftilde)
     return static_fail(c, VLB_ERR_UNSUPPORTED, "static-scratch stepping covers the chi formulation up to 32 nodes per axis");
   if (!f_in || !f_out || f_in == f_out) return static_fail(c, VLB_ERR_INVALID, "need distinct input and output buffers");
+  // f_out holds stage data: its rows are bulk copies, which start on 16-byte boundaries
+  if (reinterpret_cast<uintptr_t>(f_out) % 16 != 0 || reinterpret_cast<uintptr_t>(f_in) % c->esize != 0)
+    return static_fail(c, VLB_ERR_INVALID, "the output buffer has to start on a 16-byte boundary");
   if (nsteps < 1 || !(dt > 0.0) || !std::isfinite(dt))
     return static_fail(c, VLB_ERR_INVALID, "need a finite dt > 0 and nsteps >= 1");
   if (c->Vp != c->V)
