@@ -241,13 +241,13 @@ vlb_status do_stage(vlb_ctx* c, int k, int prev, int out) {
   a.Fl = static_cast<const real*>(c->F[c->cur]);
   a.Fout = static_cast<real*>(c->F[out]);
   if (k == 1) {
-    a.ca = 0.0, a.cb = 1.0, a.cc = 1.0;
+    a.ca = 0.0, a.cc = 1.0;
   } else if (k == 2) {
-    a.ca = 0.75, a.cb = 0.25, a.cc = 0.25;
+    a.ca = 0.75, a.cc = 0.25;
   } else {
-    a.ca = 1.0 / 3.0, a.cb = 2.0 / 3.0, a.cc = 2.0 / 3.0;
+    a.ca = 1.0 / 3.0, a.cc = 2.0 / 3.0;
   }
-  a.caf = float(a.ca), a.cbf = float(a.cb), a.ccf = float(a.cc);
+  a.caf = float(a.ca), a.ccf = float(a.cc);
   a.geof = c->d_geof;
   a.inst = c->d_inst;
   a.tiles = c->d_tiles;
@@ -797,7 +797,7 @@ vlb_status vlb_create_couette(const vlb_model* model, vlb_precision prec, int n_
   c->esize = prec == VLB_FP64 ? 8 : 4;
   c->large = large;
   if (large) {
-    c->variants[0] = StageVariant{1, 256, 0};  // one launch shape: the four kernels of vlb_large.cu
+    c->variants[0] = StageVariant{1, 256, 0};  // one launch shape: the three kernels of vlb_large.cu
     c->n_variants = 1;
     vlb_status ls = setup_large(c.get());
     if (ls != VLB_OK) return ls;

@@ -179,8 +179,6 @@ __device__ __forceinline__ float2 k_mul(float2 k, float2 x) { return p_mul(k, x)
 __device__ __forceinline__ float2 k_fma(float2 k, float2 x, float2 a) { return p_fma(k, x, a); }
 __device__ __forceinline__ double2 k_mul(double k, double2 x) { return p_mul(p_set(k), x); }
 __device__ __forceinline__ double2 k_fma(double k, double2 x, double2 a) { return p_fma(p_set(k), x, a); }
-__device__ __forceinline__ float2 k_pair(float2 k) { return k; }
-__device__ __forceinline__ double2 k_pair(double k) { return p_set(k); }
 
 // Force matrices of the channel.  On each axis K = d/dp and Kt = d/dp (p .) of the projected
 // expansions satisfy
@@ -742,7 +740,7 @@ __global__ void __launch_bounds__(ChanSmem<real, Q0, Q1, CG, XW>::NT, ChanSmem<r
         }
         phi[c] = flux(V, wx.face(sx, range));
       }
-      if (__any_sync(0xffffffffu, !range.ok())) {  // some weights left their range
+      if (__any_sync(0xffffffffu, !range.ok())) {  // a face does not hold (see weno_holds)
 #pragma unroll 1
         for (int c = 0; c <= CPT; ++c) {
           V = xi_vel(c);

@@ -372,8 +372,8 @@ __device__ __forceinline__ float2 p_rcp(float2 x) {  // 1 / x of normal numbers,
   return r;
 }
 // One reciprocal for both, x.x x.y a normal number: the hardware's approximation (20 bits) and two
-// steps of Newton's iteration, r <- r + r (1 - x r), to about 1 ulp.  Seven operations of the FP64
-// pipe in place of two divisions.
+// steps of Newton's iteration, r <- r + r (1 - x r).  The product, the last step and the last multiply
+// round once each: about 2 ulp.  Seven operations of the FP64 pipe in place of two divisions.
 __device__ __forceinline__ double2 p_rcp(double2 x) {
   const double y = __dmul_rn(x.x, x.y);
   double r;
@@ -592,22 +592,7 @@ __device__ __forceinline__ void eq_moments_fast(int kind, int nmax, R u, R T, R*
   }
 }
 
-// Rescale the axis-0 equilibrium factor (which carries n) so that the stored
-// factors reproduce the cell density exactly: sum_i gn_i sum_j g1_j = n.  In
-// exact arithmetic the truncated equilibrium already has this sum (Sec. IV.D);
-// in single precision the table contraction misses it by some 1e-7, and the
-// BGK term would turn that into a mass source of (dt / tau) 1e-7 n every step.
-// The sums are taken in double.
-template <typename R>
-__device__ __forceinline__ void normalise_equilibrium(R* gn, const R* g1, int nq0, int nq1, double n) {
-  double s0 = 0.0, s1 = 0.0;
-  for (int k = 0; k < nq0; ++k) s0 += double(gn[k]);
-  for (int k = 0; k < nq1; ++k) s1 += double(g1[k]);
-  const R sc = R(n / (s0 * s1));
-  for (int k = 0; k < nq0; ++k) gn[k] *= sc;
-}
-
-// 1 / tau of the same conventions, ikn = 1 / Kn
+// 1 / tau of the conventions of relaxation_time, ikn = 1 / Kn
 template <typename R>
 __device__ __forceinline__ R relaxation_rate(int mode, R ikn, R n, R T) {
   const R r = n * ikn;

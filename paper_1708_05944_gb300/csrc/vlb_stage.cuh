@@ -31,12 +31,12 @@ struct StageArgs {
   const real* Fprev;  // distribution L acts on
   const real* Fl;     // F_l of the step (read when ca != 0)
   real* Fout;
-  // Fout = ca F_l + cb F_prev + cc dt L[F_prev] with cb = 1 - ca, evaluated as
+  // Fout = ca F_l + (1 - ca) F_prev + cc dt L[F_prev], evaluated as
   // F_prev + ca (F_l - F_prev) + cc dt L so that the weights on F sum to exactly
   // one in any precision (float(1/3) + float(2/3) = 1 + 3e-8 would add that much
   // mass every step).
-  double ca, cb, cc;
-  float caf, cbf, ccf;  // single-precision copies
+  double ca, cc;
+  float caf, ccf;  // single-precision copies
   const InstDesc* inst;
   const TileDesc* tiles;
   int n_tiles;
@@ -344,7 +344,9 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       }
     }
     // rescale g_R so that sum_i g_R sum_j g_phi is exactly the target sum D + sum R (f_eq - R
-    // of phase D then carries the cell's mass; see normalise_equilibrium): g_R <- g_R (1 - delta)
+    // of phase D then carries the cell's mass).  In exact arithmetic the truncated equilibrium has this
+    // sum (Sec. IV.D); in single precision the table contraction misses it by some 1e-7, and the BGK
+    // term would turn that into a mass source of (dt / tau) 1e-7 n every step.  g_R <- g_R (1 - delta)
     real scale0;  // FP64 path: the factor of g_R
     float delta = 0.f;
     if constexpr (F32) {
@@ -611,7 +613,9 @@ __global__ void __launch_bounds__(NT, stage_min_ctas(int(sizeof(real)), TC, NT))
       }
       const pair_t<real> G0 = p_fma(F1, p_set(real(-3)), p_fma(F0, p_set(real(3)), F2));
       const pair_t<real> G1 = p_fma(F1, p_set(real(-8)), p_fma(F0, p_set(real(6)), p_mul(F2, p_set(real(3)))));
-      // (bit for bit phase D's value: the same cell, side and order)
+      // chi: bit for bit phase D's value (the same cell, side and order).  f~: phase D walks F~ - R, formed
+      // by one fma, which agrees with this F~ to rounding; differences of F~ itself are kept here, since
+      // where sqrt(g) is far from one F~ - R is larger than F~ and n_w would carry its rounding
       const real sc = iw0[i] * iw1[j];
       const pair_t<real> SC = p_set(sc);
       WenoWin<real, false> w;

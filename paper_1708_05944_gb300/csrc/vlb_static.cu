@@ -40,12 +40,10 @@ cudaError_t launch_one(vlb_ctx* c, int k, const void* prev, const void* fl, void
   a.Fprev = static_cast<const real*>(prev);
   a.Fl = static_cast<const real*>(fl);
   a.Fout = static_cast<real*>(out);
-  const double ca[3] = {0.0, 0.75, 1.0 / 3.0}, cb[3] = {1.0, 0.25, 2.0 / 3.0}, cc[3] = {1.0, 0.25, 2.0 / 3.0};
+  const double ca[3] = {0.0, 0.75, 1.0 / 3.0}, cc[3] = {1.0, 0.25, 2.0 / 3.0};
   a.ca = ca[k - 1];
-  a.cb = cb[k - 1];
   a.cc = cc[k - 1];
   a.caf = float(a.ca);
-  a.cbf = float(a.cb);
   a.ccf = float(a.cc);
   a.inst = c->d_inst;
   a.tiles = c->d_tiles;
