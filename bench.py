@@ -60,7 +60,7 @@ WORKLOAD = (f"gradually expanding channel: {CH_NX} (xi) x {CH_NL} (lambda) cells
 # DRAM bytes (read + write) per launch of the channel stage kernel from one ncu capture, keyed by
 # the SHA-256 of the kernel's code at the time of the capture (a changed kernel reports null):
 # see profiles/ for the command and the scaling to the full grid
-CH_TRAFFIC = {"75dd4185db98bef9": 4.227e9}
+CH_TRAFFIC = {"47a90e15eb447a2e": 4.231e9}
 
 
 def dist_env():

@@ -19,12 +19,12 @@
 // reconstructions of a row of four columns take 160).  Why four columns a thread: the strip's xi
 // walk and the windows cost 34 packed operations an interface where five cells loaded afresh cost
 // 44 (windows of two columns or of raw rows in shared memory, twice the warps or half the
-// registers, measured 13.0 - 14.1 ms a step against 9.85); why unrolled: the same loop rolled
+// registers, measured 13.0 - 14.1 ms a step where this took 9.85); why unrolled: the same loop rolled
 // halves the reconstructions in flight (14.5).  A barrier at the step's end keeps the warps on
 // the same instructions; waiting later, at the next combine, lost more to instruction fetches
 // (12.5).  2048 x 512 x 192, single precision, a step of three stages: 20.3 ms for one thread per
-// (column, velocity) with 1024 threads of 64 registers, 9.8 ms now (1.32 TB/s algorithmic a
-// stage); double precision, 256 x 64: 10.9 and 6.8 ms; Cartesian split, 512 x 256: 2.39 and 1.17.
+// (column, velocity) with 1024 threads of 64 registers, 9.9 ms now (1.30 TB/s algorithmic a
+// stage); double precision, 256 x 64: 10.9 and 6.7 ms; Cartesian split, 512 x 256: 2.39 and 1.19.
 //
 // Boundaries: the centreline mirror (Sec. VII.C.3) at the bottom of the march, the diffuse wall
 // (Sec. VII.C.4) at its top with n_w per column from the zero-mass-flux balance, and the

@@ -17,8 +17,8 @@
 // What bounds it: latency (36 - 42 % of the issue slots, 35 % of the FP32 pipe, 20 warps a SM).  The
 // walk of phase D takes WENO-5 on shared differences (WenoWin), phase A sums a row of nodes per
 // lane: 285 -> 204 instructions per warp and cell-velocity row.  Single precision, 16 x 20
-// velocities, a step: 256 instances of 64 .. 1024 cells 1.90 -> 1.54 ms, 5 x 1024 cells 90 -> 72 us;
-// double precision 5 x 1024 cells 2.62 -> 1.83 ms.
+// velocities, a step: 256 instances of 64 .. 1024 cells 1.90 -> 1.51 ms, 5 x 1024 cells 90 -> 72 us;
+// double precision 5 x 1024 cells 2.62 -> 1.84 ms.
 #pragma once
 #include <type_traits>
 
